@@ -616,7 +616,7 @@ int grid_for(const Ctx &c, int64_t n) {
 // every op built so far fits the budget).
 __global__ void prune_list_kernel(const float *u_pend, const int32_t *slots, int J, int64_t n_units,
                                   const unsigned long long *st, const float *cut, int32_t *list,
-                                  int *count, int32_t *long_list, unsigned long long *potential) {
+                                  int64_t stride, int *count, int32_t *long_list, unsigned long long *potential) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_units) return;
     float p = u_pend[i];
@@ -630,9 +630,9 @@ __global__ void prune_list_kernel(const float *u_pend, const int32_t *slots, int
     if (above && p >= *cut) {
         const int j = (int)(i % J);
         const int n = slots[j + 1] - slots[j];
-        if (n <= kShortUnit) list[atomicAdd(count, 1)] = (int32_t)i;
-        else if (n <= kMaxUnit) list[n_units - 1 - atomicAdd(count + 1, 1)] = (int32_t)i;
-        else long_list[atomicAdd(count + 2, 1)] = (int32_t)i;
+        const int q = unit_class(n);
+        if (n <= kMaxUnit) list[q * stride + atomicAdd(count + q, 1)] = (int32_t)i;
+        else long_list[atomicAdd(count + kUnitClasses, 1)] = (int32_t)i;
     }
 }
 
@@ -688,16 +688,16 @@ __global__ void __launch_bounds__(1024) pend_cut_kernel(const unsigned int *hist
     if (tid == 1023 && before + own < (unsigned)m) *cut = -INFINITY;   // fewer than m qualify: no cut
 }
 
-__global__ void slot_classes_kernel(const int32_t *slots, int J, int32_t *list, int *count,
+__global__ void slot_classes_kernel(const int32_t *slots, int J, int32_t *list, int64_t stride, int *count,
                                     int32_t *long_slots) {
     int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= J) return;
     const int n = slots[j + 1] - slots[j];
-    if (n <= kShortUnit) list[atomicAdd(count, 1)] = j;
-    else if (n <= kMaxUnit) list[J - 1 - atomicAdd(count + 1, 1)] = j;
+    const int q = unit_class(n);
+    if (n <= kMaxUnit) list[q * stride + atomicAdd(count + q, 1)] = j;
     else {
-        long_slots[atomicAdd(count + 2, 1)] = j;
-        atomicAdd(count + 3, n);
+        long_slots[atomicAdd(count + kUnitClasses, 1)] = j;
+        atomicAdd(count + kUnitClasses + 1, n);
     }
 }
 
@@ -722,15 +722,15 @@ cudaError_t launch_threshold(Ctx &c, int J, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_prune_list(Ctx &c, const int32_t *slots, int J, int32_t *list, int *count,
+cudaError_t launch_prune_list(Ctx &c, const int32_t *slots, int J, int32_t *list, int64_t stride, int *count,
                               int32_t *long_list, cudaStream_t s) {
     const int64_t nu = (int64_t)c.p.L * c.p.G * J;
-    cudaError_t e = cudaMemsetAsync(count, 0, 3 * sizeof(int), s);
+    cudaError_t e = cudaMemsetAsync(count, 0, (kUnitClasses + 1) * sizeof(int), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(c.w.pend_pot, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
     prune_list_kernel<<<(unsigned)((nu + 255) / 256), 256, 0, s>>>(c.w.u_pend, slots, J, nu,
                                                                     c.w.alloc_state, c.w.pend_cut, list,
-                                                                    count, long_list, c.w.pend_pot);
+                                                                    stride, count, long_list, c.w.pend_pot);
     c.launches += 1;
     return cudaGetLastError();
 }
@@ -746,11 +746,11 @@ cudaError_t launch_pend_cut(Ctx &c, int J, int m, float *cut, unsigned int *n_qu
     return cudaGetLastError();
 }
 
-cudaError_t launch_slot_classes(Ctx &c, const int32_t *slots, int J, int32_t *list, int *count,
+cudaError_t launch_slot_classes(Ctx &c, const int32_t *slots, int J, int32_t *list, int64_t stride, int *count,
                                 int32_t *long_slots, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(count, 0, 4 * sizeof(int), s);
+    cudaError_t e = cudaMemsetAsync(count, 0, (kUnitClasses + 2) * sizeof(int), s);
     if (e != cudaSuccess) return e;
-    slot_classes_kernel<<<(J + 255) / 256, 256, 0, s>>>(slots, J, list, count, long_slots);
+    slot_classes_kernel<<<(J + 255) / 256, 256, 0, s>>>(slots, J, list, stride, count, long_slots);
     c.launches += 1;
     return cudaGetLastError();
 }

@@ -251,7 +251,7 @@ gkv_status gracekv_create(const gkv_params *pin, gracekv_ctx **out) {
     gkv::Workspace &w = c.w;
     bool ok = dalloc(x, &w.rope, (size_t)p.T * (p.d / 2)) &&
               dalloc(x, &w.rope_rel, (size_t)(2 * gkv::kMaxSlot - 1) * (p.d / 2)) &&
-              dalloc(x, &w.long_slots, (size_t)Nc + 2) && dalloc(x, &w.long_n, 4) &&
+              dalloc(x, &w.long_slots, (size_t)Nc + 2) && dalloc(x, &w.long_n, 5) &&
               dalloc(x, &w.ent, (size_t)p.budget + (size_t)p.L * p.G * (p.T - Nc)) &&
               dalloc(x, &w.inv_norm, (size_t)c.nseg * p.T) &&
               dalloc(x, &w.nrm2, (size_t)c.nseg * p.T) &&
@@ -477,7 +477,7 @@ static gkv_status build_setup(gracekv_ctx *x, const int32_t *slot_starts, int32_
         bool ok = dalloc(x, &w.u_nnodes, cap) && dalloc(x, &w.u_Uadd, cap) &&
                   dalloc(x, &w.u_Ddrop, cap) && dalloc(x, &w.u_sel, cap) &&
                   dalloc(x, &w.u_count, cap) && dalloc(x, &w.u_off, cap) &&
-                  dalloc(x, &w.u_pend, cap) && dalloc(x, &w.u_list, cap) &&
+                  dalloc(x, &w.u_pend, cap) && dalloc(x, &w.u_list, gkv::kUnitClasses * cap) &&
                   (c.p.alpha_floor <= 0.0 || dalloc(x, &w.u_floor, cap)) &&
                   dalloc(x, &w.long_list, cap) &&
                   dalloc(x, &w.u_bsum, cap / 1024 + 2) &&
@@ -488,10 +488,11 @@ static gkv_status build_setup(gracekv_ctx *x, const int32_t *slot_starts, int32_
     return GKV_OK;
 }
 
-// Work counters and the op list cleared; slots split into the short and long
-// classes of the unit kernel and the long units (cnt: their sizes and the
-// long units' tokens; synchronises s).
-static cudaError_t build_classes(Ctx &c, int cnt[4], cudaStream_t s) {
+// Work counters and the op list cleared; slots split into the classes of the
+// unit kernel and the long units (cnt: their sizes and the long units'
+// tokens; synchronises s).
+constexpr int kLongCnt = gkv::kUnitClasses, kClassCnt = gkv::kUnitClasses + 2;
+static cudaError_t build_classes(Ctx &c, int cnt[kClassCnt], cudaStream_t s) {
     gkv::Workspace &w = c.w;
     const int64_t nu = (int64_t)c.p.L * c.p.G * c.J;
     static const float kNoCut = -INFINITY;
@@ -499,12 +500,12 @@ static cudaError_t build_classes(Ctx &c, int cnt[4], cudaStream_t s) {
     if (!(c.B_free < nu)) e = cudaMemcpyAsync(w.pend_cut, &kNoCut, sizeof(float), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(w.work, 0, 4 * sizeof(unsigned long long), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(w.n_ops, 0, sizeof(unsigned int), s);
-    cnt[0] = cnt[1] = cnt[2] = cnt[3] = 0;
+    for (int q = 0; q < kClassCnt; q++) cnt[q] = 0;
     if (e == cudaSuccess) {
         gkv::StageTimer tm(c, 3, s);
-        e = gkv::launch_slot_classes(c, w.slots, c.J, w.u_list, w.dev_int + 2, w.long_slots, s);
+        e = gkv::launch_slot_classes(c, w.slots, c.J, w.u_list, w.units_cap, w.dev_int + 2, w.long_slots, s);
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(cnt, w.dev_int + 2, 4 * sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(cnt, w.dev_int + 2, kClassCnt * sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     return e;
 }
@@ -512,19 +513,19 @@ static cudaError_t build_classes(Ctx &c, int cnt[4], cudaStream_t s) {
 // The classes, and the work-item arrays of the long units sized for them: a
 // level's items of one unit are disjoint intervals of >= 2 tokens, so at most
 // n / 2 of them (or its root).
-static gkv_status classes(gracekv_ctx *x, int cnt[4], cudaStream_t s) {
+static gkv_status classes(gracekv_ctx *x, int cnt[kClassCnt], cudaStream_t s) {
     Ctx &c = x->c;
     gkv::Workspace &w = c.w;
     cudaError_t e = build_classes(c, cnt, s);
     if (e != cudaSuccess) return cuda_fail(x, e, "build_trees classes");
-    c.n_long = cnt[2];
-    if (cnt[2] == 0) return GKV_OK;
+    c.n_long = cnt[kLongCnt];
+    if (cnt[kLongCnt] == 0) return GKV_OK;
     const int64_t LG = (int64_t)c.p.L * c.p.G;
-    const int64_t items = LG * ((int64_t)cnt[3] / 2 + cnt[2]) + 16, units = LG * cnt[2];
+    const int64_t items = LG * ((int64_t)cnt[kLongCnt + 1] / 2 + cnt[kLongCnt]) + 16, units = LG * cnt[kLongCnt];
     if (items > w.long_cap) {
         bool ok = dalloc(x, &w.long_gv, items) && dalloc(x, &w.long_uid, items) &&
                   dalloc(x, &w.long_kin, items) && dalloc(x, &w.long_ufl, items) &&
-                  dalloc(x, &w.long_sub, 2 * items) &&
+                  dalloc(x, &w.long_sub, gkv::kUnitClasses * items) &&
                   dalloc(x, reinterpret_cast<unsigned char **>(&w.long_res), items * gkv::long_res_bytes());
         if (!ok) return fail(x, GKV_ENOMEM, "build_trees: long-unit work items");
         w.long_cap = items;
@@ -550,7 +551,7 @@ static cudaError_t long_to_leaves(Ctx &c, const void *K, const void *V, const vo
 
 // The first tree-building launch of the units of (l, g) in [lg0, lg0 + nlg).
 static cudaError_t build_fresh(Ctx &c, const void *K, const void *V, const void *Q, const float *omega,
-                               const int cnt[4], int lg0, int nlg, cudaStream_t s) {
+                               const int cnt[kClassCnt], int lg0, int nlg, cudaStream_t s) {
     gkv::Workspace &w = c.w;
     const int64_t nu = (int64_t)c.p.L * c.p.G * c.J;
     // with per-(l, g) capacities ("w/o GA") the global threshold cannot prune:
@@ -559,15 +560,15 @@ static cudaError_t build_fresh(Ctx &c, const void *K, const void *V, const void 
     const bool root_only = !full && c.B_free < nu;
     gkv::StageTimer tm(c, 3, s);
     cudaError_t e = gkv::launch_unit_build(c, K, V, Q, omega, w.slots, c.J, 0, root_only ? 1 : 0,
-                                           full ? 4 * gkv::kMaxUnit : 1, 0.f, w.u_list, cnt[0],
-                                           w.u_list + (c.J - cnt[1]), cnt[1], s, lg0, nlg);
-    if (e != cudaSuccess || cnt[2] == 0) return e;
-    e = gkv::launch_long_level(c, K, V, Q, omega, w.slots, c.J, 1, root_only ? 1 : 0, 0.f, w.long_slots, cnt[2],
+                                           full ? 4 * gkv::kMaxUnit : 1, 0.f,
+                                           {w.u_list, w.units_cap, {cnt[0], cnt[1], cnt[2]}}, s, lg0, nlg);
+    if (e != cudaSuccess || cnt[kLongCnt] == 0) return e;
+    e = gkv::launch_long_level(c, K, V, Q, omega, w.slots, c.J, 1, root_only ? 1 : 0, 0.f, w.long_slots, cnt[kLongCnt],
                                lg0, nlg, s, nullptr);
     if (e != cudaSuccess || !full) return e;
-    e = gkv::launch_long_units(c, w.long_slots, cnt[2], lg0, nlg, c.J, w.long_list, s);
+    e = gkv::launch_long_units(c, w.long_slots, cnt[kLongCnt], lg0, nlg, c.J, w.long_list, s);
     if (e != cudaSuccess) return e;
-    return long_to_leaves(c, K, V, Q, omega, w.long_list, cnt[2] * nlg, s);
+    return long_to_leaves(c, K, V, Q, omega, w.long_list, cnt[kLongCnt] * nlg, s);
 }
 
 // Trees (build.cu).  Every op's key is bounded before it is built: a pending
@@ -595,18 +596,18 @@ static cudaError_t build_passes(Ctx &c, const void *K, const void *V, const void
     cudaError_t e = cudaSuccess;
     for (int it = 0; e == cudaSuccess; it++) {
         struct {
-            int count[3];
+            int count[kLongCnt + 1];
             unsigned long long prefix, all, total, pot;
             float cut;
             unsigned int nqual;
-        } h = {{0, 0, 0}, 0, 0, 0, 0, 0.f, 0};
+        } h = {{0, 0, 0, 0}, 0, 0, 0, 0, 0.f, 0};
         {
             gkv::StageTimer tm(c, 3, s);
             e = gkv::launch_threshold(c, J, s);
             if (e == cudaSuccess && root_only) e = gkv::launch_pend_cut(c, J, pass_units, w.pend_cut, w.pend_n, s);
-            if (e == cudaSuccess) e = gkv::launch_prune_list(c, w.slots, J, w.u_list, w.dev_int + 2, w.long_list, s);
+            if (e == cudaSuccess) e = gkv::launch_prune_list(c, w.slots, J, w.u_list, w.units_cap, w.dev_int + 2, w.long_list, s);
         }
-        if (e == cudaSuccess) e = cudaMemcpyAsync(h.count, w.dev_int + 2, 3 * sizeof(int), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(h.count, w.dev_int + 2, sizeof h.count, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&h.prefix, w.alloc_state, 2 * sizeof(unsigned long long),
                                                   cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&h.all, w.alloc_state + 2, sizeof(unsigned long long),
@@ -618,7 +619,7 @@ static cudaError_t build_passes(Ctx &c, const void *K, const void *V, const void
         if (e == cudaSuccess) e = cudaMemcpyAsync(&h.pot, w.pend_pot, sizeof(unsigned long long),
                                                   cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess || h.count[0] + h.count[1] + h.count[2] == 0) break;
+        if (e != cudaSuccess || h.count[0] + h.count[1] + h.count[2] + h.count[kLongCnt] == 0) break;
         uint32_t bits = (uint32_t)h.prefix;
         float tau;
         memcpy(&tau, &bits, sizeof tau);
@@ -636,12 +637,12 @@ static cudaError_t build_passes(Ctx &c, const void *K, const void *V, const void
         const int levels = fits ? 4 * gkv::kMaxUnit : ((settled || c.n_long > 0) ? 4 : 1);
         tau_prev = tau;
         gkv::StageTimer tm(c, 3, s);
-        e = gkv::launch_unit_build(c, K, V, Q, omega, w.slots, J, 1, 0, levels, tau_eff, w.u_list,
-                                   h.count[0], w.u_list + (nu - h.count[1]), h.count[1], s);
-        if (e == cudaSuccess && h.count[2] > 0) {   // long units: one level, or all of them when they fit
-            e = gkv::launch_long_level(c, K, V, Q, omega, w.slots, J, 0, 0, tau_eff, w.long_list, h.count[2], 0, -1,
+        e = gkv::launch_unit_build(c, K, V, Q, omega, w.slots, J, 1, 0, levels, tau_eff,
+                                   {w.u_list, w.units_cap, {h.count[0], h.count[1], h.count[2]}}, s);
+        if (e == cudaSuccess && h.count[kLongCnt] > 0) {   // long units: one level, or all of them when they fit
+            e = gkv::launch_long_level(c, K, V, Q, omega, w.slots, J, 0, 0, tau_eff, w.long_list, h.count[kLongCnt], 0, -1,
                                        s, nullptr, tau);   // subtrees prune against tau itself, not the cut
-            if (e == cudaSuccess && fits) e = long_to_leaves(c, K, V, Q, omega, w.long_list, h.count[2], s);
+            if (e == cudaSuccess && fits) e = long_to_leaves(c, K, V, Q, omega, w.long_list, h.count[kLongCnt], s);
         }
         c.build_passes = it + 2;
     }
@@ -680,7 +681,7 @@ gkv_status gracekv_build_trees(gracekv_ctx *x, const void *K, const void *V, con
         }
     }
     c.scored = false;
-    int cnt[4];
+    int cnt[kClassCnt];
     if (e == cudaSuccess && c.p.lambda_graph > 0.0) {   // R = (1 - lambda) s-hat + lambda d-hat
         if (!c.mh_Qg) return fail(x, GKV_EINVAL, "build_trees: multi-hop relevance needs gracekv_set_graph_queries");
         c.mh_K = K;
@@ -786,7 +787,7 @@ gkv_status gracekv_compress_host(gracekv_ctx *x, const void *K, const void *V, c
     if (st) return st;
     st = build_setup(x, nullptr, 0, s);
     if (st) return st;
-    int cnt[4];
+    int cnt[kClassCnt];
     e = cudaMemsetAsync(c.w.dev_int + gkv::kScoreStatus, 0, sizeof(int), s);
     if (e != cudaSuccess) return cuda_fail(x, e, "compress_host");
     st = classes(x, cnt, s);

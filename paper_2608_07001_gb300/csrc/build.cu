@@ -53,13 +53,15 @@ namespace gkv {
 namespace {
 
 constexpr int kMaxCuts = 18;     // K + midpoint, K <= 16 (+1 spare)
-constexpr int kNT = 256;         // threads per CTA
+constexpr int kNT = 256;         // threads of one scan direction (a CTA has one or two, Smem::DIRS)
 constexpr int kNPP = 32;         // probe pairs: thread handles probes p and p + 32 (W <= 64)
 constexpr int kNCL = 8;          // threads per probe pair (4-element groups, interleaved)
 constexpr int kPPW = 32 / kNCL;  // probe pairs per warp: lane = 4 c + (pair % 4), so that the
                                  // 4 lanes reading one 16-byte chunk are adjacent (one shared-
                                  // memory wavefront serves them; lanes 8 apart would not merge)
-constexpr int kNCD = 19;         // candidate intervals per direction and batch: 17 cuts + p* side + whole node
+constexpr int kNCD = 19;         // prefix candidates of a batch: 17 cuts + p* side + whole node
+constexpr int kNCS = 18;         // suffix candidates of a batch: 17 cuts + p* side
+constexpr int kNCA = kNCD + kNCS;   // candidate k: prefixes in [0, kNCD), suffixes in [kNCD, kNCA)
 
 struct BuildArgs {
     const void *K, *V, *Q;
@@ -75,14 +77,12 @@ struct BuildArgs {
     float lam_kappa, base_frac;
     // work list: fresh launches index (slot list entry, lg), resume launches units
     int resume;                  // 0: build from the root, 1: resume pending nodes
-    int subtree;                 // 1: the list holds pending nodes of at most NMAX tokens inside
-                                 //    long units (build_long.cu), as global node indices; each CTA
-                                 //    builds its node's subtree to the leaves into the node slots
-                                 //    reserved for it (the unit-relative index in its child0)
     int root_only;               // fresh: evaluate only the root's own distortion (split stays pending)
     int max_levels;              // levels evaluated by this launch
     float tau;                   // resume: evaluate pending nodes whose key bound >= tau
-    const int32_t *list;         // fresh: slot indices; resume: unit ids
+    const int32_t *list;         // fresh: slot indices; resume: unit ids; subtree: node indices
+    int64_t stride;              // the launch's classes follow one another at this distance,
+    int c1, c2;                  // its work items c1.. and c2.. in the second and third
     int lg0, nlg;                // fresh: the (l, g) range [lg0, lg0 + nlg) of the launch
     // outputs
     int32_t *nd_a, *nd_b, *nd_child0, *nd_parent, *nd_unit;
@@ -102,29 +102,27 @@ struct BuildArgs {
 struct NodeS {
     float D;
     float kin;                   // bottleneck key of the op that created the node
-    short a, b, parent, child0;
+    short a, b;
     signed char nchild;          // -1: pending (not evaluated)
 };
 
 struct BatchNode {
-    int node;
-    int ncut;
+    unsigned long long klo, khi;   // smallest and largest curvature key over the node's cut positions
+    float cD[3];
+    short node, pstar;
+    short op;                // the node's place among the batch's Split ops (-1: none)
+    short ca[3], cb[3];
     int8_t cut[kMaxCuts];    // local cut positions xi (ascending)
     int8_t pidx[kMaxCuts];   // candidate index of [a, xi) (-1: single token)
     int8_t sidx[kMaxCuts];   // candidate index of [xi, b) (-1: single token)
-    int pstar, eL, eR, whole;
-    int forced;              // extraction at a singleton-floor position (a floor op)
-    int pre_b, pre_e, suf_b, suf_e;   // prefixes (ascending end) in [0, NCD),
-                                      // suffixes (descending start) in [NCD, 2 NCD)
-    int pre_r, suf_r;                 // ends of the reserved ranges (unused entries empty)
-    double kmin;             // smallest curvature over the node's cut positions
-    float krange;            // 1 / (largest - smallest), 0 when they are equal
-    int nchild, ca[3], cb[3];
-    float cD[3];
+    int8_t ncut, eL, eR, whole, nchild;
+    int8_t forced;           // extraction at a singleton-floor position (a floor op)
+    int8_t pre_b, pre_e, suf_b, suf_e;   // prefixes (ascending end) in [0, kNCD),
+                                         // suffixes (descending start) in [kNCD, kNCA)
 };
 
 struct Cand {
-    int a, b;        // local interval (a == b: unused entry)
+    short a, b;      // local interval (a == b: unused entry)
     float meff;
 };
 
@@ -220,6 +218,18 @@ __device__ __forceinline__ void ld8x2(const __nv_bfloat16 *p, float2 v[4]) {
     for (int i = 0; i < 4; i++) v[i] = __bfloat1622float2(h[i]);
 }
 
+// 8 floats to a 16-byte aligned shared-memory row.
+__device__ __forceinline__ void st8(float *p, const float v[8]) {
+    reinterpret_cast<float4 *>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<float4 *>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
+}
+
+// Order-preserving 32-bit key of a float (-0 and +0 alike).
+__device__ __forceinline__ unsigned fkey_ordered(float x) {
+    const unsigned u = __float_as_uint(x + 0.f);
+    return u >> 31 ? ~u : u | 0x80000000u;
+}
+
 // N consecutive elements of a shared-memory row as floats (N = 1 or 2).
 template <int N>
 __device__ __forceinline__ void ld_pairs(const float *p, float v[N]) {
@@ -242,60 +252,161 @@ __device__ __forceinline__ void ld_pairs(const __nv_bfloat16 *p, float v[N]) {
     }
 }
 
-template <int DH, typename Tin, int NMAX>
+// Sum over a probe pair's 8 chunk lanes (lane bits 2..4) of each of 8 values,
+// as a reduce-scatter: 7 exchanges instead of the 24 of 8 butterflies, and the
+// lane with chunk index c ends with the sum of v[c].  Every sum pairs the
+// lanes in the butterfly's order (bit 2, then 3, then 4), so its bits are the
+// butterfly's.
+__device__ __forceinline__ float reduce_scatter8(const float v[8], int lane) {
+    float x[4], y[2];
+    const bool h0 = lane & kPPW, h1 = lane & (2 * kPPW), h2 = lane & (4 * kPPW);
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const float send = h0 ? v[2 * i] : v[2 * i + 1], keep = h0 ? v[2 * i + 1] : v[2 * i];
+        x[i] = keep + __shfl_xor_sync(0xffffffffu, send, kPPW);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; i++) {
+        const float send = h1 ? x[2 * i] : x[2 * i + 1], keep = h1 ? x[2 * i + 1] : x[2 * i];
+        y[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * kPPW);
+    }
+    const float send = h2 ? y[0] : y[1], keep = h2 ? y[1] : y[0];
+    return keep + __shfl_xor_sync(0xffffffffu, send, 4 * kPPW);
+}
+
+// Running sums of an interval's prototype: PPL rotation pairs (i, i + d/2) per
+// lane, PPL consecutive i (a packed pair when PPL = 2; each lane of a packed
+// add or FMA rounds like the scalar one).
+template <int PPL, int HALF> struct ProtoSum;
+template <int HALF> struct ProtoSum<2, HALF> {
+    float2 m0, m1, r0, r1, s0, s1, q;   // sum k_circ, R v, v (both halves); q = (sum R, sum ||k||)
+    __device__ __forceinline__ void clear() {
+        m0 = m1 = r0 = r1 = s0 = s1 = q = make_float2(0.f, 0.f);
+    }
+    struct Tok {
+        float2 k0, k1, x0, x1, rk;
+        __device__ __forceinline__ void load(const float *k, const float *v, const float2 *r) {
+            k0 = *reinterpret_cast<const float2 *>(k);
+            k1 = *reinterpret_cast<const float2 *>(k + HALF);
+            x0 = *reinterpret_cast<const float2 *>(v);
+            x1 = *reinterpret_cast<const float2 *>(v + HALF);
+            rk = *r;
+        }
+    };
+    __device__ __forceinline__ void add(const Tok &t) {
+        const float2 rr = make_float2(t.rk.x, t.rk.x);
+        q = fadd2(q, t.rk);
+        m0 = fadd2(m0, t.k0);
+        m1 = fadd2(m1, t.k1);
+        r0 = ffma2(rr, t.x0, r0);
+        r1 = ffma2(rr, t.x1, r1);
+        s0 = fadd2(s0, t.x0);
+        s1 = fadd2(s1, t.x1);
+    }
+    __device__ __forceinline__ void get(int j, float &a, float &b, float &c, float &d, float &e, float &f) const {
+        a = j ? m0.y : m0.x; b = j ? m1.y : m1.x;
+        c = j ? r0.y : r0.x; d = j ? r1.y : r1.x;
+        e = j ? s0.y : s0.x; f = j ? s1.y : s1.x;
+    }
+};
+template <int HALF> struct ProtoSum<1, HALF> {
+    float m0, m1, r0, r1, s0, s1;
+    float2 q;
+    __device__ __forceinline__ void clear() {
+        m0 = m1 = r0 = r1 = s0 = s1 = 0.f;
+        q = make_float2(0.f, 0.f);
+    }
+    struct Tok {
+        float k0, k1, x0, x1;
+        float2 rk;
+        __device__ __forceinline__ void load(const float *k, const float *v, const float2 *r) {
+            k0 = k[0]; k1 = k[HALF]; x0 = v[0]; x1 = v[HALF];
+            rk = *r;
+        }
+    };
+    __device__ __forceinline__ void add(const Tok &t) {
+        q = fadd2(q, t.rk);
+        m0 += t.k0;
+        m1 += t.k1;
+        r0 = fmaf(t.rk.x, t.x0, r0);
+        r1 = fmaf(t.rk.x, t.x1, r1);
+        s0 += t.x0;
+        s1 += t.x1;
+    }
+    __device__ __forceinline__ void get(int, float &a, float &b, float &c, float &d, float &e, float &f) const {
+        a = m0; b = m1; c = r0; d = r1; e = s0; f = s1;
+    }
+};
+
+// Instances by slot length: up to kTinyUnit tokens three CTAs per SM, up to
+// kShortUnit two, longer slots one CTA of twice the threads.
+template <int DH, int NMAX>
 struct Smem {
-    static constexpr int NWARPS = kNT / 32;
+    static constexpr int DIRS = NMAX <= kShortUnit ? 1 : 2;   // scan directions that run side by side
+    static constexpr int CTAS = NMAX <= kTinyUnit ? 3 : (NMAX <= kShortUnit ? 2 : 1);   // per SM
+    static constexpr int NT = kNT * DIRS;
+    static constexpr int NWARPS = NT / 32;
     static constexpr int NB = 16;            // nodes per batch
     static constexpr int MAXNODES = 2 * NMAX;
-    float kc[NMAX][DH + 8];                  // rows padded by 32 B: the probe-weight MMA reads
-                                             // 8 rows at once, which then fall in distinct banks
+    static constexpr int NROW = DIRS == 2 ? kNCA : kNCD;   // candidate rows held at a time
+    static constexpr int KTW = DH < 128 ? 128 : DH;        // a row also holds 32 float4 of sums
+    static constexpr int MW = (MAXNODES + 31) / 32;
+    static constexpr int KPAD = NMAX <= kShortUnit ? 8 : 0;
+    float kc[NMAX][DH + KPAD];               // rows padded by 32 B where there is room: the probe-weight
+                                             // MMA reads 8 rows at once, which then fall in distinct banks
     float vv[NMAX][DH];                      // values, converted once to fp32
     float2 E[NMAX][kNPP];                    // probe weights of probes (p, p + 32)
-    float ktil[kNCD][DH];                    // prototypes of one direction at a time
-    float vtil[kNCD][DH];
-    float Rt[NMAX];
-    float Ff[NMAX];                          // floor score of an accepted floor position, -inf elsewhere
-    float kn[NMAX];
+    float ktil[NROW][KTW];                   // key prototypes; once the logits are taken, the row holds
+                                             // (residual / ||M||^2, Z) of the probes p and p + 32
+    float vtil[NROW][DH];
+    float2 zt[NROW][kNPP];                   // m_eff exp(logit) of the probes (p, p + 32)
+    float2 RK[NMAX];                         // token value, ||k||
     unsigned long long kap[NMAX];            // order-preserving keys of the curvature
-    float redD[2 * kNCD][NWARPS];
-    float redP[2 * kNCD][NWARPS];
-    float candD[2 * kNCD], candP[2 * kNCD];  // per-candidate D and drop mass
-    Cand cand[2 * kNCD];
-    NodeS nodes[MAXNODES];
     BatchNode bn[NB];
-    short lvl[2][MAXNODES];
-    int nlvl[2];
-    int nnodes;
-    int batch_n, batch_next, batch_pre, batch_suf;   // candidate entries reserved per direction
-    unsigned long long wcnt[kNT / 32][3];   // per-warp work counters
+    Cand cand[kNCA];
+    NodeS nodes[MAXNODES];
+    float Ff[NMAX];                          // floor score of an accepted floor position, -inf elsewhere
+    float candD[kNCA], candP[kNCA];          // per-candidate D and drop mass
+    unsigned lvl[2][MW];                     // nodes of the level (bit masks), of the next one
+    unsigned op_base;                        // the batch's first Split op in the global list
+    unsigned int wcnt[NWARPS][3];            // per-warp work counters
     float pend;
     float rootR;                             // R of a fresh root
 };
 
-// SUB: the subtree mode (BuildArgs::subtree) as a compile-time flag, so that
-// the other instances carry none of its index mapping
+// SUB: the subtree mode, a compile-time flag so that the other instances carry
+// none of its index mapping: the list holds pending nodes of at most NMAX
+// tokens inside long units (build_long.cu), as global node indices; each CTA
+// builds its node's subtree to the leaves into the node slots reserved for it
+// (the unit-relative index in its child0)
 template <int DH, typename Tin, int NMAX, bool SUB>
-__global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(BuildArgs A) {
-    using S = Smem<DH, Tin, NMAX>;
+__global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit_build_kernel(BuildArgs A) {
+    using S = Smem<DH, NMAX>;
     // thread (p, c): probes p and p + 32, elements 4 c + 32 g + j (g < NG, j < 4)
     constexpr int HALF = DH / 2, NWARPS = S::NWARPS, NG = DH / (4 * kNCL), CH = 4 * NG;
+    constexpr int NT = S::NT, DIRS = S::DIRS;
     static_assert(kNPP * kNCL == kNT && DH % (4 * kNCL) == 0, "probe layout");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     S &sm = *reinterpret_cast<S *>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int dwarp = warp & (kNT / 32 - 1);   // warp within its scan direction (DIRS = 2: warps 8..15 take the suffixes)
     int j, lg;
+    auto item = [&](int i) {
+        const int q = (i >= A.c1) + (i >= A.c2);
+        return A.list[q * A.stride + i - (q == 0 ? 0 : (q == 1 ? A.c1 : A.c2))];
+    };
     int64_t gv_sub = -1;         // subtree mode: the pending node whose subtree this CTA builds
     if constexpr (SUB) {
-        gv_sub = A.list[blockIdx.x];
+        gv_sub = item(blockIdx.x);
         const int uidr = A.nd_unit[gv_sub];
         lg = uidr / A.J;
         j = uidr - lg * A.J;
     } else if (A.resume) {
-        const int uidr = A.list[blockIdx.x];
+        const int uidr = item(blockIdx.x);
         lg = uidr / A.J;
         j = uidr - lg * A.J;
     } else {
-        j = A.list[blockIdx.x / A.nlg];   // slot-major: the units of a slot share its table rows
+        j = item(blockIdx.x / A.nlg);   // slot-major: the units of a slot share its table rows
         lg = A.lg0 + blockIdx.x % A.nlg;
     }
     const bool fresh = !A.resume && !SUB;
@@ -329,24 +440,93 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
     auto eidx = [](int t, int u) { return t * 2 * kNPP + 2 * (u & (kNPP - 1)) + (u >> 5); };
     if (A.Eg) {   // the same layout, n rows of 256 bytes: 16-byte copies
         const float *Eu = A.Eg + ((size_t)lg * A.Nc + (sa - A.cs)) * (2 * kNPP);
-        for (int idx = tid; idx < n * (2 * kNPP / 4); idx += kNT) cp_async16(Ef + 4 * idx, Eu + 4 * idx, true);
+        for (int idx = tid; idx < n * (2 * kNPP / 4); idx += NT) cp_async16(Ef + 4 * idx, Eu + 4 * idx, true);
         cp_async_commit();
     }
+    // resume: the unit's node records, one per thread (a unit has at most
+    // 2 n - 1 <= NT of them), loaded beside the slot
+    int nn = 0;
+    int32_t rec_a = 0, rec_b = 0, rec_p = -1;
+    int rec_nch = 0;
+    float rec_D = 0.f, rec_U = 0.f, rec_kin = 0.f;
+    const bool resume = !SUB && A.resume;
+    if (resume) {
+        nn = A.u_nnodes[uid];
+        if (tid < nn) {
+            const int64_t v = nbase + tid;
+            rec_a = A.nd_a[v]; rec_b = A.nd_b[v]; rec_p = A.nd_parent[v];
+            rec_nch = A.nd_nchild[v];
+            rec_D = A.nd_D[v]; rec_U = A.nd_U[v];
+        }
+    }
     // ---- load the slot ------------------------------------------------------
-    // Every global load of a group is issued before any is used.  DH / 8
-    // consecutive threads hold a token; they also form ||k_t||, which equals
-    // ||k_circ_t|| (a rotation keeps the norm).
-    {
-        const bool own = tid < n;
-        const double kapv = own ? A.kappa[sa + tid] : 0.0;
-        const float rtv = own ? A.rtok[(size_t)lg * A.Nc + (sa - A.cs) + tid] : 0.f;
-        constexpr int TPT = DH / 8, GRP = 4;
-        const int iters = (n * DH + kNT * 8 - 1) / (kNT * 8);
+    const bool own = tid < n;   // n <= NT
+    const double kapv = own ? A.kappa[sa + tid] : 0.0;
+    const float rtv = own ? A.rtok[(size_t)lg * A.Nc + (sa - A.cs) + tid] : 0.f;
+    bool bad = own && !isfinite(rtv);   // non-finite probe weights or token values
+    bool rotated = false;
+    if constexpr (std::is_same<Tin, __nv_bfloat16>::value) {
+        if (A.Eg) {
+            // Only the rotated keys are needed: HALF / 8 consecutive threads
+            // hold a token, each the 8 rotation pairs (i, i + d/2) from its
+            // i; keys, values and rotations are all loaded before any is used.
+            // The thread also forms its part of ||k_t||^2, which equals
+            // ||k_circ_t||^2 (a rotation keeps the norm).
+            rotated = true;
+            constexpr int TPT = HALF / 8, TPI = NT / TPT;   // threads per token, tokens per iteration
+            const int i = (tid % TPT) * 8;
+            for (int t0 = 0; t0 < n; t0 += TPI) {
+                const int t = t0 + tid / TPT;
+                const bool in = t < n;
+                Raw8<Tin> k0, k1, v0, v1;
+                float4 cs[4];
+                if (in) {
+                    const size_t e = (size_t)t * DH + i;
+                    k0.load(Kp + e); k1.load(Kp + e + HALF);
+                    v0.load(Vp + e); v1.load(Vp + e + HALF);
+                    const float4 *rp = reinterpret_cast<const float4 *>(A.rope + (size_t)(sa + t) * HALF + i);
+#pragma unroll
+                    for (int q = 0; q < 4; q++) cs[q] = rp[q];
+                }
+                float ss0 = 0.f, ss1 = 0.f;
+                if (in) {
+                    float x[8], y[8], lo[8], hi[8];
+                    k0.get(x);
+                    k1.get(y);
+#pragma unroll
+                    for (int u = 0; u < 8; u++) {
+                        const float cx = u & 1 ? cs[u / 2].z : cs[u / 2].x, cy = u & 1 ? cs[u / 2].w : cs[u / 2].y;
+                        ss0 = fmaf(x[u], x[u], ss0);
+                        ss1 = fmaf(y[u], y[u], ss1);
+                        lo[u] = x[u] * cx + y[u] * cy;
+                        hi[u] = y[u] * cx - x[u] * cy;
+                    }
+                    st8(&sm.kc[t][i], lo);
+                    st8(&sm.kc[t][i + HALF], hi);
+                    v0.get(x);
+                    v1.get(y);
+                    st8(&sm.vv[t][i], x);
+                    st8(&sm.vv[t][i + HALF], y);
+                }
+#pragma unroll
+                for (int o = 1; o < TPT; o <<= 1) {   // the chunks of each half, then the halves
+                    ss0 += __shfl_xor_sync(0xffffffffu, ss0, o);
+                    ss1 += __shfl_xor_sync(0xffffffffu, ss1, o);
+                }
+                if (in && i == 0) sm.RK[t].y = sqrtf(ss0 + ss1);
+            }
+        }
+    }
+    if (!rotated) {
+        // DH / 8 consecutive threads hold a token; every load of a group is
+        // issued before any is used
+        constexpr int TPT = DH / 8, GRP = 2;
+        const int iters = (n * DH + NT * 8 - 1) / (NT * 8);
         for (int i0 = 0; i0 < iters; i0 += GRP) {   // the same trip counts for every thread
             Raw8<Tin> kr[GRP], vr[GRP];
 #pragma unroll
             for (int q = 0; q < GRP; q++) {
-                const int e = (i0 + q) * kNT * 8 + tid * 8;
+                const int e = (i0 + q) * NT * 8 + tid * 8;
                 if (i0 + q < iters && e < n * DH) {
                     kr[q].load(Kp + e);
                     vr[q].load(Vp + e);
@@ -355,7 +535,7 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
 #pragma unroll
             for (int q = 0; q < GRP; q++) {
                 if (i0 + q >= iters) break;
-                const int e = (i0 + q) * kNT * 8 + tid * 8;
+                const int e = (i0 + q) * NT * 8 + tid * 8;
                 const bool in = e < n * DH;
                 const int t = e / DH, i = e - t * DH;
                 float ss = 0.f;
@@ -363,56 +543,57 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
                     float kx[8], vx[8];
                     kr[q].get(kx);
                     vr[q].get(vx);
+                    st8(&sm.kc[t][i], kx);
+                    st8(&sm.vv[t][i], vx);
 #pragma unroll
-                    for (int u = 0; u < 8; u++) {
-                        sm.kc[t][i + u] = kx[u];
-                        sm.vv[t][i + u] = vx[u];
-                        ss = fmaf(kx[u], kx[u], ss);
-                    }
+                    for (int u = 0; u < 8; u++) ss = fmaf(kx[u], kx[u], ss);
                 }
 #pragma unroll
                 for (int o = 1; o < TPT; o <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-                if (in && i == 0) sm.kn[t] = sqrtf(ss);
+                if (in && i == 0) sm.RK[t].y = sqrtf(ss);
             }
         }
-        for (int t = tid; t < n; t += kNT) {
-            sm.kap[t] = okey(t == tid ? kapv : A.kappa[sa + t]);
-            sm.Rt[t] = t == tid ? rtv : A.rtok[(size_t)lg * A.Nc + (sa - A.cs) + t];
-        }
     }
-    // probe registers: thread (pp, c) owns probes pp and pp + 32, elements
-    // 4 c + 32 g + j; the 8 chunk lanes of a pair read 128 contiguous bytes
-    const int c = lane / kPPW, pp = warp * kPPW + (lane & (kPPW - 1));
-    float2 qa0[CH / 2], qa1[CH / 2];   // q of the two probes as element pairs
-    float mu0 = 0.f, mu1 = 0.f, invZ0 = 0.f, invZ1 = 0.f;
-#pragma unroll
-    for (int h = 0; h < 2; h++) {
-        const int u = pp + kNPP * h;
-        float2 *qd = h ? qa1 : qa0;
+    if (own) {
+        sm.kap[tid] = okey(kapv);
+        sm.RK[tid].x = rtv;
+    }
+    if (resume && tid < nn && rec_p >= 0) rec_kin = A.nd_kappa[rec_p];
+    // thread (pp, c) owns probes pp and pp + 32, elements 4 c + 32 g + j; the
+    // 8 chunk lanes of a pair read 128 contiguous bytes
+    const int c = lane / kPPW, pp = dwarp * kPPW + (lane & (kPPW - 1));
+    auto qrow = [&](int u) -> size_t { return ((size_t)l * A.Hq + g * A.gq + (u % A.gq)) * A.W + u; };
+    auto load_q = [&](float2 *qd, int u) {   // the thread's chunk of probe u's query as element pairs
         if (u < A.W) {
-            const size_t row = ((size_t)l * A.Hq + g * A.gq + (u % A.gq)) * A.W + u;
-            const Tin *qp = static_cast<const Tin *>(A.Q) + row * DH + 4 * c;
+            const Tin *qp = static_cast<const Tin *>(A.Q) + qrow(u) * DH + 4 * c;
 #pragma unroll
             for (int gi = 0; gi < NG; gi++) {
-                float4 x = ld4(qp + 32 * gi);
+                const float4 x = ld4(qp + 32 * gi);
                 qd[2 * gi] = make_float2(x.x, x.y);
                 qd[2 * gi + 1] = make_float2(x.z, x.w);
             }
-            (h ? mu1 : mu0) = A.row_m[row];
-            (h ? invZ1 : invZ0) = 1.0f / A.row_Z[row];
         } else {
 #pragma unroll
             for (int q = 0; q < CH / 2; q++) qd[q] = make_float2(0.f, 0.f);
         }
-    }
-    __syncthreads();
-
-    // ---- E[t][u] from the raw (post-RoPE) keys -------------------------------
+    };
+    // logits: the lane's reduced value belongs to probe pp + 32 (c / 4); the
+    // candidate sums: lane p of a warp takes the probes p and p + 32
+    const int ulog = pp + kNPP * (c >> 2);
+    const float mu_log = ulog < A.W ? A.row_m[qrow(ulog)] : 0.f;
+    const float invZ0 = lane < A.W ? 1.0f / A.row_Z[qrow(lane)] : 0.f;
+    const float invZ1 = lane + kNPP < A.W ? 1.0f / A.row_Z[qrow(lane + kNPP)] : 0.f;
+    // ---- E[t][u] ---------------------------------------------------------------
     if (A.Eg) {
-        cp_async_wait<0>();   // the copies above have landed (each thread its own)
+        cp_async_wait<0>();   // the thread's own copies have landed
+        for (int idx = tid; idx < n * (2 * kNPP / 4); idx += NT) {
+            const float4 e = reinterpret_cast<const float4 *>(Ef)[idx];
+            bad |= !(isfinite(e.x) && isfinite(e.y) && isfinite(e.z) && isfinite(e.w));
+        }
     } else if constexpr (std::is_same<Tin, __nv_bfloat16>::value) {
         // Tensor cores: logits = Q_probes (64 x DH) . K_slot^T, one 16x8 tile
         // per (probe block, token block); warp w keeps probe block w % 4.
+        __syncthreads();   // the raw keys
         constexpr int MT = 4, WSTEP = NWARPS / MT;
         const int gr = lane >> 2, c2 = 2 * (lane & 3);
         const int mt = warp % MT;
@@ -452,7 +633,13 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
             }
         }
     } else {
-        for (int t = 0; t < n; t++) {
+        __syncthreads();   // the raw keys
+        float2 qa0[CH / 2], qa1[CH / 2];
+        load_q(qa0, pp);
+        load_q(qa1, pp + kNPP);
+        const float mu0 = pp < A.W ? A.row_m[qrow(pp)] : 0.f;
+        const float mu1 = pp + kNPP < A.W ? A.row_m[qrow(pp + kNPP)] : 0.f;
+        for (int t = DIRS == 2 ? warp / (kNT / 32) : 0; t < n; t += DIRS) {
             float2 x0 = make_float2(0.f, 0.f), x1 = make_float2(0.f, 0.f);
 #pragma unroll
             for (int gi = 0; gi < NG; gi++) {
@@ -472,15 +659,15 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
                                           pp + kNPP < A.W ? expf(y1 * A.inv_sqrt_d - mu1) : 0.f);
         }
     }
-    __syncthreads();
+    if (!A.Eg) {
+        __syncthreads();
+        for (int e = tid; e < n * 2 * kNPP; e += NT) bad |= !isfinite(Ef[e]);
+    }
     // Non-finite probe weights or token values (NaN/Inf in K, Q or the row
     // statistics) make every decision of the unit meaningless: record the
     // unit as a single uncovered leaf with zero gain and flag the error, which
     // the host reports as GKV_ENONFINITE at the allocation's count sync.
     {
-        bool bad = false;
-        for (int e = tid; e < n * 2 * kNPP; e += kNT) bad |= !isfinite(Ef[e]);
-        for (int t = tid; t < n; t += kNT) bad |= !isfinite(sm.Rt[t]);
         if (__syncthreads_or(bad)) {
             if constexpr (SUB) {   // the node stays a leaf; the unit is reported
                 if (tid == 0) {
@@ -499,7 +686,7 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
                 A.u_nnodes[uid] = 1; A.u_Uadd[uid] = 0.f; A.u_Ddrop[uid] = 0.f; A.u_sel[uid] = 0;
                 A.u_pend[uid] = -1.f;
             }
-            for (int k = tid; k < 2 * n; k += kNT) A.nd_cost[nbase + k] = 0;
+            for (int k = tid; k < 2 * n; k += NT) A.nd_cost[nbase + k] = 0;
             return;
         }
     }
@@ -509,7 +696,7 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
     bool ufl = false;
     if (A.fl_acc) {
         bool any = false;
-        for (int t = tid; t < n; t += kNT) {
+        for (int t = tid; t < n; t += NT) {
             const size_t q = (size_t)lg * A.Nc + (sa - A.cs) + t;
             const bool ac = A.fl_acc[q] != 0;
             sm.Ff[t] = ac ? A.fl_f[q] : -INFINITY;
@@ -517,15 +704,14 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
         }
         ufl = __syncthreads_or(any);
     }
-    // ---- k_circ = RoPE^-1(k, t) ----------------------------------------------
-    // batches of RB rotation-table loads are issued before any is used
-    {
-        constexpr int RB = 8;
-        for (int e0 = tid; e0 < n * HALF; e0 += kNT * RB) {
+    // ---- k_circ = RoPE^-1(k, t), where the raw keys were needed ----------------
+    if (!rotated) {
+        constexpr int RB = 4;   // rotation-table loads issued before any is used
+        for (int e0 = tid; e0 < n * HALF; e0 += NT * RB) {
             float2 cs[RB];
 #pragma unroll
             for (int q = 0; q < RB; q++) {
-                const int e = e0 + q * kNT;
+                const int e = e0 + q * NT;
                 if (e < n * HALF) {
                     const int t = e / HALF, i = e - t * HALF;
                     cs[q] = A.rope[(size_t)(sa + t) * HALF + i];
@@ -533,7 +719,7 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
             }
 #pragma unroll
             for (int q = 0; q < RB; q++) {
-                const int e = e0 + q * kNT;
+                const int e = e0 + q * NT;
                 if (e < n * HALF) {
                     const int t = e / HALF, i = e - t * HALF;
                     const float x = sm.kc[t][i], y = sm.kc[t][i + HALF];
@@ -547,214 +733,202 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
     if constexpr (SUB) {
         if (tid == 0) {
             NodeS &nd = sm.nodes[0];
-            nd.a = 0; nd.b = (short)n; nd.parent = -1; nd.child0 = -1; nd.nchild = -1;
+            nd.a = 0; nd.b = (short)n; nd.nchild = -1;
             nd.D = A.nd_D[gv_sub];
             const int32_t pg = A.nd_parent[gv_sub];   // a node of the long unit, already evaluated
             nd.kin = pg < 0 ? FLT_MAX : A.nd_kappa[pg];
-            sm.nnodes = 1;
-            sm.lvl[0][0] = 0;
-            sm.nlvl[0] = 1;
             sm.pend = -1.f;
         }
-    } else if (!A.resume) {
+        if (tid < S::MW) sm.lvl[0][tid] = tid == 0 ? 1u : 0u;
+        nn = 1;
+    } else if (!resume) {
         if (warp == 0) {
             float r = 0.f;
-            for (int t = lane; t < n; t += 32) r += sm.Rt[t];
+            for (int t = lane; t < n; t += 32) r += sm.RK[t].x;
             r = warp_sum(r);
             if (lane == 0) {
                 NodeS &nd = sm.nodes[0];
-                nd.a = 0; nd.b = (short)n; nd.parent = -1; nd.child0 = -1; nd.nchild = 0;
+                nd.a = 0; nd.b = (short)n; nd.nchild = 0;
                 nd.D = 0.f; nd.kin = 0.f;
                 sm.rootR = r;
-                sm.nnodes = 1;
-                sm.lvl[0][0] = 0;
-                sm.nlvl[0] = 1;
                 sm.pend = -1.f;
                 A.nd_a[nbase] = sa; A.nd_b[nbase] = sb; A.nd_R[nbase] = (float)r;
                 A.nd_parent[nbase] = (int32_t)(-2 - uid);
                 A.nd_unit[nbase] = (int32_t)uid;
             }
         }
+        if (tid < S::MW) sm.lvl[0][tid] = tid == 0 ? 1u : 0u;
+        nn = 1;
     } else {
-        const int nn = A.u_nnodes[uid];
-        float *bnd_stage = &sm.redD[0][0];   // scratch until the first evaluation
-        static_assert(sizeof(sm.redD) >= sizeof(float) * S::MAXNODES, "bound staging");
-        for (int k = tid; k < nn; k += kNT) {
-            const int64_t v = nbase + k;
-            NodeS &nd = sm.nodes[k];
-            nd.a = (short)(A.nd_a[v] - sa);
-            nd.b = (short)(A.nd_b[v] - sa);
-            int32_t pg = A.nd_parent[v];
-            nd.parent = pg < 0 ? (short)-1 : (short)(pg - nbase);
-            nd.child0 = (short)A.nd_child0[v];
-            nd.nchild = A.nd_nchild[v];
-            nd.D = A.nd_D[v];
-            nd.kin = pg < 0 ? (ufl ? FLT_MAX : A.u_Uadd[uid]) : A.nd_kappa[pg];
-            bnd_stage[k] = nd.nchild == -1 ? A.nd_U[v] : -1.f;   // key bound of a pending node
-        }
-        if (tid == 0) { sm.nnodes = nn; sm.nlvl[0] = 0; sm.pend = -1.f; }
+        // the pending nodes whose key bound reaches tau form the first level
+        if (tid == 0) sm.pend = -1.f;
         __syncthreads();
-        if (tid == 0) {   // pending nodes that qualify, in creation order
-            for (int k = 0; k < nn; k++) {
-                if (sm.nodes[k].nchild != -1) continue;
-                if (bnd_stage[k] >= A.tau) sm.lvl[0][sm.nlvl[0]++] = (short)k;
-                else sm.pend = fmaxf(sm.pend, bnd_stage[k]);
+        bool q = false;
+        if (tid < nn) {
+            NodeS &nd = sm.nodes[tid];
+            nd.a = (short)(rec_a - sa);
+            nd.b = (short)(rec_b - sa);
+            nd.nchild = (signed char)rec_nch;
+            nd.D = rec_D;
+            nd.kin = rec_p < 0 ? (ufl ? FLT_MAX : A.u_Uadd[uid]) : rec_kin;
+            if (rec_nch == -1) {   // nd_U holds the key bound of a pending node
+                q = rec_U >= A.tau;
+                if (!q) atomicMax(reinterpret_cast<int *>(&sm.pend), __float_as_int(rec_U));
             }
         }
+        const unsigned m = __ballot_sync(0xffffffffu, q);
+        if (lane == 0 && warp < S::MW) sm.lvl[0][warp] = m;
     }
     __syncthreads();
 
-    unsigned long long w_scan = 0, w_eval = 0, w_len = 0;   // work counters (lane 0 of each warp)
+    int upre = 0, usuf = 0;   // the batch's candidate entries per direction
+    unsigned int w_scan = 0, w_eval = 0, w_len = 0;   // work counters (lane 0 of each warp)
 
-    // Prototypes of the batch's prefix (or suffix) candidates, warp per
-    // candidate; reserved entries a node did not use are empty and skipped.
+    // candidate rows of a direction: prefixes k, suffixes k - kNCD (after the
+    // prefixes' rows when the directions run side by side)
+    auto row_of = [](int k) { return DIRS == 2 ? k : (k >= kNCD ? k - kNCD : k); };
+
+    // Prototype (ktil, vtil, m_eff) of candidate k from its interval's sums.
+    constexpr int PPL = HALF / 32;   // rotation pairs per lane: (i, i + d/2), i = PPL lane + j
+    using PS = ProtoSum<PPL, HALF>;
+    const int pi0 = lane * PPL;
+    auto finish_proto = [&](int k, int nJ, const float2 *rot, const PS &acc) {
+        const int row = row_of(k);
+        const float rs = acc.q.x, ks = acc.q.y;
+        const float ninv = 1.0f / (float)nJ;
+        const float beta = (float)A.base_frac * (rs * ninv);
+        const float winv = 1.0f / ((rs + (float)nJ * beta) + A.eps);
+        float mu2 = 0.f;
+#pragma unroll
+        for (int j = 0; j < PPL; j++) {
+            float m0, m1, r0, r1, s0, s1;
+            acc.get(j, m0, m1, r0, r1, s0, s1);
+            const float a0 = m0 * ninv, a1 = m1 * ninv;
+            mu2 = fmaf(a0, a0, fmaf(a1, a1, mu2));
+            const float2 cs = rot[j];
+            sm.ktil[row][pi0 + j] = a0 * cs.x - a1 * cs.y;
+            sm.ktil[row][pi0 + j + HALF] = a0 * cs.y + a1 * cs.x;
+            sm.vtil[row][pi0 + j] = fmaf(beta, s0, r0) * winv;
+            sm.vtil[row][pi0 + j + HALF] = fmaf(beta, s1, r1) * winv;
+        }
+        mu2 = warp_sum(mu2);
+        if (lane == 0) {
+            const float coh = sqrtf(mu2) / (ks * ninv + A.eps);
+            const float me = (float)nJ * coh * coh;
+            sm.cand[k].meff = me < 1.0f ? 1.0f : (me > (float)nJ ? (float)nJ : me);
+        }
+    };
+    // Prototypes of the batch's candidates of one direction: a warp takes two
+    // adjacent candidates at a time (2 i, 2 i + 1).  Two prefixes of a node
+    // share their first tokens, so one running sum gives both; two suffixes
+    // share their last ones, so one set of loads feeds both sums.  Every sum
+    // runs over its interval's tokens in ascending order.
     auto prototypes = [&](bool suffix) {
-        const int kb = suffix ? kNCD : 0, ke = suffix ? kNCD + sm.batch_suf : sm.batch_pre;
-        for (int k = kb + warp; k < ke; k += NWARPS) {
-            const int row = k - kb;
-            const int ja = sm.cand[k].a, jb = sm.cand[k].b, nJ = jb - ja;
-            if (nJ <= 0) continue;
-            const int p = round_half_even_mid(sa + ja, sa + jb);   // absolute positions
-            // lane owns the rotation pairs (i, i + d/2), i = PPL lane + j; the
-            // rotation to p is loaded first so that its latency overlaps the sums
-            constexpr int PPL = HALF / 32;
-            const int i0 = lane * PPL;
-            float2 rot[PPL];
-#pragma unroll
-            for (int j = 0; j < PPL; j++) rot[j] = A.rope[(size_t)p * HALF + i0 + j];
-            // one pass over the tokens: sum k_circ, sum R v and sum v (the weights
-            // R_t + beta need the mean R, so sum (R + beta) v = sum R v + beta sum v),
-            // and the scalars sum R, sum ||k_circ|| (the same in every lane)
-            float m0[PPL], m1[PPL], r0[PPL], r1[PPL], s0[PPL], s1[PPL];
-            float rs = 0.f, ks = 0.f;
-#pragma unroll
-            for (int j = 0; j < PPL; j++) m0[j] = m1[j] = r0[j] = r1[j] = s0[j] = s1[j] = 0.f;
-#pragma unroll 8
-            for (int t = ja; t < jb; t++) {
-                float k0[PPL], k1[PPL], x0[PPL], x1[PPL];
-                ld_pairs<PPL>(&sm.kc[t][i0], k0);
-                ld_pairs<PPL>(&sm.kc[t][i0 + HALF], k1);
-                ld_pairs<PPL>(&sm.vv[t][i0], x0);
-                ld_pairs<PPL>(&sm.vv[t][i0 + HALF], x1);
-                const float rt = sm.Rt[t];
-                rs += rt;
-                ks += sm.kn[t];
-#pragma unroll
-                for (int j = 0; j < PPL; j++) {
-                    m0[j] += k0[j];
-                    m1[j] += k1[j];
-                    r0[j] = fmaf(rt, x0[j], r0[j]);
-                    r1[j] = fmaf(rt, x1[j], r1[j]);
-                    s0[j] += x0[j];
-                    s1[j] += x1[j];
-                }
-            }
-            const float ninv = 1.0f / (float)nJ;
-            const float beta = (float)A.base_frac * (rs * ninv);
-            const float winv = 1.0f / ((rs + (float)nJ * beta) + A.eps);
-            float mu2 = 0.f;
+        const int kb = suffix ? kNCD : 0, nk = suffix ? usuf : upre;
+        for (int i = 2 * dwarp; i < nk; i += 2 * (kNT / 32)) {
+            const int k0 = kb + i, k1 = k0 + 1;
+            int a0 = sm.cand[k0].a, b0 = sm.cand[k0].b;
+            int a1 = 0, b1 = 0;
+            if (i + 1 < nk) { a1 = sm.cand[k1].a; b1 = sm.cand[k1].b; }
+            float2 rot0[PPL], rot1[PPL];   // loaded first, so that their latency overlaps the sums
+            const int p0 = round_half_even_mid(sa + a0, sa + b0), p1 = round_half_even_mid(sa + a1, sa + b1);
 #pragma unroll
             for (int j = 0; j < PPL; j++) {
-                const float a0 = m0[j] * ninv, a1 = m1[j] * ninv;
-                mu2 = fmaf(a0, a0, fmaf(a1, a1, mu2));
-                const float2 cs = rot[j];
-                sm.ktil[row][i0 + j] = a0 * cs.x - a1 * cs.y;
-                sm.ktil[row][i0 + j + HALF] = a0 * cs.y + a1 * cs.x;
-                sm.vtil[row][i0 + j] = fmaf(beta, s0[j], r0[j]) * winv;
-                sm.vtil[row][i0 + j + HALF] = fmaf(beta, s1[j], r1[j]) * winv;
+                rot0[j] = b0 > a0 ? A.rope[(size_t)p0 * HALF + pi0 + j] : make_float2(0.f, 0.f);
+                rot1[j] = b1 > a1 ? A.rope[(size_t)p1 * HALF + pi0 + j] : make_float2(0.f, 0.f);
             }
-            mu2 = warp_sum(mu2);
-            if (lane == 0) {
-                const float coh = sqrtf(mu2) / (ks * ninv + A.eps);
-                const float me = (float)nJ * coh * coh;
-                sm.cand[k].meff = me < 1.0f ? 1.0f : (me > (float)nJ ? (float)nJ : me);
+            PS s0, s1;
+            s0.clear();
+            typename PS::Tok tk;
+            if (!suffix) {
+#pragma unroll 4
+                for (int t = a0; t < b0; t++) { tk.load(&sm.kc[t][pi0], &sm.vv[t][pi0], &sm.RK[t]); s0.add(tk); }
+                if (b0 > a0) finish_proto(k0, b0 - a0, rot0, s0);
+                int t = b0;
+                if (!(b0 > a0 && a1 == a0)) { s0.clear(); t = a1; }   // another node's prefix
+#pragma unroll 4
+                for (; t < b1; t++) { tk.load(&sm.kc[t][pi0], &sm.vv[t][pi0], &sm.RK[t]); s0.add(tk); }
+                if (b1 > a1) finish_proto(k1, b1 - a1, rot1, s0);
+            } else {
+                s1.clear();
+                const bool both = b1 > a1 && b1 == b0 && a1 < a0 && b0 > a0;
+                if (b1 > a1) {   // the longer one's own tokens
+                    const int stop = both ? a0 : b1;
+#pragma unroll 4
+                    for (int t = a1; t < stop; t++) { tk.load(&sm.kc[t][pi0], &sm.vv[t][pi0], &sm.RK[t]); s1.add(tk); }
+                }
+                if (both) {
+#pragma unroll 2
+                    for (int t = a0; t < b0; t++) {
+                        tk.load(&sm.kc[t][pi0], &sm.vv[t][pi0], &sm.RK[t]);
+                        s0.add(tk);
+                        s1.add(tk);
+                    }
+                } else {
+#pragma unroll 4
+                    for (int t = a0; t < b0; t++) { tk.load(&sm.kc[t][pi0], &sm.vv[t][pi0], &sm.RK[t]); s0.add(tk); }
+                }
+                if (b0 > a0) finish_proto(k0, b0 - a0, rot0, s0);
+                if (b1 > a1) finish_proto(k1, b1 - a1, rot1, s1);
             }
         }
     };
-    // D_u of candidate k (prototype row `row`) from the probe statistics Z, M
-    // of its interval; per-warp partial sums of pi_u D_u and pi_u.
     const float inv_sqrt_d = A.inv_sqrt_d, lamZ = A.lamZ, lamM = A.lamM, epsf = A.eps;
-    // D_u of candidate k (prototype row `row`) for the thread's two probes from
-    // their running statistics Z, M; per-warp partial sums of pi_u D_u and pi_u.
-    auto evaluate = [&](int k, int row, float Z0, float Z1, const float2 *M0, const float2 *M1) {
-        float2 kt[CH / 2];
+    // zt = m_eff exp(q_u . ktil / sqrt d - m_u) of the direction's candidates,
+    // four at a time: 8 dot products per thread chunk, one reduce-scatter, and
+    // one exponential per (candidate, probe).
+    auto logits = [&](bool suffix) {
+        const int kb = suffix ? kNCD : 0, nk = suffix ? usuf : upre;
+        if (nk == 0) return;
+        const int rb = row_of(kb);
+        float2 qa0[CH / 2], qa1[CH / 2];
+        load_q(qa0, pp);
+        load_q(qa1, pp + kNPP);
+        for (int i = 0; i < nk; i += 4) {
+            float v[8];   // [candidate i + (index & 3)][probe pp + 32 (index >> 2)]
 #pragma unroll
-        for (int gi = 0; gi < NG; gi++) {
-            const float4 x = *reinterpret_cast<const float4 *>(&sm.ktil[row][4 * c + 32 * gi]);
-            kt[2 * gi] = make_float2(x.x, x.y);
-            kt[2 * gi + 1] = make_float2(x.z, x.w);
-        }
-        float2 xa = make_float2(0.f, 0.f), xb = make_float2(0.f, 0.f);
+            for (int j = 0; j < 4; j++) {
+                const int row = rb + min(i + j, nk - 1);
+                float2 xa = make_float2(0.f, 0.f), xb = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int q = 0; q < CH / 2; q++) {
-            xa = ffma2(qa0[q], kt[q], xa);
-            xb = ffma2(qa1[q], kt[q], xb);
-        }
-        float x0 = xa.x + xa.y, x1 = xb.x + xb.y;
-#pragma unroll
-        for (int o = kPPW; o < 32; o <<= 1) {   // over the pair's chunk lanes
-            x0 += __shfl_xor_sync(0xffffffffu, x0, o);
-            x1 += __shfl_xor_sync(0xffffffffu, x1, o);
-        }
-        const float me = sm.cand[k].meff;
-        const float zt0 = me * expf(x0 * inv_sqrt_d - mu0), zt1 = me * expf(x1 * inv_sqrt_d - mu1);
-        const float2 nz0 = make_float2(-zt0, -zt0), nz1 = make_float2(-zt1, -zt1);
-        float2 r0 = make_float2(0.f, 0.f), r1 = r0, m0 = r0, m1 = r0;
-#pragma unroll
-        for (int gi = 0; gi < NG; gi++) {
-            const float4 x = *reinterpret_cast<const float4 *>(&sm.vtil[row][4 * c + 32 * gi]);
-            const float2 va = make_float2(x.x, x.y), vb = make_float2(x.z, x.w);
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const int q = 2 * gi + h;
-                const float2 vt = h ? vb : va;
-                const float2 d0 = ffma2(nz0, vt, M0[q]), d1 = ffma2(nz1, vt, M1[q]);   // M - zt vtil
-                r0 = ffma2(d0, d0, r0);
-                r1 = ffma2(d1, d1, r1);
-                m0 = ffma2(M0[q], M0[q], m0);
-                m1 = ffma2(M1[q], M1[q], m1);
+                for (int gi = 0; gi < NG; gi++) {
+                    const float4 x = *reinterpret_cast<const float4 *>(&sm.ktil[row][4 * c + 32 * gi]);
+                    const float2 ka = make_float2(x.x, x.y), kb2 = make_float2(x.z, x.w);
+                    xa = ffma2(qa0[2 * gi], ka, xa);
+                    xa = ffma2(qa0[2 * gi + 1], kb2, xa);
+                    xb = ffma2(qa1[2 * gi], ka, xb);
+                    xb = ffma2(qa1[2 * gi + 1], kb2, xb);
+                }
+                v[j] = xa.x + xa.y;
+                v[4 + j] = xb.x + xb.y;
+            }
+            const float x = reduce_scatter8(v, lane);
+            const int ii = i + (c & 3);
+            if (ii < nk) {
+                const float z = sm.cand[kb + ii].meff * expf(x * inv_sqrt_d - mu_log);
+                reinterpret_cast<float *>(&sm.zt[rb + ii][pp])[c >> 2] = z;
             }
         }
-        float res0 = r0.x + r0.y, res1 = r1.x + r1.y, mm0 = m0.x + m0.y, mm1 = m1.x + m1.y;
-#pragma unroll
-        for (int o = kPPW; o < 32; o <<= 1) {
-            res0 += __shfl_xor_sync(0xffffffffu, res0, o);
-            res1 += __shfl_xor_sync(0xffffffffu, res1, o);
-            mm0 += __shfl_xor_sync(0xffffffffu, mm0, o);
-            mm1 += __shfl_xor_sync(0xffffffffu, mm1, o);
-        }
-        // D_u (Eq. app_probe_distortion), weighted by the probe's attention
-        // mass; probes past W have E = 0 and invZ = 0, so they add nothing.
-        // Fast division: at most 2 ulp, far below the distortion tolerance.
-        const float dz0 = Z0 - zt0, dz1 = Z1 - zt1;
-        const float D0 = lamZ * __fdividef(dz0 * dz0, fmaf(Z0, Z0, epsf)) + lamM * __fdividef(res0, mm0 + epsf);
-        const float D1 = lamZ * __fdividef(dz1 * dz1, fmaf(Z1, Z1, epsf)) + lamM * __fdividef(res1, mm1 + epsf);
-        const float p0 = Z0 * invZ0, p1 = Z1 * invZ1;
-        float pd = fmaf(p0, D0, p1 * D1), pw = p0 + p1;
-#pragma unroll
-        for (int o = 1; o < kPPW; o <<= 1) {   // over the warp's probe pairs
-            pd += __shfl_xor_sync(0xffffffffu, pd, o);
-            pw += __shfl_xor_sync(0xffffffffu, pw, o);
-        }
-        if (lane == 0) { sm.redD[k][warp] = pd; sm.redP[k][warp] = pw; }
     };
-    // Probe scan of one node in one direction (SUF: suffixes, descending),
-    // evaluating each candidate when the running sums reach its far end.
+    // Probe scan of one node in one direction (SUF: suffixes, descending):
+    // running sums Z_u, M_u over the tokens; at each candidate's far end the
+    // thread's parts of ||M - zt vtil||^2 and ||M||^2, reduced two candidates
+    // at a time; ||M - zt vtil||^2 / ||M||^2 and Z go into the candidates' (no
+    // longer needed) key prototype rows.
     auto scan = [&](const BatchNode &B, auto SUF) {
         constexpr bool suffix = decltype(SUF)::value;
-        const int a = sm.nodes[B.node].a, b = sm.nodes[B.node].b;
         int k = suffix ? B.suf_b : B.pre_b;
         const int ke = suffix ? B.suf_e : B.pre_e;
         if (k >= ke) return;
+        int t = suffix ? sm.nodes[B.node].b - 1 : sm.nodes[B.node].a;   // next token to add
         float2 M0[CH / 2], M1[CH / 2];
-        float Z0 = 0.f, Z1 = 0.f;
+        float2 Z = make_float2(0.f, 0.f);
 #pragma unroll
         for (int q = 0; q < CH / 2; q++) M0[q] = M1[q] = make_float2(0.f, 0.f);
         auto add = [&](int t) {
             const float2 e = sm.E[t][pp];
             const float2 e0 = make_float2(e.x, e.x), e1 = make_float2(e.y, e.y);
-            Z0 += e.x;
-            Z1 += e.y;
+            Z = fadd2(Z, e);
 #pragma unroll
             for (int gi = 0; gi < NG; gi++) {
                 const float4 x = *reinterpret_cast<const float4 *>(&sm.vv[t][4 * c + 32 * gi]);
@@ -765,113 +939,161 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
                 M1[2 * gi + 1] = ffma2(e1, vb, M1[2 * gi + 1]);
             }
         };
-        int t = suffix ? b - 1 : a;   // next token to add
-        for (; k < ke; k++) {
+        auto partial = [&](int k, float *v) {
+            const int row = row_of(k);
             if (suffix) {
                 const int stop = sm.cand[k].a;   // candidates in descending start, all >= a
 #pragma unroll 1
                 for (; t >= stop; t--) add(t);
-                evaluate(k, k - kNCD, Z0, Z1, M0, M1);
             } else {
                 const int stop = sm.cand[k].b;   // candidates in ascending end, all <= b
 #pragma unroll 1
                 for (; t < stop; t++) add(t);
-                evaluate(k, k, Z0, Z1, M0, M1);
+            }
+            const float2 z = sm.zt[row][pp];
+            const float2 nz0 = make_float2(-z.x, -z.x), nz1 = make_float2(-z.y, -z.y);
+            float2 r0 = make_float2(0.f, 0.f), r1 = r0, m0 = r0, m1 = r0;
+#pragma unroll
+            for (int gi = 0; gi < NG; gi++) {
+                const float4 x = *reinterpret_cast<const float4 *>(&sm.vtil[row][4 * c + 32 * gi]);
+                const float2 va = make_float2(x.x, x.y), vb = make_float2(x.z, x.w);
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const int q = 2 * gi + h;
+                    const float2 vt = h ? vb : va;
+                    const float2 d0 = ffma2(nz0, vt, M0[q]), d1 = ffma2(nz1, vt, M1[q]);   // M - zt vtil
+                    r0 = ffma2(d0, d0, r0);
+                    r1 = ffma2(d1, d1, r1);
+                    m0 = ffma2(M0[q], M0[q], m0);
+                    m1 = ffma2(M1[q], M1[q], m1);
+                }
+            }
+            v[0] = r0.x + r0.y;   // index bits: probe pp + 32 (0), ||M||^2 (1), candidate (2)
+            v[1] = r1.x + r1.y;
+            v[2] = m0.x + m0.y;
+            v[3] = m1.x + m1.y;
+        };
+        for (; k < ke; k += 2) {
+            float v[8];
+            partial(k, v);
+            float Zk = (c & 1) ? Z.y : Z.x;   // of the candidate and probe that the lane ends up with
+            if (k + 1 < ke) {
+                partial(k + 1, v + 4);
+                if (c >> 2) Zk = (c & 1) ? Z.y : Z.x;
+            } else {
+                v[4] = v[5] = v[6] = v[7] = 0.f;
+            }
+            // lane c: probe pp + 32 (c & 1), ||M||^2 if c & 2 else the residual,
+            // candidate k + (c >> 2); the residual's lane divides, its partner
+            // keeps Z.  Fast division: at most 2 ulp, far below the distortion
+            // tolerance.
+            const float x = reduce_scatter8(v, lane);
+            const float y = __shfl_xor_sync(0xffffffffu, x, 2 * kPPW);
+            const int kk = k + (c >> 2);
+            if (kk < ke) sm.ktil[row_of(kk)][4 * pp + (c & 3)] = (c & 2) ? Zk : __fdividef(x, y + epsf);
+        }
+    };
+    // D_u (Eq. app_probe_distortion) of the direction's candidates, weighted by
+    // the probe's attention mass, and their means over the W probes: a warp per
+    // candidate, lane p the probes p and p + 32.  The sums run over groups of
+    // four lanes, then over the groups in order.  Probes past W have E = 0 and
+    // invZ = 0, so they add nothing.  Fast division: at most 2 ulp, far below
+    // the distortion tolerance.  Rows belong to the same warps as in
+    // prototypes(), which may follow without a barrier.
+    auto finish = [&](bool suffix) {
+        const int kb = suffix ? kNCD : 0, nk = suffix ? usuf : upre;
+        const float invW = 1.0f / A.W;
+        for (int i = dwarp; i < (nk + 1) / 2; i += kNT / 32) {
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const int k = kb + 2 * i + h;
+                if (2 * i + h >= nk || sm.cand[k].b <= sm.cand[k].a) continue;
+                const int row = row_of(k);
+                const float4 q = *reinterpret_cast<const float4 *>(&sm.ktil[row][4 * lane]);   // ratios, Z
+                const float2 z = sm.zt[row][lane];
+                const float Z0 = q.z, Z1 = q.w;
+                const float dz0 = Z0 - z.x, dz1 = Z1 - z.y;
+                const float D0 = lamZ * __fdividef(dz0 * dz0, fmaf(Z0, Z0, epsf)) + lamM * q.x;
+                const float D1 = lamZ * __fdividef(dz1 * dz1, fmaf(Z1, Z1, epsf)) + lamM * q.y;
+                const float p0 = Z0 * invZ0, p1 = Z1 * invZ1;
+                float pd = fmaf(p0, D0, p1 * D1), pw = p0 + p1;
+#pragma unroll
+                for (int o = 1; o < kPPW; o <<= 1) {
+                    pd += __shfl_xor_sync(0xffffffffu, pd, o);
+                    pw += __shfl_xor_sync(0xffffffffu, pw, o);
+                }
+                const float x = (lane & 1) ? pw : pd;   // even lanes sum D, odd lanes the mass
+                float d = 0.f;
+#pragma unroll
+                for (int w = 0; w < 32 / kPPW; w++) d += __shfl_sync(0xffffffffu, x, kPPW * w + (lane & 1));
+                if (lane < 2) (lane ? sm.candP : sm.candD)[k] = d * invW;
             }
         }
+        __syncwarp();   // the rows are free
     };
 
     int cur = 0;
-    int levels_left = A.max_levels;
-    while (sm.nlvl[cur] > 0) {
-        const int nl = sm.nlvl[cur];
-        if (levels_left == 0) {   // depth limit: the level's nodes stay pending
-            if (tid == 0) {
-                float pm = sm.pend;
-                for (int k = 0; k < nl; k++) {
-                    const int v = sm.lvl[cur][k];
-                    A.nd_nchild[gidx(v)] = -1;
-                    pm = fmaxf(pm, A.nd_U[gidx(v)]);   // the key bound written at its creation
-                }
-                sm.pend = pm;
-            }
-            break;
-        }
-        levels_left--;
-        if (tid == 0) { sm.nlvl[cur ^ 1] = 0; sm.batch_next = 0; }
-        __syncthreads();
-        while (sm.batch_next < nl) {
-            // ---- batch assignment (thread 0) --------------------------------
-            if (tid == 0) {
-                int nb = 0, upre = 0, usuf = 0, k = sm.batch_next;
-                while (k < nl && nb < S::NB) {
-                    const int v = sm.lvl[cur][k];
-                    const int nv = sm.nodes[v].b - sm.nodes[v].a;
-                    const bool root = v == 0 && fresh;
-                    const int nc = (nv >= 3 && !(root && A.root_only)) ? min(A.k_cand + 1, nv - 1) + 1 : 0;
-                    const int bp = nc + (root ? 1 : 0), bs = nc;
-                    if (upre + bp > kNCD || usuf + bs > kNCD) break;
-                    sm.bn[nb].node = v;
-                    sm.bn[nb].pre_b = upre;
-                    sm.bn[nb].suf_b = kNCD + usuf;
-                    upre += bp;
-                    usuf += bs;
-                    sm.bn[nb].pre_r = upre;
-                    sm.bn[nb].suf_r = kNCD + usuf;
-                    nb++;
-                    k++;
-                }
-                sm.batch_n = nb;
-                sm.batch_next = k;
-                sm.batch_pre = upre;
-                sm.batch_suf = usuf;
-            }
-            __syncthreads();
-            const int nb = sm.batch_n;
-            // ---- phase A: cut candidates per node (warp per node) ------------
-            for (int bi = warp; bi < nb; bi += NWARPS) {
-                BatchNode &B = sm.bn[bi];
-                const int v = B.node;
+    for (int levels_left = A.max_levels;; cur ^= 1) {
+        unsigned any = 0;
+        for (int w = 0; w < S::MW; w++) any |= sm.lvl[cur][w];
+        if (!any) break;
+        levels_left--;   // the last level's children stay pending (D2)
+        if (tid < S::MW) sm.lvl[cur ^ 1][tid] = 0;
+        int lw = 0;
+        unsigned lbits = sm.lvl[cur][0];
+        for (;;) {
+            // ---- batch: the level's next nodes in creation order.  Every warp
+            // walks them; phase A (cut candidates) runs on a node's own warp.
+            int nb = 0, nops = 0;
+            upre = usuf = 0;
+            while (nb < S::NB) {
+                while (!lbits && lw < S::MW - 1) lbits = sm.lvl[cur][++lw];
+                if (!lbits) break;
+                const int v = lw * 32 + __ffs(lbits) - 1;
                 const int a = sm.nodes[v].a, b = sm.nodes[v].b, nv = b - a;
-                const bool ronly = v == 0 && fresh && A.root_only;   // only the node's own distortion
+                const bool root = v == 0 && fresh;
+                const bool ronly = root && A.root_only;   // only the node's own distortion
+                const int nc = (nv >= 3 && !ronly) ? min(A.k_cand + 1, nv - 1) + 1 : 0;
+                const int bp = nc + (root ? 1 : 0), bs = nc;
+                if (upre + bp > kNCD || usuf + bs > kNCS) break;
+                lbits &= lbits - 1;
+                const int pre_b = upre, suf_b = kNCD + usuf;
+                upre += bp;
+                usuf += bs;
+                const int op = nv >= 2 && !ronly ? nops++ : -1;
+                const int bi = nb++;
+                if (bi % NWARPS != warp) continue;
+                BatchNode &B = sm.bn[bi];
                 // top-K by curvature over positions [a, b-2] (ties: lower t)
-                unsigned sel[NMAX / 32];
-                unsigned long long kmin = ~0ull, kmax = 0ull;
+                unsigned sel[(NMAX + 31) / 32];
 #pragma unroll
-                for (int w = 0; w < NMAX / 32; w++) {
-                    int t = a + w * 32 + lane;
-                    bool in = !ronly && t <= b - 2;
+                for (int w = 0; w < (NMAX + 31) / 32; w++) {
+                    const int t = a + w * 32 + lane;
                     bool s = false;
-                    if (in) {
+                    if (!ronly && t <= b - 2) {
                         const unsigned long long kt = sm.kap[t];
-                        kmin = min(kmin, kt);
-                        kmax = max(kmax, kt);
                         int rank = 0;
+#pragma unroll 4
                         for (int q = a; q <= b - 2; q++) {
                             const unsigned long long kq = sm.kap[q];
                             rank += (kq > kt) || (kq == kt && q < t);
                         }
+                        if (rank == 0) B.khi = kt;
+                        if (rank == nv - 2) B.klo = kt;
                         s = rank < A.k_cand || t == a + nv / 2 - 1;   // + midpoint
                     }
                     sel[w] = __ballot_sync(0xffffffffu, s);
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    kmin = min(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
-                    kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
                 }
                 // salient token p* = argmax R_tok over [a, b) (ties: lower t)
                 float rb = -INFINITY;
                 int pb = 0x7fffffff;
                 for (int t = a + lane; t < b; t += 32) {
-                    float r = sm.Rt[t];
+                    const float r = sm.RK[t].x;
                     if (r > rb) { rb = r; pb = t; }
                 }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    float r2 = __shfl_xor_sync(0xffffffffu, rb, o);
-                    int p2 = __shfl_xor_sync(0xffffffffu, pb, o);
-                    if (r2 > rb || (r2 == rb && p2 < pb)) { rb = r2; pb = p2; }
+                {
+                    const unsigned key = fkey_ordered(rb), kmx = __reduce_max_sync(0xffffffffu, key);
+                    pb = __reduce_min_sync(0xffffffffu, key == kmx ? pb : 0x7fffffff);
                 }
                 if (pb < a || pb >= b) pb = a;   // only reachable with non-finite values
                 // a node holding an accepted floor position is extracted at the one
@@ -903,7 +1125,7 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
                 const int maxc = cands ? min(A.k_cand + 1, nv - 1) : 0;
                 int ncut = 0;
 #pragma unroll
-                for (int w = 0; w < NMAX / 32; w++) {
+                for (int w = 0; w < (NMAX + 31) / 32; w++) {
                     const unsigned m = sel[w];
                     const int q = ncut + __popc(m & ((1u << lane) - 1u));
                     if (((m >> lane) & 1u) && q < maxc) B.cut[q] = (int8_t)(a + w * 32 + lane + 1);
@@ -920,11 +1142,11 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
                 const unsigned pbm = __ballot_sync(FULL, hq && xi == pb);
                 const bool el_cand = cands && pb - a >= 2;
                 const bool el_sep = el_cand && pbm == 0u;
-                const int pidx = pv ? B.pre_b + __popc(pm & lt) + (el_sep && pb < xi ? 1 : 0) : -1;
-                const int eL_sep = B.pre_b + __popc(__ballot_sync(FULL, pv && xi < pb));
+                const int pidx = pv ? pre_b + __popc(pm & lt) + (el_sep && pb < xi ? 1 : 0) : -1;
+                const int eL_sep = pre_b + __popc(__ballot_sync(FULL, pv && xi < pb));
                 const int eL_cut = __shfl_sync(FULL, pidx, pbm ? __ffs(pbm) - 1 : 0);
                 if (hq) B.pidx[lane] = (int8_t)pidx;
-                if (pv) sm.cand[pidx] = {a, xi, 0.f};
+                if (pv) sm.cand[pidx] = {(short)a, (short)xi, 0.f};
                 // suffixes
                 const int er = pb + 1;
                 const bool sv = hq && b - xi >= 2;
@@ -932,75 +1154,83 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
                 const unsigned erm = __ballot_sync(FULL, hq && xi == er);
                 const bool er_cand = cands && b - er >= 2;
                 const bool er_sep = er_cand && erm == 0u;
-                const int sidx = sv ? B.suf_b + __popc(smk & gt) + (er_sep && er > xi ? 1 : 0) : -1;
-                const int eR_sep = B.suf_b + __popc(__ballot_sync(FULL, sv && xi > er));
+                const int sidx = sv ? suf_b + __popc(smk & gt) + (er_sep && er > xi ? 1 : 0) : -1;
+                const int eR_sep = suf_b + __popc(__ballot_sync(FULL, sv && xi > er));
                 const int eR_cut = __shfl_sync(FULL, sidx, erm ? __ffs(erm) - 1 : 0);
                 if (hq) B.sidx[lane] = (int8_t)sidx;
-                if (sv) sm.cand[sidx] = {xi, b, 0.f};
+                if (sv) sm.cand[sidx] = {(short)xi, (short)b, 0.f};
                 // work counters: tokens swept, candidates evaluated, their lengths
                 int len = (pv ? xi - a : 0) + (sv ? b - xi : 0);
                 int pe = pv ? xi : a, ss = sv ? xi : b;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    len += __shfl_xor_sync(FULL, len, o);
-                    pe = max(pe, __shfl_xor_sync(FULL, pe, o));
-                    ss = min(ss, __shfl_xor_sync(FULL, ss, o));
-                }
+                len = __reduce_add_sync(FULL, len);
+                pe = __reduce_max_sync(FULL, pe);
+                ss = __reduce_min_sync(FULL, ss);
                 if (lane == 0) {
-                    const double kmn = nv >= 2 ? okey_inv(kmin) : 0.0, kmx = nv >= 2 ? okey_inv(kmax) : 0.0;
-                    B.kmin = kmn;
-                    B.krange = kmx > kmn ? 1.0f / (float)(kmx - kmn) : 0.f;
-                    B.pstar = pb;
-                    B.forced = forced;
-                    B.ncut = ncut;
-                    B.eL = el_sep ? eL_sep : (el_cand ? eL_cut : -1);
-                    if (el_sep) sm.cand[eL_sep] = {a, pb, 0.f};
-                    int k = B.pre_b + __popc(pm) + (el_sep ? 1 : 0);
-                    const bool whole = v == 0 && fresh;
+                    B.node = (short)v;
+                    B.op = (short)op;
+                    B.pre_b = (int8_t)pre_b;
+                    B.suf_b = (int8_t)suf_b;
+                    B.pstar = (short)pb;
+                    B.forced = (int8_t)forced;
+                    B.ncut = (int8_t)ncut;
+                    B.eL = (int8_t)(el_sep ? eL_sep : (el_cand ? eL_cut : -1));
+                    if (el_sep) sm.cand[eL_sep] = {(short)a, (short)pb, 0.f};
+                    int k = pre_b + __popc(pm) + (el_sep ? 1 : 0);
                     B.whole = -1;
-                    if (whole) { sm.cand[k] = {a, b, 0.f}; B.whole = k++; }
-                    B.pre_e = k;
-                    B.eR = er_sep ? eR_sep : (er_cand ? eR_cut : -1);
-                    if (er_sep) sm.cand[eR_sep] = {er, b, 0.f};
-                    B.suf_e = B.suf_b + __popc(smk) + (er_sep ? 1 : 0);
-                    for (int q = B.pre_e; q < B.pre_r; q++) sm.cand[q].a = sm.cand[q].b = 0;
-                    for (int q = B.suf_e; q < B.suf_r; q++) sm.cand[q].a = sm.cand[q].b = 0;
+                    if (root) { sm.cand[k] = {(short)a, (short)b, 0.f}; B.whole = (int8_t)k++; }
+                    B.pre_e = (int8_t)k;
+                    B.eR = (int8_t)(er_sep ? eR_sep : (er_cand ? eR_cut : -1));
+                    if (er_sep) sm.cand[eR_sep] = {(short)er, (short)b, 0.f};
+                    B.suf_e = (int8_t)(suf_b + __popc(smk) + (er_sep ? 1 : 0));
+                    for (int q = B.pre_e; q < pre_b + bp; q++) sm.cand[q].a = sm.cand[q].b = 0;
+                    for (int q = B.suf_e; q < suf_b + bs; q++) sm.cand[q].a = sm.cand[q].b = 0;
                     if (el_sep) { pe = max(pe, pb); len += pb - a; }
                     if (er_sep) { ss = min(ss, er); len += b - er; }
-                    if (whole) { pe = b; len += b - a; }
+                    if (root) { pe = b; len += b - a; }
                     w_scan += (pe - a) + (b - ss);
-                    w_eval += (B.pre_e - B.pre_b) + (B.suf_e - B.suf_b);
+                    w_eval += (B.pre_e - pre_b) + (B.suf_e - suf_b);
                     w_len += len;
                 }
             }
+            // the ops' places in the global list, fetched while the batch is evaluated
+            if (nops > 0 && tid == NT - 1) sm.op_base = atomicAdd(A.n_ops, (unsigned)nops);
+            if (nb == 0) break;
             __syncthreads();
-            // ---- phases B/C: prefixes, then suffixes ---------------------------
-            prototypes(false);
-            __syncthreads();
-            for (int bi = 0; bi < nb; bi++) scan(sm.bn[bi], std::false_type());
-            __syncthreads();
-            prototypes(true);
-            __syncthreads();
-            for (int bi = 0; bi < nb; bi++) scan(sm.bn[bi], std::true_type());
+            // ---- phases B/C: prefixes and suffixes, side by side or in turn ------
+            if constexpr (DIRS == 2) {
+                const bool suf = warp >= kNT / 32;
+                prototypes(suf);
+                __syncthreads();
+                logits(suf);
+                __syncthreads();
+                for (int bi = 0; bi < nb; bi++) {
+                    if (suf) scan(sm.bn[bi], std::true_type());
+                    else scan(sm.bn[bi], std::false_type());
+                }
+                __syncthreads();
+                finish(suf);
+            } else {
+                prototypes(false);
+                __syncthreads();
+                logits(false);
+                __syncthreads();
+                for (int bi = 0; bi < nb; bi++) scan(sm.bn[bi], std::false_type());
+                __syncthreads();
+                finish(false);
+                prototypes(true);
+                __syncthreads();
+                logits(true);
+                __syncthreads();
+                for (int bi = 0; bi < nb; bi++) scan(sm.bn[bi], std::true_type());
+                __syncthreads();
+                finish(true);
+            }
             __syncthreads();
             // ---- phase D1: candidate sums and decisions (warp per node) -------------
             for (int bi = warp; bi < nb; bi += NWARPS) {
                 BatchNode &B = sm.bn[bi];
                 NodeS &nd = sm.nodes[B.node];
                 const int a = nd.a, b = nd.b, nv = b - a;
-                // D and drop mass of this node's candidates: mean over the W probes
-                // of the per-warp partial sums
-                const float invW = 1.0f / A.W;
-                for (int k = lane; k < 2 * kNCD; k += 32) {
-                    const bool mine = k < kNCD ? (k >= B.pre_b && k < B.pre_e) : (k >= B.suf_b && k < B.suf_e);
-                    if (!mine) continue;
-                    float d = 0.f, pw = 0.f;
-#pragma unroll
-                    for (int w = 0; w < NWARPS; w++) { d += sm.redD[k][w]; pw += sm.redP[k][w]; }
-                    sm.candD[k] = d * invW;
-                    sm.candP[k] = pw * invW;
-                }
-                __syncwarp();
                 if (B.whole >= 0 && lane == 0) {   // root: D, Ddrop, Add gain (Eq. app_operation_gains)
                     const float Pd = sm.candP[B.whole];
                     const float D = nv >= 2 ? sm.candD[B.whole] : 0.f;
@@ -1022,8 +1252,8 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
                         B.nchild = 0;
                         if (nv == 2) {
                             B.nchild = 2;
-                            B.ca[0] = a; B.cb[0] = a + 1; B.cD[0] = 0.f;
-                            B.ca[1] = a + 1; B.cb[1] = b; B.cD[1] = 0.f;
+                            B.ca[0] = (short)a; B.cb[0] = (short)(a + 1); B.cD[0] = 0.f;
+                            B.ca[1] = (short)(a + 1); B.cb[1] = (short)b; B.cD[1] = 0.f;
                         }
                     }
                     continue;
@@ -1038,15 +1268,17 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
                     const float DR = B.sidx[lane] >= 0 ? sm.candD[B.sidx[lane]] : 0.f;
                     // normalised curvature: the difference is taken in fp64 (the
                     // curvatures may be close), the rest in fp32
-                    const float kh = (float)(okey_inv(sm.kap[xi - 1]) - B.kmin) * B.krange;
+                    const double kmn = okey_inv(B.klo), kmx = okey_inv(B.khi);
+                    const float krange = kmx > kmn ? 1.0f / (float)(kmx - kmn) : 0.f;
+                    const float kh = (float)(okey_inv(sm.kap[xi - 1]) - kmn) * krange;
                     best = ((DI - DL) - DR) + A.lam_kappa * kh;
                     bq = lane;
                 }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    float ov = __shfl_xor_sync(0xffffffffu, best, o);
-                    int oq = __shfl_xor_sync(0xffffffffu, bq, o);
-                    if (ov > best || (ov == best && oq < bq)) { best = ov; bq = oq; }
+                {
+                    const unsigned key = lane < B.ncut ? fkey_ordered(best) : 0u;
+                    const unsigned top = __ballot_sync(0xffffffffu, key == __reduce_max_sync(0xffffffffu, key) && lane < B.ncut);
+                    bq = top ? __ffs(top) - 1 : 0x7fffffff;
+                    best = __shfl_sync(0xffffffffu, best, bq & 31);
                 }
                 if (lane) continue;
                 int bxi = -1;
@@ -1072,12 +1304,12 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
                 }
                 const float rho_ext = ne == 3 ? 0.5f * gext : gext;   // G_ext / (|children| - 1), exact
                 if (B.forced || rho_ext > best) {
-                    B.nchild = ne;
-                    for (int q = 0; q < ne; q++) { B.ca[q] = ea[q]; B.cb[q] = eb[q]; B.cD[q] = eD[q]; }
+                    B.nchild = (int8_t)ne;
+                    for (int q = 0; q < ne; q++) { B.ca[q] = (short)ea[q]; B.cb[q] = (short)eb[q]; B.cD[q] = eD[q]; }
                 } else {
                     B.nchild = 2;
-                    B.ca[0] = a; B.cb[0] = bxi; B.cD[0] = bL;
-                    B.ca[1] = bxi; B.cb[1] = b; B.cD[1] = bR;
+                    B.ca[0] = (short)a; B.cb[0] = (short)bxi; B.cD[0] = bL;
+                    B.ca[1] = (short)bxi; B.cb[1] = (short)b; B.cD[1] = bR;
                 }
             }
             __syncthreads();
@@ -1088,24 +1320,24 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
                 const BatchNode &B = sm.bn[bi];
                 NodeS &nd = sm.nodes[B.node];
                 const int64_t gv = gidx(B.node);
-                int before = lane < bi ? max(sm.bn[lane].nchild, 0) : 0;
+                int before = lane < bi ? max((int)sm.bn[lane].nchild, 0) : 0;
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
                 const int nch = B.nchild;
                 if (nch < 0) {   // pending root: its split key is at most min(U_add, omega R D)
                     if (lane == 0) {
                         const float bnd = B.forced ? FLT_MAX : fminf(nd.kin, key_bound(om * sm.rootR * nd.D));
-                        nd.nchild = -1; nd.child0 = -1;
+                        nd.nchild = -1;
                         A.nd_child0[gv] = -1; A.nd_nchild[gv] = -1; A.nd_cost[gv] = 0;
                         A.nd_U[gv] = bnd; A.nd_kappa[gv] = 0.f; A.nd_sel[gv] = 0;
                         atomicMax(reinterpret_cast<int *>(&sm.pend), __float_as_int(bnd));
                     }
                     continue;
                 }
-                const int child0 = nch ? sm.nnodes + before : -1;
+                const int child0 = nch ? nn + before : -1;
                 if (nch == 0) {
                     if (lane == 0) {
-                        nd.nchild = 0; nd.child0 = -1;
+                        nd.nchild = 0;
                         A.nd_child0[gv] = -1; A.nd_nchild[gv] = 0; A.nd_cost[gv] = 0;
                         A.nd_U[gv] = 0.f; A.nd_kappa[gv] = 0.f; A.nd_sel[gv] = 0;
                     }
@@ -1114,7 +1346,7 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
                 float rch[3] = {0.f, 0.f, 0.f};
                 for (int q = 0; q < nch; q++) {
                     float r = 0.f;
-                    for (int t = B.ca[q] + lane; t < B.cb[q]; t += 32) r += sm.Rt[t];
+                    for (int t = B.ca[q] + lane; t < B.cb[q]; t += 32) r += sm.RK[t].x;
                     rch[q] = warp_sum(r);
                 }
                 const float rnode = (rch[0] + rch[1]) + rch[2];   // R of the node = sum over its children
@@ -1126,18 +1358,16 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
                 const float kap = B.forced ? FLT_MAX : fminf(U, nd.kin);
                 if (lane == 0) {
                     nd.nchild = (signed char)nch;
-                    nd.child0 = (short)child0;
                     A.nd_child0[gv] = (int32_t)(gidx(child0) - nbase); A.nd_nchild[gv] = (int8_t)nch;
                     A.nd_cost[gv] = (int8_t)cost; A.nd_U[gv] = U; A.nd_kappa[gv] = kap;
                     A.nd_sel[gv] = 0;
-                    A.ops[atomicAdd(A.n_ops, 1u)] = make_uint2(__float_as_uint(kap), ((uint32_t)gv << 1) | (uint32_t)(cost - 1));
+                    A.ops[sm.op_base + B.op] = make_uint2(__float_as_uint(kap), ((uint32_t)gv << 1) | (uint32_t)(cost - 1));
                 }
                 if (lane < nch) {   // lane q writes child q
                     const int q = lane, ci = child0 + q;
                     const float rq = q == 0 ? rch[0] : (q == 1 ? rch[1] : rch[2]);
                     NodeS &ch = sm.nodes[ci];
-                    ch.a = (short)B.ca[q]; ch.b = (short)B.cb[q]; ch.parent = (short)B.node;
-                    ch.child0 = -1; ch.nchild = 0; ch.D = B.cD[q]; ch.kin = kap;
+                    ch.a = B.ca[q]; ch.b = B.cb[q]; ch.nchild = 0; ch.D = B.cD[q]; ch.kin = kap;
                     const int64_t gc = gidx(ci);
                     A.nd_a[gc] = sa + B.ca[q]; A.nd_b[gc] = sa + B.cb[q];
                     A.nd_parent[gc] = (int32_t)gv; A.nd_unit[gc] = (int32_t)uid;
@@ -1152,10 +1382,9 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
                     A.nd_U[gc] = cbnd;
                     A.nd_kappa[gc] = 0.f; A.nd_sel[gc] = 0;
                     if (B.cb[q] - B.ca[q] >= 2) {
-                        if (cbnd >= A.tau) {   // evaluated at the next level of this launch
-                            const int pos = atomicAdd(&sm.nlvl[cur ^ 1], 1);
-                            sm.lvl[cur ^ 1][pos] = (short)ci;
-                        } else {   // its key cannot reach this pass's threshold: it stays pending
+                        if (cbnd >= A.tau && levels_left > 0) {   // evaluated at the next level of this launch
+                            atomicOr(&sm.lvl[cur ^ 1][ci >> 5], 1u << (ci & 31));
+                        } else {   // the launch's last level, or a key that cannot reach its threshold
                             ch.nchild = -1;
                             A.nd_nchild[gc] = -1;
                             atomicMax(reinterpret_cast<int *>(&sm.pend), __float_as_int(cbnd));
@@ -1163,32 +1392,16 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
                     }
                 }
             }
-            __syncthreads();
-            if (tid == 0) {   // nodes created by this batch (read by the next batch's D2)
-                int total = 0;
-                for (int bi = 0; bi < nb; bi++) total += max(sm.bn[bi].nchild, 0);
-                sm.nnodes += total;
-            }
+            // nodes created by this batch
+            nn += __reduce_add_sync(0xffffffffu, lane < nb ? max((int)sm.bn[lane].nchild, 0) : 0);
             __syncthreads();
         }
-        // keep the next level in creation order (atomic appends may permute it)
-        if (tid == 0) {
-            int nx = cur ^ 1, m = sm.nlvl[nx];
-            for (int x = 1; x < m; x++) {
-                short v = sm.lvl[nx][x];
-                int y = x - 1;
-                while (y >= 0 && sm.lvl[nx][y] > v) { sm.lvl[nx][y + 1] = sm.lvl[nx][y]; y--; }
-                sm.lvl[nx][y + 1] = v;
-            }
-        }
-        __syncthreads();
-        cur ^= 1;
     }
     if (lane == 0) { sm.wcnt[warp][0] = w_scan; sm.wcnt[warp][1] = w_eval; sm.wcnt[warp][2] = w_len; }
     __syncthreads();
     if (tid == 0) {
         if constexpr (!SUB) {   // a subtree stays inside its reserved slots; what it left pending is never needed
-            A.u_nnodes[uid] = sm.nnodes;
+            A.u_nnodes[uid] = nn;
             A.u_pend[uid] = sm.pend;
         }
         if (fresh) A.u_sel[uid] = 0;
@@ -1202,19 +1415,20 @@ __global__ void __launch_bounds__(kNT, NMAX <= 64 ? 2 : 1) unit_build_kernel(Bui
     }
     // unused node slots of the unit carry cost 0 (no op)
     if (fresh)
-        for (int k = sm.nnodes + tid; k < 2 * n; k += kNT) A.nd_cost[nbase + k] = 0;
+        for (int k = nn + tid; k < 2 * n; k += NT) A.nd_cost[nbase + k] = 0;
 }
 
 template <int DH, typename Tin, int NMAX, bool SUB = false>
 cudaError_t launch_t(Ctx &c, BuildArgs &A, unsigned grid, cudaStream_t s) {
-    using S = Smem<DH, Tin, NMAX>;
+    using S = Smem<DH, NMAX>;
     static_assert(sizeof(S) <= 227 * 1024, "unit kernel shared memory above the per-CTA limit");
+    static_assert((sizeof(S) + 1024) * S::CTAS <= 228 * 1024, "unit kernel shared memory above the SM's");
     if (grid == 0) return cudaSuccess;
     size_t sm = sizeof(S);
     cudaError_t e = cudaFuncSetAttribute(unit_build_kernel<DH, Tin, NMAX, SUB>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    unit_build_kernel<DH, Tin, NMAX, SUB><<<grid, kNT, sm, s>>>(A);
+    unit_build_kernel<DH, Tin, NMAX, SUB><<<grid, S::NT, sm, s>>>(A);
     c.launches += 1;
     return cudaGetLastError();
 }
@@ -1226,60 +1440,13 @@ cudaError_t launch_dt(Ctx &c, BuildArgs &A, unsigned grid, cudaStream_t s) {
 
 }  // namespace
 
-cudaError_t launch_unit_build(Ctx &c, const void *K, const void *V, const void *Q,
-                              const float *omega, const int32_t *slots, int J, int resume,
-                              int root_only, int max_levels, float tau, const int32_t *list_short, int n_short,
-                              const int32_t *list_long, int n_long, cudaStream_t s, int lg0, int nlg) {
+static void fill_args(BuildArgs &A, Ctx &c, const void *K, const void *V, const void *Q, const float *omega,
+                      const int32_t *slots, int J) {
     const gkv_params &p = c.p;
-    BuildArgs A;
     A.K = K; A.V = V; A.Q = Q;
     A.slots = slots; A.rope = c.w.rope; A.kappa = c.w.kappa;
     A.rtok = c.w.rtok; A.row_m = c.w.row_m; A.row_Z = c.w.row_Z; A.omega = omega;
-    A.Eg = use_tc(c) ? c.w.Eg : nullptr;
-    A.fl_acc = c.p.alpha_floor > 0.0 ? c.w.fl_acc : nullptr;
-    A.fl_f = c.w.fl_f;   // written by the tensor-core pass B
-    A.L = p.L; A.G = p.G; A.Hq = p.Hq; A.T = p.T; A.d = p.d; A.W = p.W; A.gq = p.Hq / p.G;
-    A.cs = p.ctx_start; A.Nc = c.Nc; A.J = J; A.k_cand = p.k_cand;
-    A.inv_sqrt_d = (float)(1.0 / sqrt((double)p.d));
-    A.lamZ = (float)p.lambda_Z; A.lamM = (float)p.lambda_M; A.eps = (float)p.eps;
-    A.lam_kappa = p.lambda_kappa; A.base_frac = p.base_frac;
-    A.resume = resume; A.subtree = 0; A.root_only = root_only; A.max_levels = max_levels; A.tau = tau;
-    A.nd_a = c.w.nd_a; A.nd_b = c.w.nd_b; A.nd_child0 = c.w.nd_child0;
-    A.nd_parent = c.w.nd_parent; A.nd_unit = c.w.nd_unit;
-    A.nd_nchild = c.w.nd_nchild; A.nd_cost = c.w.nd_cost;
-    A.ops = c.w.ops; A.n_ops = c.w.n_ops;
-    A.nd_D = c.w.nd_D; A.nd_R = c.w.nd_R; A.nd_U = c.w.nd_U; A.nd_kappa = c.w.nd_kappa;
-    A.nd_sel = c.w.nd_sel;
-    A.u_nnodes = c.w.u_nnodes; A.u_Uadd = c.w.u_Uadd; A.u_Ddrop = c.w.u_Ddrop; A.u_sel = c.w.u_sel;
-    A.u_pend = c.w.u_pend;
-    A.status = c.w.dev_int + 1;
-    A.work = c.w.work;
-    if (nlg < 0) nlg = p.L * p.G - lg0;
-    A.lg0 = lg0;
-    A.nlg = nlg;
-    const unsigned LG = (unsigned)nlg;
-    const bool bf = p.dtype == GKV_BF16;
-    // short slots (<= 64 tokens) on the two-CTA-per-SM instance, the rest on the 128-token one
-    A.list = list_short;
-    unsigned g1 = resume ? (unsigned)n_short : (unsigned)n_short * LG;
-    cudaError_t e = bf ? launch_dt<__nv_bfloat16, 64>(c, A, g1, s) : launch_dt<float, 64>(c, A, g1, s);
-    if (e != cudaSuccess) return e;
-    A.list = list_long;
-    unsigned g2 = resume ? (unsigned)n_long : (unsigned)n_long * LG;
-    return bf ? launch_dt<__nv_bfloat16, kMaxUnit>(c, A, g2, s) : launch_dt<float, kMaxUnit>(c, A, g2, s);
-}
-
-cudaError_t launch_unit_subtrees(Ctx &c, const void *K, const void *V, const void *Q, const float *omega,
-                                 const int32_t *slots, int J, const int32_t *list_short, int n_short,
-                                 const int32_t *list_long, int n_long, float tau_prune, cudaStream_t s) {
-    if (n_short + n_long == 0) return cudaSuccess;
-    cudaError_t e;
-    const gkv_params &p = c.p;
-    BuildArgs A;
-    A.K = K; A.V = V; A.Q = Q;
-    A.slots = slots; A.rope = c.w.rope; A.kappa = c.w.kappa;
-    A.rtok = c.w.rtok; A.row_m = c.w.row_m; A.row_Z = c.w.row_Z; A.omega = omega;
-    A.Eg = use_tc(c) ? c.w.Eg : nullptr;
+    A.Eg = use_tc(c) ? c.w.Eg : nullptr;   // written by the tensor-core pass B
     A.fl_acc = p.alpha_floor > 0.0 ? c.w.fl_acc : nullptr;
     A.fl_f = c.w.fl_f;
     A.L = p.L; A.G = p.G; A.Hq = p.Hq; A.T = p.T; A.d = p.d; A.W = p.W; A.gq = p.Hq / p.G;
@@ -1287,7 +1454,6 @@ cudaError_t launch_unit_subtrees(Ctx &c, const void *K, const void *V, const voi
     A.inv_sqrt_d = (float)(1.0 / sqrt((double)p.d));
     A.lamZ = (float)p.lambda_Z; A.lamM = (float)p.lambda_M; A.eps = (float)p.eps;
     A.lam_kappa = p.lambda_kappa; A.base_frac = p.base_frac;
-    A.resume = 0; A.subtree = 1; A.root_only = 0; A.max_levels = 4 * kMaxUnit; A.tau = tau_prune;
     A.nd_a = c.w.nd_a; A.nd_b = c.w.nd_b; A.nd_child0 = c.w.nd_child0;
     A.nd_parent = c.w.nd_parent; A.nd_unit = c.w.nd_unit;
     A.nd_nchild = c.w.nd_nchild; A.nd_cost = c.w.nd_cost;
@@ -1298,16 +1464,60 @@ cudaError_t launch_unit_subtrees(Ctx &c, const void *K, const void *V, const voi
     A.u_pend = c.w.u_pend;
     A.status = c.w.dev_int + 1;
     A.work = c.w.work;
+}
+
+// One launch per class, `per` CTAs per listed item.  Classes that together fit
+// one wave of a larger instance's CTAs share its launch.
+template <typename Tin, bool SUB>
+static cudaError_t launch_classes(Ctx &c, BuildArgs &A, const UnitLists &u, unsigned per, cudaStream_t s) {
+    const int64_t n0 = (int64_t)u.cnt[0] * per, n1 = (int64_t)u.cnt[1] * per, n2 = (int64_t)u.cnt[2] * per;
+    const int far = 1 << 30;
+    A.stride = u.stride;
+    auto range = [&](int a, int b) {   // classes [a, b]: returns the CTAs
+        A.list = u.list + a * u.stride;
+        A.c1 = b > a ? u.cnt[a] : far;
+        A.c2 = b > a + 1 ? u.cnt[a] + u.cnt[a + 1] : far;
+        int64_t n = 0;
+        for (int q = a; q <= b; q++) n += (int64_t)u.cnt[q] * per;
+        return (unsigned)n;
+    };
+    if (n0 + n1 + n2 <= c.num_sms) return launch_dt<Tin, kMaxUnit, SUB>(c, A, range(0, 2), s);
+    cudaError_t e = cudaSuccess;
+    if (n0 + n1 <= 2 * c.num_sms) {
+        e = launch_dt<Tin, kShortUnit, SUB>(c, A, range(0, 1), s);
+    } else {
+        e = launch_dt<Tin, kTinyUnit, SUB>(c, A, range(0, 0), s);
+        if (e == cudaSuccess) e = launch_dt<Tin, kShortUnit, SUB>(c, A, range(1, 1), s);
+    }
+    if (e == cudaSuccess) e = launch_dt<Tin, kMaxUnit, SUB>(c, A, range(2, 2), s);
+    return e;
+}
+
+cudaError_t launch_unit_build(Ctx &c, const void *K, const void *V, const void *Q,
+                              const float *omega, const int32_t *slots, int J, int resume,
+                              int root_only, int max_levels, float tau, const UnitLists &u, cudaStream_t s,
+                              int lg0, int nlg) {
+    BuildArgs A;
+    fill_args(A, c, K, V, Q, omega, slots, J);
+    A.resume = resume; A.root_only = root_only; A.max_levels = max_levels; A.tau = tau;
+    if (nlg < 0) nlg = c.p.L * c.p.G - lg0;
+    A.lg0 = lg0;
+    A.nlg = nlg;
+    const unsigned per = resume ? 1u : (unsigned)nlg;
+    return c.p.dtype == GKV_BF16 ? launch_classes<__nv_bfloat16, false>(c, A, u, per, s)
+                                 : launch_classes<float, false>(c, A, u, per, s);
+}
+
+cudaError_t launch_unit_subtrees(Ctx &c, const void *K, const void *V, const void *Q, const float *omega,
+                                 const int32_t *slots, int J, const UnitLists &u, float tau_prune,
+                                 cudaStream_t s) {
+    BuildArgs A;
+    fill_args(A, c, K, V, Q, omega, slots, J);
+    A.resume = 0; A.root_only = 0; A.max_levels = 4 * kMaxUnit; A.tau = tau_prune;
     A.lg0 = 0;
-    A.nlg = p.L * p.G;
-    const bool bf = p.dtype == GKV_BF16;
-    A.list = list_short;
-    e = bf ? launch_dt<__nv_bfloat16, 64, true>(c, A, (unsigned)n_short, s)
-           : launch_dt<float, 64, true>(c, A, (unsigned)n_short, s);
-    if (e != cudaSuccess) return e;
-    A.list = list_long;
-    return bf ? launch_dt<__nv_bfloat16, kMaxUnit, true>(c, A, (unsigned)n_long, s)
-              : launch_dt<float, kMaxUnit, true>(c, A, (unsigned)n_long, s);
+    A.nlg = c.p.L * c.p.G;
+    return c.p.dtype == GKV_BF16 ? launch_classes<__nv_bfloat16, true>(c, A, u, 1, s)
+                                 : launch_classes<float, true>(c, A, u, 1, s);
 }
 
 }  // namespace gkv

@@ -88,7 +88,7 @@ struct LongArgs {
     uint8_t *it_ufl;               // the node's unit holds a singleton-floor position
     LongRes *res;
     int32_t *u_start, *u_cnt;      // per listed unit: its block of work items
-    unsigned int *n_items;         // [3]: work items, small subtrees (<= kShortUnit, <= kMaxUnit tokens)
+    unsigned int *n_items;         // [4]: work items, small subtrees of each class
     unsigned int *it_next;         // the next work item to take (zero at the level's start)
     int32_t *sub;                  // [2][cap_items] small subtrees' roots (global node indices)
     int64_t cap_items;
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kLT) long_collect_kernel(LongArgs A) {
         // a subtree has none, but its bound is below a threshold that only
         // rises, so it never reaches this point; it is skipped all the same.
         if (A.nd_child0[v] < 0) continue;
-        const int cls = len <= kShortUnit ? 0 : 1;
+        const int cls = unit_class(len);
         const unsigned int pos = atomicAdd(&A.n_items[1 + cls], 1u);
         if ((int64_t)pos < A.cap_items) A.sub[(size_t)cls * A.cap_items + pos] = (int32_t)v;
         else atomicOr(A.status, 64);
@@ -1189,20 +1189,20 @@ cudaError_t launch_long_level(Ctx &c, const void *K, const void *V, const void *
     A.status = w.dev_int + 1;
     A.work = w.work;
     A.sub = w.long_sub;
-    A.it_next = w.long_n + 3;
-    cudaError_t e = cudaMemsetAsync(w.long_n, 0, 4 * sizeof(unsigned int), s);
+    A.it_next = w.long_n + 1 + kUnitClasses;
+    cudaError_t e = cudaMemsetAsync(w.long_n, 0, (2 + kUnitClasses) * sizeof(unsigned int), s);
     if (e != cudaSuccess) return e;
     long_collect_kernel<<<(unsigned)n_units, kLT, 0, s>>>(A);
     c.launches += 1;
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // the level's counts: long work items, small subtrees of each class
-    unsigned int cnt[3] = {0, 0, 0};
+    unsigned int cnt[1 + kUnitClasses] = {0, 0, 0, 0};
     e = cudaMemcpyAsync(cnt, w.long_n, sizeof cnt, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
-    for (int q = 0; q < 3; q++) cnt[q] = (unsigned)std::min<int64_t>((int64_t)cnt[q], w.long_cap);
-    if (n_items_host) *n_items_host = cnt[0] + cnt[1] + cnt[2];
+    for (int q = 0; q <= kUnitClasses; q++) cnt[q] = (unsigned)std::min<int64_t>((int64_t)cnt[q], w.long_cap);
+    if (n_items_host) *n_items_host = cnt[0] + cnt[1] + cnt[2] + cnt[3];
     if (cnt[0] > 0) {
         // one resident wave: items are taken dynamically
         int occ = 1;
@@ -1219,8 +1219,8 @@ cudaError_t launch_long_level(Ctx &c, const void *K, const void *V, const void *
         if (e != cudaSuccess) return e;
     }
     // nodes of at most kMaxUnit tokens: their subtrees on the unit kernel
-    return launch_unit_subtrees(c, K, V, Q, omega, slots, J, w.long_sub, (int)cnt[1], w.long_sub + w.long_cap,
-                                (int)cnt[2], tau_prune, s);
+    return launch_unit_subtrees(c, K, V, Q, omega, slots, J,
+                                {w.long_sub, w.long_cap, {(int)cnt[1], (int)cnt[2], (int)cnt[3]}}, tau_prune, s);
 }
 
 }  // namespace gkv

@@ -94,7 +94,7 @@ struct Workspace {
     uint8_t *u_sel = nullptr;      // Add selected (1), discarded tie (2)
     int32_t *u_count = nullptr;    // frontier entries per unit
     int64_t *u_off = nullptr;      // entry offset of each unit's frontier
-    int32_t *u_list = nullptr;     // compacted unit ids (ties)
+    int32_t *u_list = nullptr;     // [kUnitClasses][units_cap] work lists of the unit kernel
     long long *u_bsum = nullptr;   // [units_cap / 1024 + 2] block sums of the gather's offset scan
     long long *tie_bsum = nullptr; // [units_cap / 1024 + L G + 2] chunk sums of the allocation's tie scan
     // allocation
@@ -115,9 +115,9 @@ struct Workspace {
     uint8_t *long_ufl = nullptr;
     void *long_res = nullptr;      // [long_cap] results (long_res_bytes() each)
     int32_t *long_start = nullptr, *long_cnt = nullptr;   // [long_units_cap]
-    unsigned int *long_n = nullptr;                       // [4] the level's work items, small subtrees, next item
-                                                          //     of <= kShortUnit and <= kMaxUnit tokens
-    int32_t *long_sub = nullptr;    // [2][long_cap] the small subtrees' root nodes (global indices)
+    unsigned int *long_n = nullptr;                       // [5] the level's work items, small subtrees of each
+                                                          //     class, next item
+    int32_t *long_sub = nullptr;    // [kUnitClasses][long_cap] the small subtrees' root nodes (global indices)
     int32_t *long_slots = nullptr;  // [N_c + 1] slot indices of the long slots
     int32_t *long_list = nullptr;   // [units_cap] long units to resume
 };
@@ -282,6 +282,16 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
     return d;
 }
 
+__device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+
 // Two floats (exactly representable in bf16) packed as a bf16x2 operand word.
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
@@ -312,28 +322,37 @@ int tc_row_chunks(const Ctx &c);
 cudaError_t launch_row_stats_tc(Ctx &c, const void *K, const void *Q, cudaStream_t s, int lg0, int nlg);
 cudaError_t launch_token_values_tc(Ctx &c, const void *K, const void *Q, cudaStream_t s, int lg0, int nlg);
 cudaError_t launch_token_values(Ctx &c, const void *K, const void *Q, cudaStream_t s, int l0 = 0, int l1 = -1);
-// Slots of at most kShortUnit tokens run on the unit kernel instance that fits
-// two CTAs per SM; the work lists hold them (slot indices for a fresh build,
-// unit ids for a resumed one) separately from the longer ones.
+// Slots run on one of three instances of the unit kernel: up to kTinyUnit
+// tokens three CTAs fit on an SM, up to kShortUnit two, up to kMaxUnit one (of
+// twice the threads).  The work lists (slot indices for a fresh build, unit
+// ids for a resumed one, node indices in subtree mode) hold each class apart:
+// class q at list + q stride, cnt[q] entries.  A launch too small to fill the
+// GPU joins the next class up, so that all of its units run side by side.
+constexpr int kTinyUnit = 36;
 constexpr int kShortUnit = 64;
+constexpr int kUnitClasses = 3;
+__host__ __device__ __forceinline__ int unit_class(int n) { return n <= kTinyUnit ? 0 : (n <= kShortUnit ? 1 : 2); }
+struct UnitLists {
+    const int32_t *list;
+    int64_t stride;
+    int cnt[kUnitClasses];
+};
 cudaError_t launch_unit_build(Ctx &c, const void *K, const void *V, const void *Q,
                               const float *omega, const int32_t *slots, int J, int resume,
-                              int root_only, int max_levels, float tau, const int32_t *list_short,
-                              int n_short, const int32_t *list_long, int n_long, cudaStream_t s,
+                              int root_only, int max_levels, float tau, const UnitLists &u, cudaStream_t s,
                               int lg0 = 0, int nlg = -1);   // fresh launches: (l, g) in [lg0, lg0 + nlg);
 // Subtree mode of the unit kernel (build.cu): the listed pending nodes of
-// long units (global node indices; at most kShortUnit tokens in list_short,
-// at most kMaxUnit in list_long) each get their subtree built to the leaves
+// long units (global node indices) each get their subtree built to the leaves
 // into the node slots reserved for it (its child0, unit-relative), except the
 // children whose key bound is below tau_prune (the threshold of the ops built
 // so far: it only rises, so they can never be selected); they stay pending.
 cudaError_t launch_unit_subtrees(Ctx &c, const void *K, const void *V, const void *Q, const float *omega,
-                                 const int32_t *slots, int J, const int32_t *list_short, int n_short,
-                                 const int32_t *list_long, int n_long, float tau_prune, cudaStream_t s);
-// Slot indices split by length class: short ones at list[0, count[0]), those
-// of kShortUnit + 1 .. kMaxUnit tokens at list[J - count[1], J), longer ones
-// at long_slots[0, count[2]); count[3] receives the tokens of the longer ones.
-cudaError_t launch_slot_classes(Ctx &c, const int32_t *slots, int J, int32_t *list, int *count,
+                                 const int32_t *slots, int J, const UnitLists &u, float tau_prune,
+                                 cudaStream_t s);
+// Slot indices split by length class: class q at list + q stride, count[q]
+// entries, longer slots at long_slots[0, count[3]); count[4] receives the
+// tokens of the longer ones.
+cudaError_t launch_slot_classes(Ctx &c, const int32_t *slots, int J, int32_t *list, int64_t stride, int *count,
                                 int32_t *long_slots, cudaStream_t s);
 // One level of the trees of long units (build_long.cu): with fresh = 1 the
 // roots of the listed slots for (l, g) in [lg0, lg0 + nlg) (root_only: their
@@ -354,12 +373,11 @@ cudaError_t launch_long_units(Ctx &c, const int32_t *long_slots, int n_long, int
                               int32_t *out, cudaStream_t s);
 // Allocation threshold tau over the ops built so far (alloc_state prefix /
 // all-fit flag), and the units whose largest pending key bound reaches
-// max(tau, cut), split by slot length class: short units at list[0, count[0]),
-// those of up to kMaxUnit tokens at list[n_units - count[1], n_units), longer
-// ones at long_list[0, count[2]); *pend_pot receives the entries a complete
+// max(tau, cut), split by slot length class: class q at list + q stride,
+// count[q] entries, longer ones at long_list[0, count[3]); *pend_pot receives the entries a complete
 // expansion of every unit reaching tau could take.
 cudaError_t launch_threshold(Ctx &c, int J, cudaStream_t s);
-cudaError_t launch_prune_list(Ctx &c, const int32_t *slots, int J, int32_t *list, int *count,
+cudaError_t launch_prune_list(Ctx &c, const int32_t *slots, int J, int32_t *list, int64_t stride, int *count,
                               int32_t *long_list, cudaStream_t s);
 // Bound-ordered expansion: among the units whose largest pending key bound
 // reaches the threshold, the cut that keeps about `m` of them (the lower edge

@@ -1,0 +1,44 @@
+"""Slot lengths at the unit kernel's class edges against the oracle.
+
+The unit kernel has an instance for slots of up to 36, 64 and 128 tokens, and
+classes too small to fill the GPU share a launch: with no short slots beside
+the edge lengths every unit runs on the 128-token instance, with 200 of them
+the 36-token class joins the 64-token one, with 340 every class has its own
+launch.  The inputs cover the three ways the probe weights are formed (by the
+score pass; on mma.sync, above 256 probe rows per KV head; in fp32).
+"""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2608_07001_gb300 import synth
+from tests import parity as P
+
+pytestmark = pytest.mark.gpu
+
+EDGES = [36, 1, 128, 37, 2, 64, 3, 65, 35, 127, 63, 17]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__ as g
+    g.build()
+    assert torch.cuda.is_available()
+
+
+@pytest.mark.parametrize("fill", [0, 200, 340])
+@pytest.mark.parametrize("dtype,d,gq,W", [("bf16", 64, 4, 8), ("bf16", 128, 8, 40), ("fp32", 128, 2, 8)])
+def test_class_edges_match_the_oracle(dtype, d, gq, W, fill):
+    lens = EDGES + [1 + i % 3 for i in range(fill)]
+    w = dataclasses.replace(synth.WORKLOADS["small"], L=1, G=1, Hq=gq, d=d)
+    x = synth.make_inputs(w, T=sum(lens) + 32, W=W)
+    K, V, Q = x.K, x.V, x.Q
+    if dtype == "fp32":
+        K, V, Q = K.float(), V.float(), Q.float()
+    slots = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    B = K.shape[2] // 3
+    g = P.run_gpu(K, V, Q, B, w.rope_base, slot_starts=slots)
+    o = P.run_oracle(K, V, Q, B, w.rope_base, slot_starts=slots)
+    P.compare(g, o, torch.float32 if dtype == "fp32" else torch.bfloat16)
