@@ -59,9 +59,7 @@ constexpr int kNCL = 8;          // threads per probe pair (4-element groups, in
 constexpr int kPPW = 32 / kNCL;  // probe pairs per warp: lane = 4 c + (pair % 4), so that the
                                  // 4 lanes reading one 16-byte chunk are adjacent (one shared-
                                  // memory wavefront serves them; lanes 8 apart would not merge)
-constexpr int kNCD = 19;         // prefix candidates of a batch: 17 cuts + p* side + whole node
-constexpr int kNCS = 18;         // suffix candidates of a batch: 17 cuts + p* side
-constexpr int kNCA = kNCD + kNCS;   // candidate k: prefixes in [0, kNCD), suffixes in [kNCD, kNCA)
+constexpr int kNCR = 19;         // candidate rows held at a time: 17 cuts + p* side (+ 1)
 
 struct BuildArgs {
     const void *K, *V, *Q;
@@ -75,6 +73,7 @@ struct BuildArgs {
     int L, G, Hq, T, d, W, gq, cs, Nc, J, k_cand;
     float inv_sqrt_d, lamZ, lamM, eps;
     float lam_kappa, base_frac;
+    int prune;                   // lambda_Z, lambda_M >= 0, so every D >= 0: cuts may be ruled out by bounds
     // work list: fresh launches index (slot list entry, lg), resume launches units
     int resume;                  // 0: build from the root, 1: resume pending nodes
     int root_only;               // fresh: evaluate only the root's own distortion (split stays pending)
@@ -108,23 +107,38 @@ struct NodeS {
 
 struct BatchNode {
     unsigned long long klo, khi;   // smallest and largest curvature key over the node's cut positions
+    float kh[kMaxCuts];      // normalised curvature of the cuts
     float cD[3];
+    unsigned more;           // cuts that the first one evaluated does not rule out
     short node, pstar;
     short op;                // the node's place among the batch's Split ops (-1: none)
     short ca[3], cb[3];
     int8_t cut[kMaxCuts];    // local cut positions xi (ascending)
-    int8_t pidx[kMaxCuts];   // candidate index of [a, xi) (-1: single token)
-    int8_t sidx[kMaxCuts];   // candidate index of [xi, b) (-1: single token)
-    int8_t ncut, eL, eR, whole, nchild;
+    int8_t ncut, k1;         // cuts; the one of largest curvature reward
+    int8_t rl, rr, whole;    // rows of its sides (-1: single token) and of the node itself
+    int8_t nchild;           // -1: pending root, -2: undecided
     int8_t forced;           // extraction at a singleton-floor position (a floor op)
-    int8_t pre_b, pre_e, suf_b, suf_e;   // prefixes (ascending end) in [0, kNCD),
-                                         // suffixes (descending start) in [kNCD, kNCA)
+    int8_t ext;              // the extraction's sides are needed
+    int8_t pre_b, pre_e, suf_b, suf_e;   // rows: prefixes (ascending end), suffixes (descending start)
 };
 
 struct Cand {
     short a, b;      // local interval (a == b: unused entry)
     float meff;
 };
+
+// Sums of two products round one product and fuse the other.  Which one is
+// written out, so that the compiler's choice cannot move a result's last bit
+// (and with it a near-tie between cuts) from one build or instance to another.
+__device__ __forceinline__ void rotate_back(float x, float y, float c, float s, float &lo, float &hi) {
+    lo = fmaf(x, c, y * s);
+    hi = fmaf(y, c, -(x * s));
+}
+template <bool SINE_FUSED>
+__device__ __forceinline__ void rotate_to(float x, float y, float c, float s, float &lo, float &hi) {
+    lo = fmaf(x, c, -(y * s));
+    hi = SINE_FUSED ? fmaf(x, s, y * c) : fmaf(y, c, x * s);
+}
 
 // Upper bound of a split's utility: U = omega R (D - sum D_children) / cost
 // <= omega R D, since every D >= 0 and cost >= 1 (Eqs. app_operation_gains,
@@ -274,69 +288,87 @@ __device__ __forceinline__ float reduce_scatter8(const float v[8], int lane) {
     return keep + __shfl_xor_sync(0xffffffffu, send, 4 * kPPW);
 }
 
+// The same over four values; lane c ends with the sum of v[c & 3] (both halves
+// of the lanes hold it).
+__device__ __forceinline__ float reduce_scatter4(float v0, float v1, float v2, float v3, int lane) {
+    const bool h0 = lane & kPPW, h1 = lane & (2 * kPPW);
+    const float x0 = (h0 ? v1 : v0) + __shfl_xor_sync(0xffffffffu, h0 ? v0 : v1, kPPW);
+    const float x1 = (h0 ? v3 : v2) + __shfl_xor_sync(0xffffffffu, h0 ? v2 : v3, kPPW);
+    const float y = (h1 ? x1 : x0) + __shfl_xor_sync(0xffffffffu, h1 ? x0 : x1, 2 * kPPW);
+    return y + __shfl_xor_sync(0xffffffffu, y, 4 * kPPW);
+}
+
 // Running sums of an interval's prototype: PPL rotation pairs (i, i + d/2) per
 // lane, PPL consecutive i (a packed pair when PPL = 2; each lane of a packed
 // add or FMA rounds like the scalar one).
-template <int PPL, int HALF> struct ProtoSum;
-template <int HALF> struct ProtoSum<2, HALF> {
-    float2 m0, m1, r0, r1, s0, s1, q;   // sum k_circ, R v, v (both halves); q = (sum R, sum ||k||)
-    __device__ __forceinline__ void clear() {
-        m0 = m1 = r0 = r1 = s0 = s1 = q = make_float2(0.f, 0.f);
+template <int PPL, int HALF> struct KeySum;     // sum k_circ of both halves, sum ||k||
+template <int HALF> struct KeySum<2, HALF> {
+    float2 m0, m1;
+    float ks;
+    __device__ __forceinline__ void clear() { m0 = m1 = make_float2(0.f, 0.f); ks = 0.f; }
+    __device__ __forceinline__ void add(const float *k, float kn) {
+        m0 = fadd2(m0, *reinterpret_cast<const float2 *>(k));
+        m1 = fadd2(m1, *reinterpret_cast<const float2 *>(k + HALF));
+        ks += kn;
     }
-    struct Tok {
-        float2 k0, k1, x0, x1, rk;
-        __device__ __forceinline__ void load(const float *k, const float *v, const float2 *r) {
-            k0 = *reinterpret_cast<const float2 *>(k);
-            k1 = *reinterpret_cast<const float2 *>(k + HALF);
-            x0 = *reinterpret_cast<const float2 *>(v);
-            x1 = *reinterpret_cast<const float2 *>(v + HALF);
-            rk = *r;
-        }
-    };
-    __device__ __forceinline__ void add(const Tok &t) {
-        const float2 rr = make_float2(t.rk.x, t.rk.x);
-        q = fadd2(q, t.rk);
-        m0 = fadd2(m0, t.k0);
-        m1 = fadd2(m1, t.k1);
-        r0 = ffma2(rr, t.x0, r0);
-        r1 = ffma2(rr, t.x1, r1);
-        s0 = fadd2(s0, t.x0);
-        s1 = fadd2(s1, t.x1);
-    }
-    __device__ __forceinline__ void get(int j, float &a, float &b, float &c, float &d, float &e, float &f) const {
-        a = j ? m0.y : m0.x; b = j ? m1.y : m1.x;
-        c = j ? r0.y : r0.x; d = j ? r1.y : r1.x;
-        e = j ? s0.y : s0.x; f = j ? s1.y : s1.x;
-    }
+    __device__ __forceinline__ float lo(int j) const { return j ? m0.y : m0.x; }
+    __device__ __forceinline__ float hi(int j) const { return j ? m1.y : m1.x; }
 };
-template <int HALF> struct ProtoSum<1, HALF> {
-    float m0, m1, r0, r1, s0, s1;
-    float2 q;
-    __device__ __forceinline__ void clear() {
-        m0 = m1 = r0 = r1 = s0 = s1 = 0.f;
-        q = make_float2(0.f, 0.f);
+template <int HALF> struct KeySum<1, HALF> {
+    float m0, m1, ks;
+    __device__ __forceinline__ void clear() { m0 = m1 = ks = 0.f; }
+    __device__ __forceinline__ void add(const float *k, float kn) {
+        m0 += k[0];
+        m1 += k[HALF];
+        ks += kn;
     }
-    struct Tok {
-        float k0, k1, x0, x1;
-        float2 rk;
-        __device__ __forceinline__ void load(const float *k, const float *v, const float2 *r) {
-            k0 = k[0]; k1 = k[HALF]; x0 = v[0]; x1 = v[HALF];
-            rk = *r;
-        }
-    };
-    __device__ __forceinline__ void add(const Tok &t) {
-        q = fadd2(q, t.rk);
-        m0 += t.k0;
-        m1 += t.k1;
-        r0 = fmaf(t.rk.x, t.x0, r0);
-        r1 = fmaf(t.rk.x, t.x1, r1);
-        s0 += t.x0;
-        s1 += t.x1;
-    }
-    __device__ __forceinline__ void get(int, float &a, float &b, float &c, float &d, float &e, float &f) const {
-        a = m0; b = m1; c = r0; d = r1; e = s0; f = s1;
-    }
+    __device__ __forceinline__ float lo(int) const { return m0; }
+    __device__ __forceinline__ float hi(int) const { return m1; }
 };
+template <int PPL, int HALF> struct ValueSum;   // sum R v and sum v of both halves, sum R
+template <int HALF> struct ValueSum<2, HALF> {
+    float2 r0, r1, s0, s1;
+    float rs;
+    __device__ __forceinline__ void clear() { r0 = r1 = s0 = s1 = make_float2(0.f, 0.f); rs = 0.f; }
+    __device__ __forceinline__ void add(const float *v, float r) {
+        const float2 x0 = *reinterpret_cast<const float2 *>(v), x1 = *reinterpret_cast<const float2 *>(v + HALF);
+        const float2 rr = make_float2(r, r);
+        r0 = ffma2(rr, x0, r0);
+        r1 = ffma2(rr, x1, r1);
+        s0 = fadd2(s0, x0);
+        s1 = fadd2(s1, x1);
+        rs += r;
+    }
+    __device__ __forceinline__ float rlo(int j) const { return j ? r0.y : r0.x; }
+    __device__ __forceinline__ float rhi(int j) const { return j ? r1.y : r1.x; }
+    __device__ __forceinline__ float slo(int j) const { return j ? s0.y : s0.x; }
+    __device__ __forceinline__ float shi(int j) const { return j ? s1.y : s1.x; }
+};
+template <int HALF> struct ValueSum<1, HALF> {
+    float r0, r1, s0, s1, rs;
+    __device__ __forceinline__ void clear() { r0 = r1 = s0 = s1 = rs = 0.f; }
+    __device__ __forceinline__ void add(const float *v, float r) {
+        r0 = fmaf(r, v[0], r0);
+        r1 = fmaf(r, v[HALF], r1);
+        s0 += v[0];
+        s1 += v[HALF];
+        rs += r;
+    }
+    __device__ __forceinline__ float rlo(int) const { return r0; }
+    __device__ __forceinline__ float rhi(int) const { return r1; }
+    __device__ __forceinline__ float slo(int) const { return s0; }
+    __device__ __forceinline__ float shi(int) const { return s1; }
+};
+
+// A node's decision: extraction at its p* (Eq. app_extract_split).
+__device__ __forceinline__ void set_extraction(BatchNode &B, int a, int b, float DL, float DR) {
+    const int ps = B.pstar;
+    int ne = 0;
+    if (ps > a) { B.ca[ne] = (short)a; B.cb[ne] = (short)ps; B.cD[ne] = ps - a >= 2 ? DL : 0.f; ne++; }
+    B.ca[ne] = (short)ps; B.cb[ne] = (short)(ps + 1); B.cD[ne] = 0.f; ne++;
+    if (ps + 1 < b) { B.ca[ne] = (short)(ps + 1); B.cb[ne] = (short)b; B.cD[ne] = b - ps - 1 >= 2 ? DR : 0.f; ne++; }
+    B.nchild = (int8_t)ne;
+}
 
 // Instances by slot length: up to kTinyUnit tokens three CTAs per SM, up to
 // kShortUnit two, longer slots one CTA of twice the threads.
@@ -348,7 +380,7 @@ struct Smem {
     static constexpr int NWARPS = NT / 32;
     static constexpr int NB = 16;            // nodes per batch
     static constexpr int MAXNODES = 2 * NMAX;
-    static constexpr int NROW = DIRS == 2 ? kNCA : kNCD;   // candidate rows held at a time
+    static constexpr int NROW = kNCR;        // candidate rows held at a time
     static constexpr int KTW = DH < 128 ? 128 : DH;        // a row also holds 32 float4 of sums
     static constexpr int MW = (MAXNODES + 31) / 32;
     static constexpr int KPAD = NMAX <= kShortUnit ? 8 : 0;
@@ -363,10 +395,10 @@ struct Smem {
     float2 RK[NMAX];                         // token value, ||k||
     unsigned long long kap[NMAX];            // order-preserving keys of the curvature
     BatchNode bn[NB];
-    Cand cand[kNCA];
+    Cand cand[NROW];
     NodeS nodes[MAXNODES];
     float Ff[NMAX];                          // floor score of an accepted floor position, -inf elsewhere
-    float candD[kNCA], candP[kNCA];          // per-candidate D and drop mass
+    float candD[NROW], candP[NROW];          // per-row D and drop mass
     unsigned lvl[2][MW];                     // nodes of the level (bit masks), of the next one
     unsigned op_base;                        // the batch's first Split op in the global list
     unsigned int wcnt[NWARPS][3];            // per-warp work counters
@@ -498,8 +530,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                         const float cx = u & 1 ? cs[u / 2].z : cs[u / 2].x, cy = u & 1 ? cs[u / 2].w : cs[u / 2].y;
                         ss0 = fmaf(x[u], x[u], ss0);
                         ss1 = fmaf(y[u], y[u], ss1);
-                        lo[u] = x[u] * cx + y[u] * cy;
-                        hi[u] = y[u] * cx - x[u] * cy;
+                        rotate_back(x[u], y[u], cx, cy, lo[u], hi[u]);
                     }
                     st8(&sm.kc[t][i], lo);
                     st8(&sm.kc[t][i + HALF], hi);
@@ -723,8 +754,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                 if (e < n * HALF) {
                     const int t = e / HALF, i = e - t * HALF;
                     const float x = sm.kc[t][i], y = sm.kc[t][i + HALF];
-                    sm.kc[t][i] = x * cs[q].x + y * cs[q].y;
-                    sm.kc[t][i + HALF] = y * cs[q].x - x * cs[q].y;
+                    rotate_back(x, y, cs[q].x, cs[q].y, sm.kc[t][i], sm.kc[t][i + HALF]);
                 }
             }
         }
@@ -781,146 +811,173 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
     }
     __syncthreads();
 
-    int upre = 0, usuf = 0;   // the batch's candidate entries per direction
     unsigned int w_scan = 0, w_eval = 0, w_len = 0;   // work counters (lane 0 of each warp)
 
-    // candidate rows of a direction: prefixes k, suffixes k - kNCD (after the
-    // prefixes' rows when the directions run side by side)
-    auto row_of = [](int k) { return DIRS == 2 ? k : (k >= kNCD ? k - kNCD : k); };
-
-    // Prototype (ktil, vtil, m_eff) of candidate k from its interval's sums.
+    // Prototype (ktil, vtil, m_eff) of one or two candidate rows: row r0, and r1
+    // (-1: none), either two prefixes of a node (ascending ends; one running
+    // sum gives both) or two suffixes (descending starts; one set of loads
+    // feeds both sums).  Every sum runs over its interval's tokens in
+    // ascending order.  The keys' and the values' sums are separate tasks, so
+    // that a lone node keeps several warps busy.
     constexpr int PPL = HALF / 32;   // rotation pairs per lane: (i, i + d/2), i = PPL lane + j
-    using PS = ProtoSum<PPL, HALF>;
     const int pi0 = lane * PPL;
-    auto finish_proto = [&](int k, int nJ, const float2 *rot, const PS &acc) {
-        const int row = row_of(k);
-        const float rs = acc.q.x, ks = acc.q.y;
-        const float ninv = 1.0f / (float)nJ;
-        const float beta = (float)A.base_frac * (rs * ninv);
-        const float winv = 1.0f / ((rs + (float)nJ * beta) + A.eps);
-        float mu2 = 0.f;
+    auto proto_keys = [&](int r0, int r1, auto SUF) {
+        constexpr bool suffix = decltype(SUF)::value;
+        // the 64-channel bf16 instances' prefixes fuse the other product (their bits since the first build)
+        constexpr bool SF = DH == 64 && std::is_same<Tin, __nv_bfloat16>::value && !SUB && !suffix;
+        using PS = KeySum<PPL, HALF>;
+        const int a0 = sm.cand[r0].a, b0 = sm.cand[r0].b;
+        const int a1 = r1 >= 0 ? sm.cand[r1].a : 0, b1 = r1 >= 0 ? sm.cand[r1].b : 0;
+        float2 rot0[PPL], rot1[PPL];   // loaded first, so that their latency overlaps the sums
+        const int p0 = round_half_even_mid(sa + a0, sa + b0), p1 = round_half_even_mid(sa + a1, sa + b1);
 #pragma unroll
         for (int j = 0; j < PPL; j++) {
-            float m0, m1, r0, r1, s0, s1;
-            acc.get(j, m0, m1, r0, r1, s0, s1);
-            const float a0 = m0 * ninv, a1 = m1 * ninv;
-            mu2 = fmaf(a0, a0, fmaf(a1, a1, mu2));
-            const float2 cs = rot[j];
-            sm.ktil[row][pi0 + j] = a0 * cs.x - a1 * cs.y;
-            sm.ktil[row][pi0 + j + HALF] = a0 * cs.y + a1 * cs.x;
-            sm.vtil[row][pi0 + j] = fmaf(beta, s0, r0) * winv;
-            sm.vtil[row][pi0 + j + HALF] = fmaf(beta, s1, r1) * winv;
+            rot0[j] = A.rope[(size_t)p0 * HALF + pi0 + j];
+            rot1[j] = r1 >= 0 ? A.rope[(size_t)p1 * HALF + pi0 + j] : make_float2(0.f, 0.f);
         }
-        mu2 = warp_sum(mu2);
-        if (lane == 0) {
-            const float coh = sqrtf(mu2) / (ks * ninv + A.eps);
-            const float me = (float)nJ * coh * coh;
-            sm.cand[k].meff = me < 1.0f ? 1.0f : (me > (float)nJ ? (float)nJ : me);
-        }
-    };
-    // Prototypes of the batch's candidates of one direction: a warp takes two
-    // adjacent candidates at a time (2 i, 2 i + 1).  Two prefixes of a node
-    // share their first tokens, so one running sum gives both; two suffixes
-    // share their last ones, so one set of loads feeds both sums.  Every sum
-    // runs over its interval's tokens in ascending order.
-    auto prototypes = [&](bool suffix) {
-        const int kb = suffix ? kNCD : 0, nk = suffix ? usuf : upre;
-        for (int i = 2 * dwarp; i < nk; i += 2 * (kNT / 32)) {
-            const int k0 = kb + i, k1 = k0 + 1;
-            int a0 = sm.cand[k0].a, b0 = sm.cand[k0].b;
-            int a1 = 0, b1 = 0;
-            if (i + 1 < nk) { a1 = sm.cand[k1].a; b1 = sm.cand[k1].b; }
-            float2 rot0[PPL], rot1[PPL];   // loaded first, so that their latency overlaps the sums
-            const int p0 = round_half_even_mid(sa + a0, sa + b0), p1 = round_half_even_mid(sa + a1, sa + b1);
+        auto put = [&](int row, int nJ, const float2 *rot, const PS &acc) {
+            const float ninv = 1.0f / (float)nJ;
+            float mu2 = 0.f;
 #pragma unroll
             for (int j = 0; j < PPL; j++) {
-                rot0[j] = b0 > a0 ? A.rope[(size_t)p0 * HALF + pi0 + j] : make_float2(0.f, 0.f);
-                rot1[j] = b1 > a1 ? A.rope[(size_t)p1 * HALF + pi0 + j] : make_float2(0.f, 0.f);
+                const float a0 = acc.lo(j) * ninv, a1 = acc.hi(j) * ninv;
+                mu2 = fmaf(a0, a0, fmaf(a1, a1, mu2));
+                const float2 cs = rot[j];
+                rotate_to<SF>(a0, a1, cs.x, cs.y, sm.ktil[row][pi0 + j], sm.ktil[row][pi0 + j + HALF]);
             }
-            PS s0, s1;
-            s0.clear();
-            typename PS::Tok tk;
-            if (!suffix) {
+            mu2 = warp_sum(mu2);
+            if (lane == 0) {
+                const float coh = sqrtf(mu2) / (acc.ks * ninv + A.eps);
+                const float me = (float)nJ * coh * coh;
+                sm.cand[row].meff = me < 1.0f ? 1.0f : (me > (float)nJ ? (float)nJ : me);
+            }
+        };
+        PS s0;
+        s0.clear();
+        if (!suffix) {
 #pragma unroll 4
-                for (int t = a0; t < b0; t++) { tk.load(&sm.kc[t][pi0], &sm.vv[t][pi0], &sm.RK[t]); s0.add(tk); }
-                if (b0 > a0) finish_proto(k0, b0 - a0, rot0, s0);
-                int t = b0;
-                if (!(b0 > a0 && a1 == a0)) { s0.clear(); t = a1; }   // another node's prefix
+            for (int t = a0; t < b0; t++) s0.add(&sm.kc[t][pi0], sm.RK[t].y);
+            put(r0, b0 - a0, rot0, s0);
+            if (r1 < 0) return;
 #pragma unroll 4
-                for (; t < b1; t++) { tk.load(&sm.kc[t][pi0], &sm.vv[t][pi0], &sm.RK[t]); s0.add(tk); }
-                if (b1 > a1) finish_proto(k1, b1 - a1, rot1, s0);
+            for (int t = b0; t < b1; t++) s0.add(&sm.kc[t][pi0], sm.RK[t].y);
+            put(r1, b1 - a1, rot1, s0);
+        } else {
+            PS s1;
+            s1.clear();
+            if (r1 >= 0) {   // the longer one's own tokens
+#pragma unroll 4
+                for (int t = a1; t < a0; t++) s1.add(&sm.kc[t][pi0], sm.RK[t].y);
+#pragma unroll 4
+                for (int t = a0; t < b0; t++) {
+                    s0.add(&sm.kc[t][pi0], sm.RK[t].y);
+                    s1.add(&sm.kc[t][pi0], sm.RK[t].y);
+                }
+                put(r1, b1 - a1, rot1, s1);
             } else {
-                s1.clear();
-                const bool both = b1 > a1 && b1 == b0 && a1 < a0 && b0 > a0;
-                if (b1 > a1) {   // the longer one's own tokens
-                    const int stop = both ? a0 : b1;
 #pragma unroll 4
-                    for (int t = a1; t < stop; t++) { tk.load(&sm.kc[t][pi0], &sm.vv[t][pi0], &sm.RK[t]); s1.add(tk); }
-                }
-                if (both) {
-#pragma unroll 2
-                    for (int t = a0; t < b0; t++) {
-                        tk.load(&sm.kc[t][pi0], &sm.vv[t][pi0], &sm.RK[t]);
-                        s0.add(tk);
-                        s1.add(tk);
-                    }
-                } else {
-#pragma unroll 4
-                    for (int t = a0; t < b0; t++) { tk.load(&sm.kc[t][pi0], &sm.vv[t][pi0], &sm.RK[t]); s0.add(tk); }
-                }
-                if (b0 > a0) finish_proto(k0, b0 - a0, rot0, s0);
-                if (b1 > a1) finish_proto(k1, b1 - a1, rot1, s1);
+                for (int t = a0; t < b0; t++) s0.add(&sm.kc[t][pi0], sm.RK[t].y);
             }
+            put(r0, b0 - a0, rot0, s0);
+        }
+    };
+    auto proto_values = [&](int r0, int r1, auto SUF) {
+        constexpr bool suffix = decltype(SUF)::value;
+        using PS = ValueSum<PPL, HALF>;
+        const int a0 = sm.cand[r0].a, b0 = sm.cand[r0].b;
+        const int a1 = r1 >= 0 ? sm.cand[r1].a : 0, b1 = r1 >= 0 ? sm.cand[r1].b : 0;
+        auto put = [&](int row, int nJ, const PS &acc) {
+            const float ninv = 1.0f / (float)nJ;
+            const float beta = (float)A.base_frac * (acc.rs * ninv);
+            const float winv = 1.0f / ((acc.rs + (float)nJ * beta) + A.eps);
+#pragma unroll
+            for (int j = 0; j < PPL; j++) {
+                sm.vtil[row][pi0 + j] = fmaf(beta, acc.slo(j), acc.rlo(j)) * winv;
+                sm.vtil[row][pi0 + j + HALF] = fmaf(beta, acc.shi(j), acc.rhi(j)) * winv;
+            }
+        };
+        PS s0;
+        s0.clear();
+        if (!suffix) {
+#pragma unroll 4
+            for (int t = a0; t < b0; t++) s0.add(&sm.vv[t][pi0], sm.RK[t].x);
+            put(r0, b0 - a0, s0);
+            if (r1 < 0) return;
+#pragma unroll 4
+            for (int t = b0; t < b1; t++) s0.add(&sm.vv[t][pi0], sm.RK[t].x);
+            put(r1, b1 - a1, s0);
+        } else {
+            PS s1;
+            s1.clear();
+            if (r1 >= 0) {
+#pragma unroll 4
+                for (int t = a1; t < a0; t++) s1.add(&sm.vv[t][pi0], sm.RK[t].x);
+#pragma unroll 2
+                for (int t = a0; t < b0; t++) {
+                    s0.add(&sm.vv[t][pi0], sm.RK[t].x);
+                    s1.add(&sm.vv[t][pi0], sm.RK[t].x);
+                }
+                put(r1, b1 - a1, s1);
+            } else {
+#pragma unroll 4
+                for (int t = a0; t < b0; t++) s0.add(&sm.vv[t][pi0], sm.RK[t].x);
+            }
+            put(r0, b0 - a0, s0);
+        }
+    };
+    // The prototypes of the rows [rb, re) of one direction (one node's), two
+    // at a time; `task` counts the tasks handed out, round robin over the warps.
+    auto prototypes = [&](int rb, int re, auto SUF, int &task) {
+        for (int r = rb; r < re; r += 2) {
+            const int r1 = r + 1 < re ? r + 1 : -1;
+            if (task++ % NWARPS == warp) proto_keys(r, r1, SUF);
+            if (task++ % NWARPS == warp) proto_values(r, r1, SUF);
         }
     };
     const float inv_sqrt_d = A.inv_sqrt_d, lamZ = A.lamZ, lamM = A.lamM, epsf = A.eps;
-    // zt = m_eff exp(q_u . ktil / sqrt d - m_u) of the direction's candidates,
-    // four at a time: 8 dot products per thread chunk, one reduce-scatter, and
-    // one exponential per (candidate, probe).
-    auto logits = [&](bool suffix) {
-        const int kb = suffix ? kNCD : 0, nk = suffix ? usuf : upre;
-        if (nk == 0) return;
-        const int rb = row_of(kb);
+    // zt = m_eff exp(q_u . ktil / sqrt d - m_u) of the rows [0, nr), four at a
+    // time: 8 dot products per thread chunk, one reduce-scatter, and one
+    // exponential per (row, probe).  Starts with the barrier that the
+    // prototypes end on, after the queries' loads.
+    auto logits = [&](int nr) {
         float2 qa0[CH / 2], qa1[CH / 2];
         load_q(qa0, pp);
         load_q(qa1, pp + kNPP);
-        for (int i = 0; i < nk; i += 4) {
-            float v[8];   // [candidate i + (index & 3)][probe pp + 32 (index >> 2)]
+        __syncthreads();
+        for (int i = DIRS == 2 ? 4 * (warp / (kNT / 32)) : 0; i < nr; i += 4 * DIRS) {
+            float v[8];   // [row i + (index & 3)][probe pp + 32 (index >> 2)]
 #pragma unroll
             for (int j = 0; j < 4; j++) {
-                const int row = rb + min(i + j, nk - 1);
+                const int row = min(i + j, nr - 1);
                 float2 xa = make_float2(0.f, 0.f), xb = make_float2(0.f, 0.f);
 #pragma unroll
                 for (int gi = 0; gi < NG; gi++) {
                     const float4 x = *reinterpret_cast<const float4 *>(&sm.ktil[row][4 * c + 32 * gi]);
-                    const float2 ka = make_float2(x.x, x.y), kb2 = make_float2(x.z, x.w);
+                    const float2 ka = make_float2(x.x, x.y), kb = make_float2(x.z, x.w);
                     xa = ffma2(qa0[2 * gi], ka, xa);
-                    xa = ffma2(qa0[2 * gi + 1], kb2, xa);
+                    xa = ffma2(qa0[2 * gi + 1], kb, xa);
                     xb = ffma2(qa1[2 * gi], ka, xb);
-                    xb = ffma2(qa1[2 * gi + 1], kb2, xb);
+                    xb = ffma2(qa1[2 * gi + 1], kb, xb);
                 }
                 v[j] = xa.x + xa.y;
                 v[4 + j] = xb.x + xb.y;
             }
             const float x = reduce_scatter8(v, lane);
-            const int ii = i + (c & 3);
-            if (ii < nk) {
-                const float z = sm.cand[kb + ii].meff * expf(x * inv_sqrt_d - mu_log);
-                reinterpret_cast<float *>(&sm.zt[rb + ii][pp])[c >> 2] = z;
-            }
+            const int row = i + (c & 3);
+            if (row < nr)
+                reinterpret_cast<float *>(&sm.zt[row][pp])[c >> 2] =
+                    sm.cand[row].meff * expf(x * inv_sqrt_d - mu_log);
         }
     };
     // Probe scan of one node in one direction (SUF: suffixes, descending):
-    // running sums Z_u, M_u over the tokens; at each candidate's far end the
-    // thread's parts of ||M - zt vtil||^2 and ||M||^2, reduced two candidates
-    // at a time; ||M - zt vtil||^2 / ||M||^2 and Z go into the candidates' (no
-    // longer needed) key prototype rows.
-    auto scan = [&](const BatchNode &B, auto SUF) {
+    // running sums Z_u, M_u over the tokens from position t0; at the far end of
+    // each of the rows [k, ke) the thread's parts of ||M - zt vtil||^2 and
+    // ||M||^2 are reduced, and their ratio and Z go into the row's (no longer
+    // needed) key prototype.
+    auto scan = [&](int t0, int k, int ke, auto SUF) {
         constexpr bool suffix = decltype(SUF)::value;
-        int k = suffix ? B.suf_b : B.pre_b;
-        const int ke = suffix ? B.suf_e : B.pre_e;
         if (k >= ke) return;
-        int t = suffix ? sm.nodes[B.node].b - 1 : sm.nodes[B.node].a;   // next token to add
+        int t = t0;   // next token to add
         float2 M0[CH / 2], M1[CH / 2];
         float2 Z = make_float2(0.f, 0.f);
 #pragma unroll
@@ -939,23 +996,22 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                 M1[2 * gi + 1] = ffma2(e1, vb, M1[2 * gi + 1]);
             }
         };
-        auto partial = [&](int k, float *v) {
-            const int row = row_of(k);
+        for (; k < ke; k++) {
             if (suffix) {
-                const int stop = sm.cand[k].a;   // candidates in descending start, all >= a
-#pragma unroll 1
+                const int stop = sm.cand[k].a;   // rows in descending start
+#pragma unroll 2
                 for (; t >= stop; t--) add(t);
             } else {
-                const int stop = sm.cand[k].b;   // candidates in ascending end, all <= b
-#pragma unroll 1
+                const int stop = sm.cand[k].b;   // rows in ascending end
+#pragma unroll 2
                 for (; t < stop; t++) add(t);
             }
-            const float2 z = sm.zt[row][pp];
+            const float2 z = sm.zt[k][pp];
             const float2 nz0 = make_float2(-z.x, -z.x), nz1 = make_float2(-z.y, -z.y);
             float2 r0 = make_float2(0.f, 0.f), r1 = r0, m0 = r0, m1 = r0;
 #pragma unroll
             for (int gi = 0; gi < NG; gi++) {
-                const float4 x = *reinterpret_cast<const float4 *>(&sm.vtil[row][4 * c + 32 * gi]);
+                const float4 x = *reinterpret_cast<const float4 *>(&sm.vtil[k][4 * c + 32 * gi]);
                 const float2 va = make_float2(x.x, x.y), vb = make_float2(x.z, x.w);
 #pragma unroll
                 for (int h = 0; h < 2; h++) {
@@ -968,68 +1024,152 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                     m1 = ffma2(M1[q], M1[q], m1);
                 }
             }
-            v[0] = r0.x + r0.y;   // index bits: probe pp + 32 (0), ||M||^2 (1), candidate (2)
-            v[1] = r1.x + r1.y;
-            v[2] = m0.x + m0.y;
-            v[3] = m1.x + m1.y;
-        };
-        for (; k < ke; k += 2) {
-            float v[8];
-            partial(k, v);
-            float Zk = (c & 1) ? Z.y : Z.x;   // of the candidate and probe that the lane ends up with
-            if (k + 1 < ke) {
-                partial(k + 1, v + 4);
-                if (c >> 2) Zk = (c & 1) ? Z.y : Z.x;
-            } else {
-                v[4] = v[5] = v[6] = v[7] = 0.f;
-            }
-            // lane c: probe pp + 32 (c & 1), ||M||^2 if c & 2 else the residual,
-            // candidate k + (c >> 2); the residual's lane divides, its partner
-            // keeps Z.  Fast division: at most 2 ulp, far below the distortion
-            // tolerance.
-            const float x = reduce_scatter8(v, lane);
+            // lane c: probe pp + 32 (c & 1), ||M||^2 if c & 2 else the residual;
+            // the residual's lane divides, its partner keeps Z.  Fast division:
+            // at most 2 ulp, far below the distortion tolerance.
+            const float x = reduce_scatter4(r0.x + r0.y, r1.x + r1.y, m0.x + m0.y, m1.x + m1.y, lane);
             const float y = __shfl_xor_sync(0xffffffffu, x, 2 * kPPW);
-            const int kk = k + (c >> 2);
-            if (kk < ke) sm.ktil[row_of(kk)][4 * pp + (c & 3)] = (c & 2) ? Zk : __fdividef(x, y + epsf);
+            if (c < 4) sm.ktil[k][4 * pp + c] = (c & 2) ? ((c & 1) ? Z.y : Z.x) : __fdividef(x, y + epsf);
         }
     };
-    // D_u (Eq. app_probe_distortion) of the direction's candidates, weighted by
-    // the probe's attention mass, and their means over the W probes: a warp per
-    // candidate, lane p the probes p and p + 32.  The sums run over groups of
-    // four lanes, then over the groups in order.  Probes past W have E = 0 and
-    // invZ = 0, so they add nothing.  Fast division: at most 2 ulp, far below
-    // the distortion tolerance.  Rows belong to the same warps as in
-    // prototypes(), which may follow without a barrier.
-    auto finish = [&](bool suffix) {
-        const int kb = suffix ? kNCD : 0, nk = suffix ? usuf : upre;
+    // D_u (Eq. app_probe_distortion) of the rows [0, nr), weighted by the
+    // probe's attention mass, and their means over the W probes: a warp per
+    // row, lane p the probes p and p + 32.  The sums run over groups of four
+    // lanes, then over the groups in order.  Probes past W have E = 0 and
+    // invZ = 0, so they add nothing.
+    auto finish = [&](int nr) {
         const float invW = 1.0f / A.W;
-        for (int i = dwarp; i < (nk + 1) / 2; i += kNT / 32) {
+        for (int k = warp; k < nr; k += NWARPS) {
+            if (sm.cand[k].b <= sm.cand[k].a) continue;
+            const float4 q = *reinterpret_cast<const float4 *>(&sm.ktil[k][4 * lane]);   // ratios, Z
+            const float2 z = sm.zt[k][lane];
+            const float Z0 = q.z, Z1 = q.w;
+            const float dz0 = Z0 - z.x, dz1 = Z1 - z.y;
+            const float D0 = fmaf(lamZ, __fdividef(dz0 * dz0, fmaf(Z0, Z0, epsf)), lamM * q.x);
+            const float D1 = fmaf(lamZ, __fdividef(dz1 * dz1, fmaf(Z1, Z1, epsf)), lamM * q.y);
+            const float p0 = Z0 * invZ0, p1 = Z1 * invZ1;
+            float pd = fmaf(p0, D0, p1 * D1), pw = p0 + p1;
 #pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const int k = kb + 2 * i + h;
-                if (2 * i + h >= nk || sm.cand[k].b <= sm.cand[k].a) continue;
-                const int row = row_of(k);
-                const float4 q = *reinterpret_cast<const float4 *>(&sm.ktil[row][4 * lane]);   // ratios, Z
-                const float2 z = sm.zt[row][lane];
-                const float Z0 = q.z, Z1 = q.w;
-                const float dz0 = Z0 - z.x, dz1 = Z1 - z.y;
-                const float D0 = lamZ * __fdividef(dz0 * dz0, fmaf(Z0, Z0, epsf)) + lamM * q.x;
-                const float D1 = lamZ * __fdividef(dz1 * dz1, fmaf(Z1, Z1, epsf)) + lamM * q.y;
-                const float p0 = Z0 * invZ0, p1 = Z1 * invZ1;
-                float pd = fmaf(p0, D0, p1 * D1), pw = p0 + p1;
+            for (int o = 1; o < kPPW; o <<= 1) {
+                pd += __shfl_xor_sync(0xffffffffu, pd, o);
+                pw += __shfl_xor_sync(0xffffffffu, pw, o);
+            }
+            const float x = (lane & 1) ? pw : pd;   // even lanes sum D, odd lanes the mass
+            float d = 0.f;
 #pragma unroll
-                for (int o = 1; o < kPPW; o <<= 1) {
-                    pd += __shfl_xor_sync(0xffffffffu, pd, o);
-                    pw += __shfl_xor_sync(0xffffffffu, pw, o);
+            for (int w = 0; w < 32 / kPPW; w++) d += __shfl_sync(0xffffffffu, x, kPPW * w + (lane & 1));
+            if (lane < 2) (lane ? sm.candP : sm.candD)[k] = d * invW;
+        }
+    };
+
+    // The candidates of a node that the first ones could not rule out: both
+    // sides of the cuts in B.more and of the extraction (B.ext).  The prefixes
+    // first; their D tightens the cuts' bounds before the suffixes (together
+    // when all of them fit the rows).  Warp 0 lays the rows out and decides;
+    // the same decision as over all cuts, ties to the smallest xi.
+    auto evaluate_rest = [&](BatchNode &B) {
+        NodeS &nd = sm.nodes[B.node];
+        const unsigned FULL = 0xffffffffu;
+        const int a = nd.a, b = nd.b, ps = B.pstar;
+        const float DI = nd.D;
+        const bool ext = B.ext;
+        const bool el = ext && ps - a >= 2, er = ext && b - (ps + 1) >= 2;
+        const int k1 = B.k1, ncut = B.ncut;
+        const float best1 = ((DI - B.cD[0]) - B.cD[1]) + A.lam_kappa * B.kh[k1];
+        const float DL1 = B.cD[0], DR1 = B.cD[1];
+        const int xi = lane < ncut ? B.cut[lane] : 0;
+        const float rew = lane < ncut ? B.kh[lane] : 0.f;
+        bool need = (B.more >> lane) & 1u;
+        // every warp forms the same lists; the rows are written by warp 0
+        const bool pv = need && xi - a >= 2;
+        const unsigned lt = (1u << lane) - 1u, gt = ~((2u << lane) - 1u);
+        const unsigned pm = __ballot_sync(FULL, pv);
+        const int npre = __popc(pm) + (el ? 1 : 0);
+        const int prow = __popc(pm & lt) + (el && ps < xi ? 1 : 0);
+        const int el_row = __popc(__ballot_sync(FULL, pv && xi <= ps));
+        bool sv = need && b - xi >= 2;
+        const bool both = npre + __popc(__ballot_sync(FULL, sv)) + (er ? 1 : 0) <= S::NROW;
+        float dl = 0.f, dr = 0.f, eDL = 0.f, eDR = 0.f;
+        for (int pass = both ? 1 : 0; pass < 2; pass++) {
+            const int np = both || pass == 0 ? npre : 0;
+            int ns = 0, srow = 0, er_row = 0;
+            if (pass == 1) {
+                if (!both && A.prune) need = need && !((DI - dl) + A.lam_kappa * rew < best1);
+                sv = need && b - xi >= 2;
+                const unsigned sm_ = __ballot_sync(FULL, sv);
+                ns = __popc(sm_) + (er ? 1 : 0);
+                srow = np + __popc(sm_ & gt) + (er && ps + 1 > xi ? 1 : 0);
+                er_row = np + __popc(__ballot_sync(FULL, sv && xi >= ps + 1));
+            }
+            if (warp == 0) {
+                if (np && pv) sm.cand[prow] = {(short)a, (short)xi, 0.f};
+                if (ns && sv) sm.cand[srow] = {(short)xi, (short)b, 0.f};
+                if (lane == 0) {
+                    if (np && el) sm.cand[el_row] = {(short)a, (short)ps, 0.f};
+                    if (ns && er) sm.cand[er_row] = {(short)(ps + 1), (short)b, 0.f};
                 }
-                const float x = (lane & 1) ? pw : pd;   // even lanes sum D, odd lanes the mass
-                float d = 0.f;
-#pragma unroll
-                for (int w = 0; w < 32 / kPPW; w++) d += __shfl_sync(0xffffffffu, x, kPPW * w + (lane & 1));
-                if (lane < 2) (lane ? sm.candP : sm.candD)[k] = d * invW;
+                int len = (np && pv ? xi - a : 0) + (ns && sv ? b - xi : 0);
+                int pe = np && pv ? xi : a, ss = ns && sv ? xi : b;
+                len = __reduce_add_sync(FULL, len);
+                pe = __reduce_max_sync(FULL, pe);
+                ss = __reduce_min_sync(FULL, ss);
+                if (np && el) { pe = max(pe, ps); len += ps - a; }
+                if (ns && er) { ss = min(ss, ps + 1); len += b - ps - 1; }
+                w_scan += (pe - a) + (b - ss);
+                w_eval += np + ns;
+                w_len += len;
+            }
+            if (np + ns == 0) continue;   // the same in every warp
+            __syncthreads();
+            int task = 0;
+            prototypes(0, np, std::false_type(), task);
+            prototypes(np, np + ns, std::true_type(), task);
+            logits(np + ns);
+            __syncthreads();
+            if (DIRS == 1 || warp < kNT / 32) scan(a, 0, np, std::false_type());
+            if (DIRS == 1 || warp >= kNT / 32) scan(b - 1, np, np + ns, std::true_type());
+            __syncthreads();
+            finish(np + ns);
+            __syncthreads();
+            if (np) {
+                if (pv) dl = sm.candD[prow];
+                if (el) eDL = sm.candD[el_row];
+            }
+            if (ns) {
+                if (sv) dr = sm.candD[srow];
+                if (er) eDR = sm.candD[er_row];
             }
         }
-        __syncwarp();   // the rows are free
+        // a cut ruled out by its D_L keeps G_bin's bound, which is below best1
+        float val = -INFINITY;
+        if (lane == k1) { dl = DL1; dr = DR1; val = best1; }
+        else if (need) val = ((DI - dl) - dr) + A.lam_kappa * rew;
+        const unsigned key = lane < ncut ? fkey_ordered(val) : 0u;
+        const unsigned kmx = __reduce_max_sync(FULL, key);   // every lane takes part
+        const unsigned top = __ballot_sync(FULL, lane < ncut && key == kmx);
+        int bq = __ffs(top) - 1;
+        const float best = __shfl_sync(FULL, val, bq);
+        if (!(best > -INFINITY)) bq = 0;   // only reachable with non-finite gains
+        const float bL = __shfl_sync(FULL, dl, bq), bR = __shfl_sync(FULL, dr, bq);
+        __syncthreads();   // every warp has read the node's entry
+        if (warp == 0 && lane == 0) {
+            bool take = false;
+            if (ext) {   // rho_ext = G_ext / (|children| - 1)
+                const int ne = 1 + (ps > a) + (ps + 1 < b);
+                float gext = DI;
+                if (ps > a) gext -= eDL;
+                if (ps + 1 < b) gext -= eDR;
+                take = (ne == 3 ? 0.5f * gext : gext) > best;
+            }
+            if (take) {
+                set_extraction(B, a, b, eDL, eDR);
+            } else {
+                B.nchild = 2;
+                B.ca[0] = (short)a; B.cb[0] = B.cut[bq]; B.cD[0] = bL;
+                B.ca[1] = B.cut[bq]; B.cb[1] = (short)b; B.cD[1] = bR;
+            }
+        }
+        __syncthreads();
     };
 
     int cur = 0;
@@ -1044,8 +1184,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
         for (;;) {
             // ---- batch: the level's next nodes in creation order.  Every warp
             // walks them; phase A (cut candidates) runs on a node's own warp.
-            int nb = 0, nops = 0;
-            upre = usuf = 0;
+            int nb = 0, nops = 0, nrow = 0;
             while (nb < S::NB) {
                 while (!lbits && lw < S::MW - 1) lbits = sm.lvl[cur][++lw];
                 if (!lbits) break;
@@ -1053,13 +1192,11 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                 const int a = sm.nodes[v].a, b = sm.nodes[v].b, nv = b - a;
                 const bool root = v == 0 && fresh;
                 const bool ronly = root && A.root_only;   // only the node's own distortion
-                const int nc = (nv >= 3 && !ronly) ? min(A.k_cand + 1, nv - 1) + 1 : 0;
-                const int bp = nc + (root ? 1 : 0), bs = nc;
-                if (upre + bp > kNCD || usuf + bs > kNCS) break;
+                const int rows = (nv >= 3 && !ronly ? 2 : 0) + (root ? 1 : 0);
+                if (nrow + rows > S::NROW) break;
                 lbits &= lbits - 1;
-                const int pre_b = upre, suf_b = kNCD + usuf;
-                upre += bp;
-                usuf += bs;
+                const int row0 = nrow;
+                nrow += rows;
                 const int op = nv >= 2 && !ronly ? nops++ : -1;
                 const int bi = nb++;
                 if (bi % NWARPS != warp) continue;
@@ -1114,13 +1251,8 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                     }
                     if (fb > -INFINITY) { pb = fpos; forced = 1; }
                 }
-                // Candidate lists, lane-parallel (ranks from ballots): cuts xi in
-                // ascending order; prefixes [a, xi) (xi - a >= 2) and the
-                // extraction's left side [a, p*) in ascending end, then the whole
-                // node (fresh roots); suffixes [xi, b) (b - xi >= 2) and the right
-                // side [p*+1, b) in descending start.  A side equal to a cut's
-                // interval shares its candidate.
-                const unsigned FULL = 0xffffffffu;
+                // cuts xi in ascending order, their normalised curvature, and the
+                // one of largest reward
                 const bool cands = nv >= 3 && !ronly;
                 const int maxc = cands ? min(A.k_cand + 1, nv - 1) : 0;
                 int ncut = 0;
@@ -1133,100 +1265,77 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                 }
                 ncut = min(ncut, maxc);
                 __syncwarp();
-                const bool hq = lane < ncut;
-                const int xi = hq ? B.cut[lane] : 0;
-                const unsigned lt = (1u << lane) - 1u, gt = ~((2u << lane) - 1u);
-                // prefixes
-                const bool pv = hq && xi - a >= 2;
-                const unsigned pm = __ballot_sync(FULL, pv);
-                const unsigned pbm = __ballot_sync(FULL, hq && xi == pb);
-                const bool el_cand = cands && pb - a >= 2;
-                const bool el_sep = el_cand && pbm == 0u;
-                const int pidx = pv ? pre_b + __popc(pm & lt) + (el_sep && pb < xi ? 1 : 0) : -1;
-                const int eL_sep = pre_b + __popc(__ballot_sync(FULL, pv && xi < pb));
-                const int eL_cut = __shfl_sync(FULL, pidx, pbm ? __ffs(pbm) - 1 : 0);
-                if (hq) B.pidx[lane] = (int8_t)pidx;
-                if (pv) sm.cand[pidx] = {(short)a, (short)xi, 0.f};
-                // suffixes
-                const int er = pb + 1;
-                const bool sv = hq && b - xi >= 2;
-                const unsigned smk = __ballot_sync(FULL, sv);
-                const unsigned erm = __ballot_sync(FULL, hq && xi == er);
-                const bool er_cand = cands && b - er >= 2;
-                const bool er_sep = er_cand && erm == 0u;
-                const int sidx = sv ? suf_b + __popc(smk & gt) + (er_sep && er > xi ? 1 : 0) : -1;
-                const int eR_sep = suf_b + __popc(__ballot_sync(FULL, sv && xi > er));
-                const int eR_cut = __shfl_sync(FULL, sidx, erm ? __ffs(erm) - 1 : 0);
-                if (hq) B.sidx[lane] = (int8_t)sidx;
-                if (sv) sm.cand[sidx] = {(short)xi, (short)b, 0.f};
-                // work counters: tokens swept, candidates evaluated, their lengths
-                int len = (pv ? xi - a : 0) + (sv ? b - xi : 0);
-                int pe = pv ? xi : a, ss = sv ? xi : b;
-                len = __reduce_add_sync(FULL, len);
-                pe = __reduce_max_sync(FULL, pe);
-                ss = __reduce_min_sync(FULL, ss);
+                float rew = 0.f;
+                if (lane < ncut) {
+                    // the difference is taken in fp64 (the curvatures may be close),
+                    // the rest in fp32
+                    const double kmn = okey_inv(B.klo), kmx = okey_inv(B.khi);
+                    const float krange = kmx > kmn ? 1.0f / (float)(kmx - kmn) : 0.f;
+                    const float kh = (float)(okey_inv(sm.kap[B.cut[lane] - 1]) - kmn) * krange;
+                    B.kh[lane] = kh;
+                    rew = A.lam_kappa * kh;
+                }
+                const unsigned rkey = lane < ncut ? fkey_ordered(rew) : 0u;
+                const int k1 = __ffs(__ballot_sync(0xffffffffu, rkey == __reduce_max_sync(0xffffffffu, rkey))) - 1;
                 if (lane == 0) {
+                    // the intervals evaluated first: both sides of the cut of largest
+                    // reward, or of a forced extraction; a fresh root's own
+                    const int lo = !cands ? a : (forced ? pb : B.cut[k1]), hi = !cands ? b : (forced ? pb + 1 : B.cut[k1]);
+                    const bool pv = lo - a >= 2, sv = b - hi >= 2;
+                    int k = row0;
+                    B.pre_b = (int8_t)k;
+                    B.rl = pv ? (int8_t)k : (int8_t)-1;
+                    if (pv) sm.cand[k++] = {(short)a, (short)lo, 0.f};
+                    B.whole = root ? (int8_t)k : (int8_t)-1;
+                    if (root) sm.cand[k++] = {(short)a, (short)b, 0.f};
+                    B.pre_e = B.suf_b = (int8_t)k;
+                    B.rr = sv ? (int8_t)k : (int8_t)-1;
+                    if (sv) sm.cand[k++] = {(short)hi, (short)b, 0.f};
+                    B.suf_e = (int8_t)k;
+                    for (; k < row0 + rows; k++) sm.cand[k].a = sm.cand[k].b = 0;   // reserved, not used
                     B.node = (short)v;
                     B.op = (short)op;
-                    B.pre_b = (int8_t)pre_b;
-                    B.suf_b = (int8_t)suf_b;
                     B.pstar = (short)pb;
                     B.forced = (int8_t)forced;
                     B.ncut = (int8_t)ncut;
-                    B.eL = (int8_t)(el_sep ? eL_sep : (el_cand ? eL_cut : -1));
-                    if (el_sep) sm.cand[eL_sep] = {(short)a, (short)pb, 0.f};
-                    int k = pre_b + __popc(pm) + (el_sep ? 1 : 0);
-                    B.whole = -1;
-                    if (root) { sm.cand[k] = {(short)a, (short)b, 0.f}; B.whole = (int8_t)k++; }
-                    B.pre_e = (int8_t)k;
-                    B.eR = (int8_t)(er_sep ? eR_sep : (er_cand ? eR_cut : -1));
-                    if (er_sep) sm.cand[eR_sep] = {(short)er, (short)b, 0.f};
-                    B.suf_e = (int8_t)(suf_b + __popc(smk) + (er_sep ? 1 : 0));
-                    for (int q = B.pre_e; q < pre_b + bp; q++) sm.cand[q].a = sm.cand[q].b = 0;
-                    for (int q = B.suf_e; q < suf_b + bs; q++) sm.cand[q].a = sm.cand[q].b = 0;
-                    if (el_sep) { pe = max(pe, pb); len += pb - a; }
-                    if (er_sep) { ss = min(ss, er); len += b - er; }
-                    if (root) { pe = b; len += b - a; }
-                    w_scan += (pe - a) + (b - ss);
-                    w_eval += (B.pre_e - pre_b) + (B.suf_e - suf_b);
-                    w_len += len;
+                    B.k1 = (int8_t)k1;
+                    // work counters: tokens swept, candidates evaluated, their lengths
+                    w_scan += (root ? nv : (pv ? lo - a : 0)) + (sv ? b - hi : 0);
+                    w_eval += B.suf_e - B.pre_b;
+                    w_len += (pv ? lo - a : 0) + (sv ? b - hi : 0) + (root ? nv : 0);
                 }
             }
             // the ops' places in the global list, fetched while the batch is evaluated
             if (nops > 0 && tid == NT - 1) sm.op_base = atomicAdd(A.n_ops, (unsigned)nops);
             if (nb == 0) break;
             __syncthreads();
-            // ---- phases B/C: prefixes and suffixes, side by side or in turn ------
-            if constexpr (DIRS == 2) {
-                const bool suf = warp >= kNT / 32;
-                prototypes(suf);
-                __syncthreads();
-                logits(suf);
-                __syncthreads();
-                for (int bi = 0; bi < nb; bi++) {
-                    if (suf) scan(sm.bn[bi], std::true_type());
-                    else scan(sm.bn[bi], std::false_type());
-                }
-                __syncthreads();
-                finish(suf);
-            } else {
-                prototypes(false);
-                __syncthreads();
-                logits(false);
-                __syncthreads();
-                for (int bi = 0; bi < nb; bi++) scan(sm.bn[bi], std::false_type());
-                __syncthreads();
-                finish(false);
-                prototypes(true);
-                __syncthreads();
-                logits(true);
-                __syncthreads();
-                for (int bi = 0; bi < nb; bi++) scan(sm.bn[bi], std::true_type());
-                __syncthreads();
-                finish(true);
+            // ---- phases B/C: prototypes, logits, scans in both directions, sums --
+            int task = 0;
+            for (int bi = 0; bi < nb; bi++) {
+                prototypes(sm.bn[bi].pre_b, sm.bn[bi].pre_e, std::false_type(), task);
+                prototypes(sm.bn[bi].suf_b, sm.bn[bi].suf_e, std::true_type(), task);
+            }
+            logits(nrow);   // after a barrier
+            __syncthreads();
+            for (int bi = 0; bi < nb; bi++) {
+                const BatchNode &B = sm.bn[bi];
+                const NodeS &nd = sm.nodes[B.node];
+                if (DIRS == 1 || warp < kNT / 32) scan(nd.a, B.pre_b, B.pre_e, std::false_type());
+                if (DIRS == 1 || warp >= kNT / 32) scan(nd.b - 1, B.suf_b, B.suf_e, std::true_type());
             }
             __syncthreads();
-            // ---- phase D1: candidate sums and decisions (warp per node) -------------
+            finish(nrow);
+            __syncthreads();
+            // ---- phase D1: decisions (warp per node) ---------------------------------
+            // G_bin of a cut is ((D - D_L) - D_R) + lambda_kappa kh, and D_L, D_R >= 0:
+            // D + lambda_kappa kh bounds it from above, in the rounded arithmetic too
+            // (every operation is monotone).  A cut whose bound is below G_bin of the
+            // cut already evaluated cannot be the best one, and its intervals are never
+            // evaluated; neither are the extraction's sides when that G_bin reaches D,
+            // which bounds rho_ext.  The other cuts are evaluated below, one node at a
+            // time.  D of a node is at most its attention mass, so on long contexts the
+            // curvature's reward decides nearly every cut.
+            bool open = false;   // the warp's nodes need more candidates
             for (int bi = warp; bi < nb; bi += NWARPS) {
                 BatchNode &B = sm.bn[bi];
                 NodeS &nd = sm.nodes[B.node];
@@ -1259,60 +1368,30 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                     continue;
                 }
                 const float DI = nd.D;
-                // binary cut: lane q evaluates cut q; max G_bin, ties -> smallest xi
-                float best = -INFINITY;
-                int bq = 0x7fffffff;
-                if (lane < B.ncut) {
-                    const int xi = B.cut[lane];
-                    const float DL = B.pidx[lane] >= 0 ? sm.candD[B.pidx[lane]] : 0.f;
-                    const float DR = B.sidx[lane] >= 0 ? sm.candD[B.sidx[lane]] : 0.f;
-                    // normalised curvature: the difference is taken in fp64 (the
-                    // curvatures may be close), the rest in fp32
-                    const double kmn = okey_inv(B.klo), kmx = okey_inv(B.khi);
-                    const float krange = kmx > kmn ? 1.0f / (float)(kmx - kmn) : 0.f;
-                    const float kh = (float)(okey_inv(sm.kap[xi - 1]) - kmn) * krange;
-                    best = ((DI - DL) - DR) + A.lam_kappa * kh;
-                    bq = lane;
+                const float DL = B.rl >= 0 ? sm.candD[B.rl] : 0.f, DR = B.rr >= 0 ? sm.candD[B.rr] : 0.f;
+                if (B.forced) {
+                    if (lane == 0) set_extraction(B, a, b, DL, DR);
+                    continue;
                 }
-                {
-                    const unsigned key = lane < B.ncut ? fkey_ordered(best) : 0u;
-                    const unsigned top = __ballot_sync(0xffffffffu, key == __reduce_max_sync(0xffffffffu, key) && lane < B.ncut);
-                    bq = top ? __ffs(top) - 1 : 0x7fffffff;
-                    best = __shfl_sync(0xffffffffu, best, bq & 31);
+                const int k1 = B.k1;
+                const float best = ((DI - DL) - DR) + A.lam_kappa * B.kh[k1];
+                bool need = lane < B.ncut && lane != k1;
+                if (need && A.prune) need = !(DI + A.lam_kappa * B.kh[lane] < best);
+                const unsigned more = __ballot_sync(0xffffffffu, need);
+                const bool ext = !(A.prune && best >= DI);
+                if (lane == 0) {
+                    B.ca[0] = (short)a; B.cb[0] = B.cut[k1]; B.cD[0] = DL;
+                    B.ca[1] = B.cut[k1]; B.cb[1] = (short)b; B.cD[1] = DR;
+                    B.nchild = more || ext ? -2 : 2;
+                    B.more = more;
+                    B.ext = ext;
                 }
-                if (lane) continue;
-                int bxi = -1;
-                float bL = 0.f, bR = 0.f;
-                if (bq < B.ncut && best > -INFINITY) {
-                    bxi = B.cut[bq];
-                    bL = B.pidx[bq] >= 0 ? sm.candD[B.pidx[bq]] : 0.f;
-                    bR = B.sidx[bq] >= 0 ? sm.candD[B.sidx[bq]] : 0.f;
-                }
-                // extraction at p*
-                const int ps = B.pstar;
-                int ea[3], eb[3], ne = 0;
-                float eD[3];
-                if (ps > a) { ea[ne] = a; eb[ne] = ps; eD[ne] = ps - a >= 2 ? sm.candD[B.eL] : 0.f; ne++; }
-                ea[ne] = ps; eb[ne] = ps + 1; eD[ne] = 0.f; ne++;
-                if (ps + 1 < b) { ea[ne] = ps + 1; eb[ne] = b; eD[ne] = b - ps - 1 >= 2 ? sm.candD[B.eR] : 0.f; ne++; }
-                float gext = DI;
-                for (int q = 0; q < ne; q++) gext -= eD[q];
-                if (bxi < 0) {   // only reachable with non-finite gains
-                    bxi = B.cut[0];
-                    bL = B.pidx[0] >= 0 ? sm.candD[B.pidx[0]] : 0.f;
-                    bR = B.sidx[0] >= 0 ? sm.candD[B.sidx[0]] : 0.f;
-                }
-                const float rho_ext = ne == 3 ? 0.5f * gext : gext;   // G_ext / (|children| - 1), exact
-                if (B.forced || rho_ext > best) {
-                    B.nchild = (int8_t)ne;
-                    for (int q = 0; q < ne; q++) { B.ca[q] = (short)ea[q]; B.cb[q] = (short)eb[q]; B.cD[q] = eD[q]; }
-                } else {
-                    B.nchild = 2;
-                    B.ca[0] = (short)a; B.cb[0] = (short)bxi; B.cD[0] = bL;
-                    B.ca[1] = (short)bxi; B.cb[1] = (short)b; B.cD[1] = bR;
-                }
+                open |= more || ext;
             }
-            __syncthreads();
+            if (__syncthreads_or(open)) {
+                for (int bi = 0; bi < nb; bi++)
+                    if (sm.bn[bi].nchild == -2) evaluate_rest(sm.bn[bi]);   // ends with a barrier
+            }
             // ---- phase D2: numbering, children, gains, keys (warp per node) --------
             // Child indices are deterministic: the batch's nodes in order, after the
             // nodes created before this batch.
@@ -1454,6 +1533,7 @@ static void fill_args(BuildArgs &A, Ctx &c, const void *K, const void *V, const 
     A.inv_sqrt_d = (float)(1.0 / sqrt((double)p.d));
     A.lamZ = (float)p.lambda_Z; A.lamM = (float)p.lambda_M; A.eps = (float)p.eps;
     A.lam_kappa = p.lambda_kappa; A.base_frac = p.base_frac;
+    A.prune = p.lambda_Z >= 0.0 && p.lambda_M >= 0.0;
     A.nd_a = c.w.nd_a; A.nd_b = c.w.nd_b; A.nd_child0 = c.w.nd_child0;
     A.nd_parent = c.w.nd_parent; A.nd_unit = c.w.nd_unit;
     A.nd_nchild = c.w.nd_nchild; A.nd_cost = c.w.nd_cost;

@@ -42,3 +42,20 @@ def test_class_edges_match_the_oracle(dtype, d, gq, W, fill):
     g = P.run_gpu(K, V, Q, B, w.rope_base, slot_starts=slots)
     o = P.run_oracle(K, V, Q, B, w.rope_base, slot_starts=slots)
     P.compare(g, o, torch.float32 if dtype == "fp32" else torch.bfloat16)
+
+
+@pytest.mark.parametrize("lam", [0.0, 0.002, 1.0])
+@pytest.mark.parametrize("dtype,d", [("bf16", 64), ("fp32", 128)])
+def test_cut_bounds_match_the_oracle(dtype, d, lam):
+    # A cut is left out when D + lambda_kappa kh is below the best cut found: with
+    # lambda_kappa 0 none is, at 1 nearly all are, at 0.002 some nodes keep a few
+    # and compare them with the extraction.
+    w = dataclasses.replace(synth.WORKLOADS["small"], L=1, G=2, Hq=4, d=d)
+    x = synth.make_inputs(w, T=700, W=16)
+    K, V, Q = x.K, x.V, x.Q
+    if dtype == "fp32":
+        K, V, Q = K.float(), V.float(), Q.float()
+    B = 2 * 700 // 4
+    g = P.run_gpu(K, V, Q, B, w.rope_base, lambda_kappa=lam)
+    o = P.run_oracle(K, V, Q, B, w.rope_base, lambda_kappa=lam)
+    P.compare(g, o, torch.float32 if dtype == "fp32" else torch.bfloat16)
