@@ -25,11 +25,13 @@
 //   long_collect  (CTA per listed unit) the nodes to evaluate -- a fresh root,
 //                 or the pending nodes whose key bound reaches tau -- as one
 //                 contiguous, ordered block of work items per unit;
-//   long_eval     (CTA per work item, grid-stride) one node: cut candidates,
-//                 per-segment sums between the candidate boundaries (at most
-//                 20 segments; each candidate's prototype sums are the sum of
-//                 its segments), the probe scans reading K, V and the token
-//                 values from global memory, the decision;
+//   long_eval     (CTA per work item, taken from a counter) one node: cut
+//                 candidates, per-segment sums between the candidate boundaries
+//                 (at most 20 segments; each candidate's prototype sums are the
+//                 sum of its segments), the probe scans reading V and the probe
+//                 weights through a staging ring, the decision.  Only the cut of
+//                 largest curvature reward is evaluated at first; a cut whose
+//                 exact bound is below it is never evaluated (build.cu);
 //   long_commit   (warp per unit) children numbered in work-item order after
 //                 the unit's existing nodes (deterministic), records, Split ops,
 //                 pending bounds.
@@ -52,10 +54,12 @@ constexpr int kLCL = 8;           // threads per probe pair (4-element groups, i
 constexpr int kLPPW = 32 / kLCL;  // probe pairs per warp
 constexpr int kLNW = kLT / 32;    // warps
 constexpr int kLNCD = 20;         // candidate rows per direction (17 cuts + p* side + whole node)
-constexpr int kLMaxCut = 18;      // K + midpoint, K <= 16 (+1 spare)
+constexpr int kLMaxK = 16;        // largest K
+constexpr int kLMaxCut = 18;      // K + midpoint (+1 spare)
 constexpr int kLMaxSeg = 24;      // segments between the boundaries a, b, the cuts, p*, p* + 1
 constexpr int kLFold = 32;        // tokens per fp32 partial sum of a scan
 constexpr int kLChunk = 32;       // tokens per staged chunk of a scan
+constexpr int kLU = 4;            // tokens loaded at a time by the segment sums (divides kLFold)
 
 struct LongRes {
     int nch;               // -1: pending (root only), 0: leaf (non-finite inputs), 2 or 3
@@ -79,6 +83,7 @@ struct LongArgs {
     float inv_sqrt_d, lamZ, lamM, eps, lam_kappa, base_frac;
     int fresh;                     // 1: the roots of the listed slots; 0: pending nodes of listed units
     int root_only;                 // fresh: only the root's own distortion (its split stays pending)
+    int prune;                     // lambda_Z, lambda_M >= 0, so every D >= 0: cuts may be ruled out by bounds
     float tau;                     // resume: evaluate pending nodes whose key bound >= tau
     const int32_t *list;           // fresh: slot indices; resume: unit ids
     int n_list, lg0, nlg;          // fresh units: slot list x (l, g) in [lg0, lg0 + nlg)
@@ -132,38 +137,30 @@ __device__ __forceinline__ float4 lld4(const __nv_bfloat16 *p) {
     const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.y));
     return make_float4(a.x, a.y, b.x, b.y);
 }
-template <int N>
-__device__ __forceinline__ void lld_pairs(const float *p, float v[N]) {
-#pragma unroll
-    for (int j = 0; j < N; j++) v[j] = p[j];
-}
-template <int N>
-__device__ __forceinline__ void lld_pairs(const __nv_bfloat16 *p, float v[N]) {
-#pragma unroll
-    for (int j = 0; j < N; j++) v[j] = __bfloat162float(p[j]);
-}
-
-// Block-wide best (key descending, position ascending); pos = INT_MAX: none.
-// Every thread returns the winner.  scratch: kLNW keys and positions.
-__device__ __forceinline__ void block_best(unsigned long long &key, int &pos, unsigned long long *sk, int *sp) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, key, o);
-        const int p2 = __shfl_xor_sync(0xffffffffu, pos, o);
-        if (p2 != INT_MAX && (pos == INT_MAX || k2 > key || (k2 == key && p2 < pos))) { key = k2; pos = p2; }
+// N consecutive elements of a row, held raw until they are used (one load for N = 2).
+template <typename T, int N> struct LRaw;
+template <int N> struct LRaw<float, N> {
+    float v[N];
+    __device__ __forceinline__ void load(const float *p) {
+        if constexpr (N == 2) {
+            const float2 x = *reinterpret_cast<const float2 *>(p);
+            v[0] = x.x; v[1] = x.y;
+        } else {
+            v[0] = p[0];
+        }
     }
-    if (lane == 0) { sk[warp] = key; sp[warp] = pos; }
-    __syncthreads();
-    key = sk[0];
-    pos = sp[0];
-    for (int w = 1; w < kLNW; w++) {
-        const unsigned long long k2 = sk[w];
-        const int p2 = sp[w];
-        if (p2 != INT_MAX && (pos == INT_MAX || k2 > key || (k2 == key && p2 < pos))) { key = k2; pos = p2; }
+    __device__ __forceinline__ float get(int j) const { return v[j]; }
+};
+template <int N> struct LRaw<__nv_bfloat16, N> {
+    uint32_t u;
+    __device__ __forceinline__ void load(const __nv_bfloat16 *p) {
+        if constexpr (N == 2) u = *reinterpret_cast<const uint32_t *>(p);
+        else u = *reinterpret_cast<const uint16_t *>(p);
     }
-    __syncthreads();
-}
+    __device__ __forceinline__ float get(int j) const {   // bf16 -> fp32 is exact: the bits move to the high half
+        return __uint_as_float(j ? u & 0xFFFF0000u : u << 16);
+    }
+};
 
 // Block-wide sum of a float (fixed order: lanes, then warps ascending).
 __device__ __forceinline__ float block_sum(float v, float *sf) {
@@ -315,61 +312,65 @@ __global__ void __launch_bounds__(kLT) long_collect_kernel(LongArgs A) {
 // ---------------------------------------------------------------------------
 // long_eval: one node per CTA (grid-stride over the level's work items)
 // ---------------------------------------------------------------------------
-template <int DH>
+template <int DH, typename Tin>
 struct LongSmem {
+    static constexpr int RB = DH * (int)sizeof(Tin);                // bytes of a K or V row
+    static constexpr int AB = RB > kLPP * 8 ? RB : kLPP * 8;        // of a key row or a row of probe weights
     float sk[kLMaxSeg][DH];          // per segment: sum of k_circ
     float srv[kLMaxSeg][DH];         //              sum of R v
     float ssv[kLMaxSeg][DH];         //              sum of v
+    float ktil[2 * kLNCD][DH], vtil[2 * kLNCD][DH];
+    union {
+        // the probe scans' staging ring: per buffer kLChunk value rows, then as
+        // many probe-weight rows (32 float2) or key rows
+        __align__(16) unsigned char ring[2][kLChunk * (RB + AB)];
+        float red[kLNW][3 * DH + 2];     // per-warp partials of one segment (before the scans)
+        struct {                         // the warps' largest curvatures (before the segments)
+            unsigned long long key[kLNW * kLMaxK];
+            int pos[kLNW * kLMaxK];
+        } top;
+    };
+    float redD[2 * kLNCD][kLNW], redP[2 * kLNCD][kLNW];
     float sR[kLMaxSeg], sKn[kLMaxSeg];
     int sF[kLMaxSeg];                // accepted floor positions in the segment
-    float red[kLNW][3 * DH + 2];     // per-warp partials of one segment
-    float ktil[2 * kLNCD][DH], vtil[2 * kLNCD][DH];
-    float redD[2 * kLNCD][kLNW], redP[2 * kLNCD][kLNW];
     float candD[2 * kLNCD], candP[2 * kLNCD], meff[2 * kLNCD];
-    // the probe scans' staging ring: per buffer kLChunk value rows, then as
-    // many probe-weight rows (32 float2) or key rows
-    __align__(16) unsigned char ring[2][kLChunk * DH * 4 * 2];
     int ca[2 * kLNCD], cb[2 * kLNCD];   // prefixes at [0, npre) by ascending end, suffixes at
                                         // [kLNCD, kLNCD + nsuf) by descending start (absolute)
+    uint8_t need[2 * kLNCD];            // rows that the next scans evaluate
     int segb[kLMaxSeg + 1];
     int nseg;
     int sel[kLMaxCut], cut[kLMaxCut], pidx[kLMaxCut], sidx[kLMaxCut];
-    int ncut, npre, nsuf, eL, eR, whole, pstar, forced;
-    double kmin;
-    float krange;
-    unsigned long long bk[kLNW];
-    int bp[kLNW];
-    float bf[kLNW];
+    float kh[kLMaxCut];              // normalised curvature of the cuts
+    int ncut, npre, nsuf, eL, eR, whole, pstar, forced, k1;
+    unsigned long long kmaxk;        // largest curvature key
+    unsigned long long bk[kLNW];     // per warp: smallest curvature key
+    unsigned rk[kLNW], fk[kLNW];     //           largest token value, floor score (keys)
+    int rp[kLNW], fp[kLNW];          //           and their positions
     int bad;
+    unsigned alive;                  // cuts whose both sides are evaluated
+    int extn;                        // the extraction's sides are evaluated
+    int more;                        // rows are left to evaluate
 };
 
-// Order-preserving 32-bit key of a float, widened (larger value -> larger key).
-__device__ __forceinline__ unsigned long long fokey(float x) {
+// Order-preserving 32-bit key of a float (larger value -> larger key).
+__device__ __forceinline__ unsigned fokey(float x) {
     const uint32_t u = __float_as_uint(x);
-    return (u >> 31) ? (unsigned long long)(~u) : (unsigned long long)(u | 0x80000000u);
+    return (u >> 31) ? ~u : u | 0x80000000u;
 }
 
-// Sort the rows [r0, r0 + m) of (ca, cb) by key (ascending), remapping the
-// indices in idx[0 .. ni) that point into them.  Thread 0 only; m <= kLNCD.
-__device__ void sort_rows(int *ca, int *cb, int r0, int m, bool by_end_asc, int *const *idx, int ni) {
-    int perm[kLNCD], inv[kLNCD], ta[kLNCD], tb[kLNCD];
-    for (int q = 0; q < m; q++) perm[q] = q;
-    auto key = [&](int q) { return by_end_asc ? cb[r0 + q] : -ca[r0 + q]; };
-    for (int x = 1; x < m; x++) {
-        const int v = perm[x];
-        int y = x - 1;
-        while (y >= 0 && key(perm[y]) > key(v)) { perm[y + 1] = perm[y]; y--; }
-        perm[y + 1] = v;
-    }
-    for (int q = 0; q < m; q++) { inv[perm[q]] = q; ta[q] = ca[r0 + perm[q]]; tb[q] = cb[r0 + perm[q]]; }
-    for (int q = 0; q < m; q++) { ca[r0 + q] = ta[q]; cb[r0 + q] = tb[q]; }
-    for (int k = 0; k < ni; k++)
-        if (*idx[k] >= r0 && *idx[k] < r0 + m) *idx[k] = r0 + inv[*idx[k] - r0];
-}
-
-template <int DH, typename Tin>
-__global__ void __launch_bounds__(kLT, 1) long_eval_kernel(LongArgs A) {
-    using S = LongSmem<DH>;
+// Bound by the fp32 FMAs of the probe scan (2 W d per token) and by latency, so
+// two CTAs share an SM: the staging ring's bytes hold the segment partials and
+// the curvature candidates before the scans, and the queries are read back for
+// each evaluated row.  Skew 64K at 32x, all 16 launches: 161 -> 77 ms with the
+// bound (half of the scanned tokens, 3 rows of about 36 for most nodes), the
+// second CTA, tokens loaded four at a time by the segment sums, scans in
+// stretches between fold points without a test per token, and the top-K drawn
+// per warp in place of 16 block-wide passes over the curvature.
+// EG: the probe weights of every token were written by the score pass; only
+// then the queries need no registers during the scans.
+template <int DH, typename Tin, bool EG>
+__global__ void __launch_bounds__(kLT, EG ? 2 : 1) long_eval_kernel(LongArgs A) {
+    using S = LongSmem<DH, Tin>;
     constexpr int HALF = DH / 2, NG = DH / (4 * kLCL), CH = 4 * NG, PPL = HALF / 32;
     static_assert(kLPP * kLCL == kLT && DH % (4 * kLCL) == 0 && HALF % 32 == 0, "layout");
     extern __shared__ __align__(16) unsigned char lsm_raw[];
@@ -396,220 +397,325 @@ __global__ void __launch_bounds__(kLT, 1) long_eval_kernel(LongArgs A) {
         const float *Rg = A.rtok + (size_t)lg * A.Nc - A.cs;   // Rg[t]: token value at absolute t
         const Tin *Kl = static_cast<const Tin *>(A.K) + (size_t)lg * A.T * DH;
         const Tin *Vl = static_cast<const Tin *>(A.V) + (size_t)lg * A.T * DH;
+        const unsigned FULL = 0xffffffffu;
         if (tid == 0) sm.bad = 0;
+        __syncthreads();
         // ---- phase A: cut candidates, curvature range, p*, forced floor position
+        // top-K positions of [a, b-2] by (kappa descending, position ascending):
+        // every warp draws its own K, a lane looking for its next position only
+        // when its last one was taken; the K best of them are ranked by counting.
         {
-            unsigned long long kmin = ~0ull, kmax = 0ull;
+            unsigned long long kmin = ~0ull, bkey = 0ull;
+            int bpos = INT_MAX;
+#pragma unroll 4
             for (int t = a + tid; t <= b - 2; t += kLT) {
                 const unsigned long long k = lokey(A.kappa[t]);
                 kmin = min(kmin, k);
-                kmax = max(kmax, k);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                kmin = min(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
-                kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
-            }
-            if (lane == 0) { sm.bk[warp] = kmin; sm.bp[warp] = (int)0; }
-            __syncthreads();
-            if (tid == 0) {
-                unsigned long long mn = ~0ull;
-                for (int w = 0; w < kLNW; w++) mn = min(mn, sm.bk[w]);
-                sm.kmin = n >= 2 ? lokey_inv(mn) : 0.0;
-            }
-            __syncthreads();
-            if (lane == 0) sm.bk[warp] = kmax;
-            __syncthreads();
-            if (tid == 0) {
-                unsigned long long mx = 0ull;
-                for (int w = 0; w < kLNW; w++) mx = max(mx, sm.bk[w]);
-                const double kmx = n >= 2 ? lokey_inv(mx) : 0.0;
-                sm.krange = kmx > sm.kmin ? 1.0f / (float)(kmx - sm.kmin) : 0.f;
-            }
-            __syncthreads();
-        }
-        // top-K positions of [a, b-2] by (kappa descending, position ascending)
-        const int K = cands ? min(A.k_cand, n - 1) : 0;
-        unsigned long long pk = 0ull;
-        int ppos = -1, nsel = 0;
-        for (int r = 0; r < K; r++) {
-            unsigned long long bkey = 0ull;
-            int bpos = INT_MAX;
-            for (int t = a + tid; t <= b - 2; t += kLT) {
-                const unsigned long long k = lokey(A.kappa[t]);
-                if (r > 0 && !(k < pk || (k == pk && t > ppos))) continue;   // taken in an earlier round
-                if (bpos == INT_MAX || k > bkey || (k == bkey && t < bpos)) { bkey = k; bpos = t; }
-            }
-            block_best(bkey, bpos, sm.bk, sm.bp);
-            if (bpos == INT_MAX) break;
-            if (tid == 0) sm.sel[r] = bpos;
-            pk = bkey;
-            ppos = bpos;
-            nsel++;
-        }
-        // salient token p* = argmax R_tok over [a, b) (ties: lower t)
-        {
-            unsigned long long bkey = 0ull;
-            int bpos = INT_MAX;
-            for (int t = a + tid; t < b; t += kLT) {
-                const float r = Rg[t];
-                if (!isfinite(r)) sm.bad = 1;
-                const unsigned long long k = fokey(r);
                 if (bpos == INT_MAX || k > bkey) { bkey = k; bpos = t; }
             }
-            block_best(bkey, bpos, sm.bk, sm.bp);
-            if (tid == 0) sm.pstar = (bpos >= a && bpos < b) ? bpos : a;
-        }
-        // a node holding an accepted floor position is extracted at the one of
-        // largest floor score (ties: lower t)
-        {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) kmin = min(kmin, __shfl_xor_sync(FULL, kmin, o));
+            // salient token p* = argmax R_tok over [a, b) (ties: lower t)
+            unsigned rkey = 0u;
+            int rpos = INT_MAX;
+            bool nonf = false;
+#pragma unroll 4
+            for (int t = a + tid; t < b; t += kLT) {
+                const float r = Rg[t];
+                nonf |= !isfinite(r);
+                const unsigned k = fokey(r);
+                if (rpos == INT_MAX || k > rkey) { rkey = k; rpos = t; }
+            }
+            if (nonf) sm.bad = 1;
+            // a node holding an accepted floor position is extracted at the one of
+            // largest floor score (ties: lower t)
+            unsigned fkey = 0u;
             int fpos = INT_MAX;
-            if (A.fl_acc) {
-                unsigned long long bkey = 0ull;
+            if (A.fl_acc)
                 for (int t = a + tid; t < b; t += kLT) {
                     const size_t q = (size_t)lg * A.Nc + (t - A.cs);
                     if (!A.fl_acc[q]) continue;
-                    const unsigned long long k = fokey(A.fl_f[q]);
-                    if (fpos == INT_MAX || k > bkey) { bkey = k; fpos = t; }
+                    const unsigned k = fokey(A.fl_f[q]);
+                    if (fpos == INT_MAX || k > fkey) { fkey = k; fpos = t; }
                 }
-                block_best(bkey, fpos, sm.bk, sm.bp);
+            const unsigned rmx = __reduce_max_sync(FULL, rpos != INT_MAX ? rkey : 0u);
+            const int rmp = __reduce_min_sync(FULL, rpos != INT_MAX && rkey == rmx ? rpos : INT_MAX);
+            const unsigned fmx = __reduce_max_sync(FULL, fpos != INT_MAX ? fkey : 0u);
+            const int fmp = __reduce_min_sync(FULL, fpos != INT_MAX && fkey == fmx ? fpos : INT_MAX);
+            if (lane == 0) {
+                sm.bk[warp] = kmin;
+                sm.rk[warp] = rmx; sm.rp[warp] = rmp;
+                sm.fk[warp] = fmx; sm.fp[warp] = fmp;
             }
-            if (tid == 0) {
-                sm.forced = fpos != INT_MAX ? 1 : 0;
-                if (fpos != INT_MAX) sm.pstar = fpos;
+            // one at least, for the curvature range (n > kMaxUnit > K)
+            const int K = cands ? max(A.k_cand, 1) : 0;
+            for (int r = 0; r < K; r++) {
+                const unsigned hi = (unsigned)(bkey >> 32), lo = (unsigned)bkey;
+                const bool v0 = bpos != INT_MAX;
+                const unsigned mh = __reduce_max_sync(FULL, v0 ? hi : 0u);
+                const bool v1 = v0 && hi == mh;
+                const unsigned ml = __reduce_max_sync(FULL, v1 ? lo : 0u);
+                const int mp = __reduce_min_sync(FULL, v1 && lo == ml ? bpos : INT_MAX);
+                if (lane == 0) {
+                    sm.top.key[warp * kLMaxK + r] = ((unsigned long long)mh << 32) | ml;
+                    sm.top.pos[warp * kLMaxK + r] = mp;   // INT_MAX: the warp's positions are used up
+                }
+                if (bpos == mp && v0) {   // this lane's position was taken: its next one
+                    const unsigned long long pk = bkey;
+                    const int ppos = bpos;
+                    bkey = 0ull;
+                    bpos = INT_MAX;
+#pragma unroll 4
+                    for (int t = a + tid; t <= b - 2; t += kLT) {
+                        const unsigned long long k = lokey(A.kappa[t]);
+                        if ((k < pk || (k == pk && t > ppos)) && (bpos == INT_MAX || k > bkey)) { bkey = k; bpos = t; }
+                    }
+                }
             }
+            __syncthreads();
+            if (K > 0 && tid < kLNW * K) {
+                const int i = (tid / K) * kLMaxK + tid % K;
+                const unsigned long long k = sm.top.key[i];
+                const int pos = sm.top.pos[i];
+                int rank = 0;
+                for (int w = 0; w < kLNW; w++)
+                    for (int r = 0; r < K; r++) {
+                        const unsigned long long k2 = sm.top.key[w * kLMaxK + r];
+                        const int p2 = sm.top.pos[w * kLMaxK + r];
+                        rank += p2 != INT_MAX && (k2 > k || (k2 == k && p2 < pos));
+                    }
+                if (pos != INT_MAX && rank < K) {
+                    sm.sel[rank] = pos;
+                    if (rank == 0) sm.kmaxk = k;
+                }
+            }
+            __syncthreads();
         }
-        __syncthreads();
-        // candidate lists and segment boundaries (thread 0)
-        if (tid == 0) {
-            int nc = 0;
-            if (cands) {
-                const int mid = a + n / 2;
-                bool have = false;
-                for (int r = 0; r < nsel; r++) { sm.cut[nc++] = sm.sel[r] + 1; have |= sm.sel[r] + 1 == mid; }
-                if (!have) sm.cut[nc++] = mid;
-                for (int x = 1; x < nc; x++) {
-                    const int v = sm.cut[x];
-                    int y = x - 1;
-                    while (y >= 0 && sm.cut[y] > v) { sm.cut[y + 1] = sm.cut[y]; y--; }
-                    sm.cut[y + 1] = v;
+        // candidate rows, segment boundaries and the rows evaluated first (warp 0)
+        if (warp == 0) {
+            const int wl = lane < kLNW ? lane : 0;
+            const unsigned rmx = __reduce_max_sync(FULL, sm.rp[wl] != INT_MAX ? sm.rk[wl] : 0u);
+            int ps = __reduce_min_sync(FULL, sm.rp[wl] != INT_MAX && sm.rk[wl] == rmx ? sm.rp[wl] : INT_MAX);
+            const unsigned fmx = __reduce_max_sync(FULL, sm.fp[wl] != INT_MAX ? sm.fk[wl] : 0u);
+            const int fps = __reduce_min_sync(FULL, sm.fp[wl] != INT_MAX && sm.fk[wl] == fmx ? sm.fp[wl] : INT_MAX);
+            if (!(ps >= a && ps < b)) ps = a;
+            const bool forced = fps != INT_MAX;
+            if (forced) ps = fps;
+            const int er = ps + 1;
+            const int K = cands ? A.k_cand : 0;   // n > kMaxUnit > K: K positions were found
+            // cuts in ascending order: the positions' successors and the midpoint
+            const int mid = a + n / 2;
+            int xi = lane < K ? sm.sel[lane] + 1 : INT_MAX;
+            const bool have = __any_sync(FULL, xi == mid);
+            int ncut = K;
+            if (cands && !have) {
+                if (lane == K) xi = mid;
+                ncut++;
+            }
+            int at = 0;
+            for (int q = 0; q < ncut; q++) at += __shfl_sync(FULL, xi, q) < xi;
+            __syncwarp();
+            if (lane < ncut) sm.cut[at] = xi;
+            __syncwarp();
+            xi = lane < ncut ? sm.cut[lane] : INT_MAX;
+            float kh = 0.f;
+            if (lane < ncut) {
+                unsigned long long mn = ~0ull;
+                for (int w = 0; w < kLNW; w++) mn = min(mn, sm.bk[w]);
+                const double kmn = lokey_inv(mn), kmx = lokey_inv(sm.kmaxk);
+                const float krange = kmx > kmn ? 1.0f / (float)(kmx - kmn) : 0.f;
+                kh = (float)(A.kappa[xi - 1] - kmn) * krange;
+                sm.kh[lane] = kh;
+            }
+            const unsigned rew = lane < ncut ? fokey(A.lam_kappa * kh + 0.f) : 0u;
+            const unsigned rew_mx = __reduce_max_sync(FULL, rew);
+            const int k1 = __ffs(__ballot_sync(FULL, rew == rew_mx)) - 1;
+            // rows: prefixes [a, xi) and [a, p*) by ascending end, the node itself
+            // last; suffixes [xi, b) and [p* + 1, b) by descending start
+            const unsigned lt = (1u << lane) - 1u, gt = ~((2u << lane) - 1u);
+            const bool pv = lane < ncut && xi - a >= 2, sv = lane < ncut && b - xi >= 2;
+            const bool elv = cands && ps - a >= 2, erv = cands && b - er >= 2;
+            const unsigned pm = __ballot_sync(FULL, pv), sm_ = __ballot_sync(FULL, sv);
+            const unsigned pdup = __ballot_sync(FULL, pv && xi == ps), sdup = __ballot_sync(FULL, sv && xi == er);
+            const bool elr = elv && !pdup, err = erv && !sdup;   // rows of their own
+            const int prow = __popc(pm & lt) + (elr && ps < xi ? 1 : 0);
+            const int srow = kLNCD + __popc(sm_ & gt) + (err && er > xi ? 1 : 0);
+            const int el_at = __popc(__ballot_sync(FULL, pv && xi < ps));
+            const int er_at = kLNCD + __popc(__ballot_sync(FULL, sv && xi > er));
+            const int npre0 = __popc(pm) + elr, npre = npre0 + root, nsuf = __popc(sm_) + err;
+            if (pv) { sm.ca[prow] = a; sm.cb[prow] = xi; }
+            if (sv) { sm.ca[srow] = xi; sm.cb[srow] = b; }
+            if (lane < ncut) { sm.pidx[lane] = pv ? prow : -1; sm.sidx[lane] = sv ? srow : -1; }
+            for (int q = lane; q < 2 * kLNCD; q += 32) sm.need[q] = 0;
+            __syncwarp();
+            const int eL = elv ? el_at : -1, eR = erv ? er_at : -1;
+            if (lane == 0) {
+                if (elr) { sm.ca[eL] = a; sm.cb[eL] = ps; }
+                if (err) { sm.ca[eR] = er; sm.cb[eR] = b; }
+                if (root) { sm.ca[npre0] = a; sm.cb[npre0] = b; sm.need[npre0] = 1; }
+                sm.npre = npre; sm.nsuf = nsuf; sm.eL = eL; sm.eR = eR; sm.whole = root ? npre0 : -1;
+                sm.ncut = ncut; sm.pstar = ps; sm.forced = forced; sm.k1 = k1;
+                // evaluated first: both sides of the cut of largest reward, or of a
+                // forced extraction; a fresh root's own
+                if (cands) {
+                    const int r0 = forced ? eL : sm.pidx[k1], r1 = forced ? eR : sm.sidx[k1];
+                    if (r0 >= 0) sm.need[r0] = 1;
+                    if (r1 >= 0) sm.need[r1] = 1;
                 }
+                sm.alive = cands && !forced ? 1u << k1 : 0u;
+                sm.extn = forced;
+                sm.more = 0;
             }
-            sm.ncut = nc;
-            const int ps = sm.pstar, er = ps + 1;
-            int npre = 0, nsuf = 0;
-            for (int q = 0; q < nc; q++) {
-                const int xi = sm.cut[q];
-                sm.pidx[q] = -1;
-                if (xi - a >= 2) { sm.ca[npre] = a; sm.cb[npre] = xi; sm.pidx[q] = npre++; }
-            }
-            int eL = -1, eR = -1, whole = -1;
-            if (cands && ps - a >= 2) {
-                for (int q = 0; q < nc; q++) if (sm.cut[q] == ps && sm.pidx[q] >= 0) eL = sm.pidx[q];
-                if (eL < 0) { sm.ca[npre] = a; sm.cb[npre] = ps; eL = npre++; }
-            }
-            if (root) { sm.ca[npre] = a; sm.cb[npre] = b; whole = npre++; }
-            for (int q = 0; q < nc; q++) {
-                const int xi = sm.cut[q];
-                sm.sidx[q] = -1;
-                if (b - xi >= 2) { sm.ca[kLNCD + nsuf] = xi; sm.cb[kLNCD + nsuf] = b; sm.sidx[q] = kLNCD + nsuf++; }
-            }
-            if (cands && b - er >= 2) {
-                for (int q = 0; q < nc; q++) if (sm.cut[q] == er && sm.sidx[q] >= 0) eR = sm.sidx[q];
-                if (eR < 0) { sm.ca[kLNCD + nsuf] = er; sm.cb[kLNCD + nsuf] = b; eR = kLNCD + nsuf++; }
-            }
-            {
-                int *pi[kLMaxCut + 2];
-                int ni = 0;
-                for (int q = 0; q < nc; q++) pi[ni++] = &sm.pidx[q];
-                pi[ni++] = &eL;
-                pi[ni++] = &whole;
-                sort_rows(sm.ca, sm.cb, 0, npre, true, pi, ni);
-                ni = 0;
-                for (int q = 0; q < nc; q++) pi[ni++] = &sm.sidx[q];
-                pi[ni++] = &eR;
-                sort_rows(sm.ca, sm.cb, kLNCD, nsuf, false, pi, ni);
-            }
-            sm.npre = npre; sm.nsuf = nsuf; sm.eL = eL; sm.eR = eR; sm.whole = whole;
             // segment boundaries: a, b, the cuts, p*, p* + 1
-            int bd[kLMaxCut + 4], nb = 0;
-            bd[nb++] = a;
-            bd[nb++] = b;
-            for (int q = 0; q < nc; q++) bd[nb++] = sm.cut[q];
-            if (ps > a) bd[nb++] = ps;
-            if (er < b) bd[nb++] = er;
-            for (int x = 1; x < nb; x++) {
-                const int v = bd[x];
-                int y = x - 1;
-                while (y >= 0 && bd[y] > v) { bd[y + 1] = bd[y]; y--; }
-                bd[y + 1] = v;
-            }
-            int m = 0;
-            for (int x = 0; x < nb; x++) if (m == 0 || bd[x] != sm.segb[m - 1]) sm.segb[m++] = bd[x];
-            sm.nseg = m - 1;
+            const bool ps_in = ps > a && !__any_sync(FULL, xi == ps), er_in = er < b && !__any_sync(FULL, xi == er);
+            int bd = xi;
+            if (lane == 30) bd = ps_in ? ps : INT_MAX;
+            if (lane == 31) bd = er_in ? er : INT_MAX;
+            int slot = 1;
+            for (int q = 0; q < 32; q++) slot += __shfl_sync(FULL, bd, q) < bd;
+            if (bd != INT_MAX) sm.segb[slot] = bd;
+            const int nin = __popc(__ballot_sync(FULL, bd != INT_MAX));
+            if (lane == 0) { sm.segb[0] = a; sm.segb[nin + 1] = b; sm.nseg = nin + 1; }
         }
         __syncthreads();
         // ---- phase B: per-segment sums of k_circ, R v, v, R, ||k|| and floor positions
         // Warp w takes the tokens x + w, x + w + 8, ...; lane owns the rotation
         // pairs (i, i + d/2), i = PPL lane + j.  Each warp's running sums are
         // folded every kLFold of its tokens.
+        // Tokens are loaded kLU at a time before any is added (a token at a time
+        // was bound by the loads' latency).
         const int nseg = sm.nseg;
-        for (int s = 0; s < nseg; s++) {
-            const int x = sm.segb[s], y = sm.segb[s + 1];
-            const int i0 = lane * PPL;
-            float tk0[PPL], tk1[PPL], tr0[PPL], tr1[PPL], tv0[PPL], tv1[PPL];
-            float ck0[PPL], ck1[PPL], cr0[PPL], cr1[PPL], cv0[PPL], cv1[PPL];
-            float trs = 0.f, tks = 0.f, crs = 0.f, cks = 0.f;
+        const int i0 = lane * PPL;
+        struct Acc {
+            float k0[PPL], k1[PPL], r0[PPL], r1[PPL], v0[PPL], v1[PPL], rs, ks;
+            __device__ __forceinline__ void clear() {
 #pragma unroll
-            for (int j = 0; j < PPL; j++) tk0[j] = tk1[j] = tr0[j] = tr1[j] = tv0[j] = tv1[j] = 0.f;
-#pragma unroll
-            for (int j = 0; j < PPL; j++) ck0[j] = ck1[j] = cr0[j] = cr1[j] = cv0[j] = cv1[j] = 0.f;
-            int fold = 0;
-            for (int t = x + warp; t < y; t += kLNW) {
-                float k0[PPL], k1[PPL], v0[PPL], v1[PPL];
-                lld_pairs<PPL>(Kl + (size_t)t * DH + i0, k0);
-                lld_pairs<PPL>(Kl + (size_t)t * DH + i0 + HALF, k1);
-                lld_pairs<PPL>(Vl + (size_t)t * DH + i0, v0);
-                lld_pairs<PPL>(Vl + (size_t)t * DH + i0 + HALF, v1);
-                const float rt = Rg[t];
-                float nn = 0.f;
+                for (int j = 0; j < PPL; j++) k0[j] = k1[j] = r0[j] = r1[j] = v0[j] = v1[j] = 0.f;
+                rs = ks = 0.f;
+            }
+            __device__ __forceinline__ void add(const Acc &o) {
 #pragma unroll
                 for (int j = 0; j < PPL; j++) {
-                    nn = fmaf(k0[j], k0[j], fmaf(k1[j], k1[j], nn));
-                    const float2 cs = A.rope[(size_t)t * HALF + i0 + j];
-                    // k_circ = RoPE^-1(k, t): rotation by -t
-                    ck0[j] += k0[j] * cs.x + k1[j] * cs.y;
-                    ck1[j] += k1[j] * cs.x - k0[j] * cs.y;
-                    cr0[j] = fmaf(rt, v0[j], cr0[j]);
-                    cr1[j] = fmaf(rt, v1[j], cr1[j]);
-                    cv0[j] += v0[j];
-                    cv1[j] += v1[j];
+                    k0[j] += o.k0[j]; k1[j] += o.k1[j]; r0[j] += o.r0[j]; r1[j] += o.r1[j];
+                    v0[j] += o.v0[j]; v1[j] += o.v1[j];
                 }
-                nn = warp_sum(nn);
-                crs += rt;
-                cks += sqrtf(nn);
-                if (++fold == kLFold) {
+                rs += o.rs;
+                ks += o.ks;
+            }
+        };
+        struct Tok {
+            LRaw<Tin, PPL> k0, k1, v0, v1;
+            float2 cs[PPL];
+            float r;
+        };
+        auto load_tok = [&](Tok &x, int t) {
+            const size_t e = (size_t)t * DH + i0;
+            x.k0.load(Kl + e); x.k1.load(Kl + e + HALF);
+            x.v0.load(Vl + e); x.v1.load(Vl + e + HALF);
+            const float2 *rp = A.rope + (size_t)t * HALF + i0;
+            if constexpr (PPL == 2) {
+                const float4 c4 = *reinterpret_cast<const float4 *>(rp);
+                x.cs[0] = make_float2(c4.x, c4.y);
+                x.cs[1] = make_float2(c4.z, c4.w);
+            } else {
+                x.cs[0] = rp[0];
+            }
+            x.r = Rg[t];
+        };
+        auto norm_tok = [&](const Tok &x) {   // ||k_t||^2, the same in every lane
+            float nn = 0.f;
 #pragma unroll
-                    for (int j = 0; j < PPL; j++) {
-                        tk0[j] += ck0[j]; tk1[j] += ck1[j]; tr0[j] += cr0[j]; tr1[j] += cr1[j];
-                        tv0[j] += cv0[j]; tv1[j] += cv1[j];
-                        ck0[j] = ck1[j] = cr0[j] = cr1[j] = cv0[j] = cv1[j] = 0.f;
+            for (int j = 0; j < PPL; j++) {
+                const float k0 = x.k0.get(j), k1 = x.k1.get(j);
+                nn = fmaf(k0, k0, fmaf(k1, k1, nn));
+            }
+            return warp_sum(nn);
+        };
+        auto add_tok = [&](Acc &c, const Tok &x, float nn) {
+#pragma unroll
+            for (int j = 0; j < PPL; j++) {
+                const float k0 = x.k0.get(j), k1 = x.k1.get(j), v0 = x.v0.get(j), v1 = x.v1.get(j);
+                // k_circ = RoPE^-1(k, t): rotation by -t
+                c.k0[j] += fmaf(k0, x.cs[j].x, k1 * x.cs[j].y);
+                c.k1[j] += fmaf(k1, x.cs[j].x, -(k0 * x.cs[j].y));
+                c.r0[j] = fmaf(x.r, v0, c.r0[j]);
+                c.r1[j] = fmaf(x.r, v1, c.r1[j]);
+                c.v0[j] += v0;
+                c.v1[j] += v1;
+            }
+            c.rs += x.r;
+            c.ks += sqrtf(nn);
+        };
+        // segments of at most kLNW tokens: one token per partial sum, a segment
+        // per warp and no barrier (clustered curvature peaks make many of them)
+        for (int s = 0, k = 0; s < nseg; s++) {
+            const int x = sm.segb[s], y = sm.segb[s + 1];
+            if (y - x > kLNW || k++ % kLNW != warp) continue;
+            Acc v;
+            v.clear();
+            for (int t0 = x; t0 < y; t0 += kLU) {
+                Tok tk[kLU];
+                float nn[kLU];
+#pragma unroll
+                for (int u = 0; u < kLU; u++) load_tok(tk[u], min(t0 + u, y - 1));
+#pragma unroll
+                for (int u = 0; u < kLU; u++) nn[u] = norm_tok(tk[u]);
+#pragma unroll
+                for (int u = 0; u < kLU; u++)
+                    if (t0 + u < y) {
+                        Acc c;
+                        c.clear();
+                        add_tok(c, tk[u], nn[u]);
+                        v.add(c);
                     }
-                    trs += crs; tks += cks; crs = cks = 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < PPL; j++) {
+                sm.sk[s][i0 + j] = v.k0[j];  sm.sk[s][i0 + j + HALF] = v.k1[j];
+                sm.srv[s][i0 + j] = v.r0[j]; sm.srv[s][i0 + j + HALF] = v.r1[j];
+                sm.ssv[s][i0 + j] = v.v0[j]; sm.ssv[s][i0 + j + HALF] = v.v1[j];
+            }
+            bool f = false;
+            if (A.fl_acc && lane < y - x) f = A.fl_acc[(size_t)lg * A.Nc + (x + lane - A.cs)] != 0;
+            f = __any_sync(FULL, f);
+            if (lane == 0) { sm.sR[s] = v.rs; sm.sKn[s] = v.ks; sm.sF[s] = f; }
+        }
+        for (int s = 0; s < nseg; s++) {
+            const int x = sm.segb[s], y = sm.segb[s + 1];
+            if (y - x <= kLNW) continue;
+            Acc tot, c;
+            tot.clear();
+            c.clear();
+            int fold = 0;
+            for (int t0 = x + warp; t0 < y; t0 += kLU * kLNW) {
+                Tok tk[kLU];
+                float nn[kLU];
+#pragma unroll
+                for (int u = 0; u < kLU; u++) load_tok(tk[u], min(t0 + u * kLNW, y - 1));
+#pragma unroll
+                for (int u = 0; u < kLU; u++) nn[u] = norm_tok(tk[u]);
+#pragma unroll
+                for (int u = 0; u < kLU; u++)
+                    if (t0 + u * kLNW < y) add_tok(c, tk[u], nn[u]);
+                fold += kLU;
+                if (fold == kLFold) {   // the last, partial sum may be folded here too: it adds the same
+                    tot.add(c);
+                    c.clear();
                     fold = 0;
                 }
             }
+            tot.add(c);
             float *rw = sm.red[warp];
 #pragma unroll
             for (int j = 0; j < PPL; j++) {
-                rw[i0 + j] = tk0[j] + ck0[j];
-                rw[i0 + j + HALF] = tk1[j] + ck1[j];
-                rw[DH + i0 + j] = tr0[j] + cr0[j];
-                rw[DH + i0 + j + HALF] = tr1[j] + cr1[j];
-                rw[2 * DH + i0 + j] = tv0[j] + cv0[j];
-                rw[2 * DH + i0 + j + HALF] = tv1[j] + cv1[j];
+                rw[i0 + j] = tot.k0[j];
+                rw[i0 + j + HALF] = tot.k1[j];
+                rw[DH + i0 + j] = tot.r0[j];
+                rw[DH + i0 + j + HALF] = tot.r1[j];
+                rw[2 * DH + i0 + j] = tot.v0[j];
+                rw[2 * DH + i0 + j + HALF] = tot.v1[j];
             }
-            if (lane == 0) { rw[3 * DH] = trs + crs; rw[3 * DH + 1] = tks + cks; }
+            if (lane == 0) { rw[3 * DH] = tot.rs; rw[3 * DH + 1] = tot.ks; }
             int fc = 0;
             if (A.fl_acc)
                 for (int t = x + tid; t < y; t += kLT) fc += A.fl_acc[(size_t)lg * A.Nc + (t - A.cs)] ? 1 : 0;
@@ -627,19 +733,24 @@ __global__ void __launch_bounds__(kLT, 1) long_eval_kernel(LongArgs A) {
             if (tid == 0) sm.sF[s] = fc;
             __syncthreads();
         }
+        __syncthreads();
+        const int npre = sm.npre, nsuf = sm.nsuf;
+        unsigned long long w_scan = 0, w_eval = 0, w_len = 0;   // work counters (thread 0)
+        // Stages: 0 the rows chosen above; 1 the prefixes of the cuts that stage 0
+        // does not rule out, 2 their suffixes.
+        for (int stage = 0;; stage++) {
         // ---- phase C: candidate prototypes from their segments (warp per candidate)
         auto seg_of = [&](int pos) {   // index of the boundary at pos (every candidate end is one)
             int s = 0;
             while (s < nseg && sm.segb[s] != pos) s++;
             return s;
         };
-        const int npre = sm.npre, nsuf = sm.nsuf;
         for (int q = warp; q < npre + nsuf; q += kLNW) {
             const int k = q < npre ? q : kLNCD + (q - npre);
+            if (!sm.need[k]) continue;
             const int x = sm.ca[k], y = sm.cb[k], nJ = y - x;
             const int s0 = seg_of(x), s1 = seg_of(y);
             const int p = lround_half_even_mid(x, y);
-            const int i0 = lane * PPL;
             float2 rot[PPL];
 #pragma unroll
             for (int j = 0; j < PPL; j++) rot[j] = A.rope[(size_t)p * HALF + i0 + j];
@@ -680,46 +791,61 @@ __global__ void __launch_bounds__(kLT, 1) long_eval_kernel(LongArgs A) {
         __syncthreads();
         // ---- phase D: probe scans --------------------------------------------
         // thread (pp, c): probes pp and pp + 32, elements 4 c + 32 gi + j
-        float2 qa0[CH / 2], qa1[CH / 2];
-        float mu0 = 0.f, mu1 = 0.f, invZ0 = 0.f, invZ1 = 0.f;
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int u = pp + kLPP * h;
-            float2 *qd = h ? qa1 : qa0;
+        auto qrow = [&](int u) -> size_t { return ((size_t)l * A.Hq + g * A.gq + (u % A.gq)) * A.W + u; };
+        auto load_q = [&](float2 *qd, int u) {
             if (u < A.W) {
-                const size_t row = ((size_t)l * A.Hq + g * A.gq + (u % A.gq)) * A.W + u;
-                const Tin *qp = static_cast<const Tin *>(A.Q) + row * DH + 4 * c;
+                const Tin *qp = static_cast<const Tin *>(A.Q) + qrow(u) * DH + 4 * c;
 #pragma unroll
                 for (int gi = 0; gi < NG; gi++) {
                     const float4 x = lld4(qp + 32 * gi);
                     qd[2 * gi] = make_float2(x.x, x.y);
                     qd[2 * gi + 1] = make_float2(x.z, x.w);
                 }
-                (h ? mu1 : mu0) = A.row_m[row];
-                (h ? invZ1 : invZ0) = 1.0f / A.row_Z[row];
             } else {
 #pragma unroll
                 for (int q = 0; q < CH / 2; q++) qd[q] = make_float2(0.f, 0.f);
             }
-        }
+        };
         const bool has0 = pp < A.W, has1 = pp + kLPP < A.W;
+        const float mu0 = has0 ? A.row_m[qrow(pp)] : 0.f, mu1 = has1 ? A.row_m[qrow(pp + kLPP)] : 0.f;
+        const float invZ0 = has0 ? 1.0f / A.row_Z[qrow(pp)] : 0.f, invZ1 = has1 ? 1.0f / A.row_Z[qrow(pp + kLPP)] : 0.f;
+        // the queries: kept where every token needs them, else read back for each
+        // evaluated row (a few per node)
+        float2 qk0[EG ? 1 : CH / 2], qk1[EG ? 1 : CH / 2];
+        if constexpr (!EG) {
+            load_q(qk0, pp);
+            load_q(qk1, pp + kLPP);
+        }
         // D_u of candidate row k from the running statistics, weighted by the
         // probe's attention mass; per-warp partial sums (as in build.cu)
         auto evaluate = [&](int k, float Z0, float Z1, const float2 *M0, const float2 *M1) {
-            float2 kt[CH / 2];
+            float x0, x1;
+            {
+                float2 xa = make_float2(0.f, 0.f), xb = make_float2(0.f, 0.f);
+                float2 ql0[EG ? CH / 2 : 1], ql1[EG ? CH / 2 : 1];
+                if constexpr (EG) {
+                    load_q(ql0, pp);
+                    load_q(ql1, pp + kLPP);
+                }
 #pragma unroll
-            for (int gi = 0; gi < NG; gi++) {
-                const float4 x = *reinterpret_cast<const float4 *>(&sm.ktil[k][4 * c + 32 * gi]);
-                kt[2 * gi] = make_float2(x.x, x.y);
-                kt[2 * gi + 1] = make_float2(x.z, x.w);
-            }
-            float2 xa = make_float2(0.f, 0.f), xb = make_float2(0.f, 0.f);
+                for (int gi = 0; gi < NG; gi++) {
+                    const float4 x = *reinterpret_cast<const float4 *>(&sm.ktil[k][4 * c + 32 * gi]);
+                    const float2 kt[2] = {make_float2(x.x, x.y), make_float2(x.z, x.w)};
 #pragma unroll
-            for (int q = 0; q < CH / 2; q++) {
-                xa = ffma2(qa0[q], kt[q], xa);
-                xb = ffma2(qa1[q], kt[q], xb);
+                    for (int h = 0; h < 2; h++) {
+                        const int q = 2 * gi + h;
+                        if constexpr (EG) {
+                            xa = ffma2(ql0[q], kt[h], xa);
+                            xb = ffma2(ql1[q], kt[h], xb);
+                        } else {
+                            xa = ffma2(qk0[q], kt[h], xa);
+                            xb = ffma2(qk1[q], kt[h], xb);
+                        }
+                    }
+                }
+                x0 = xa.x + xa.y;
+                x1 = xb.x + xb.y;
             }
-            float x0 = xa.x + xa.y, x1 = xb.x + xb.y;
 #pragma unroll
             for (int o = kLPPW; o < 32; o <<= 1) {
                 x0 += __shfl_xor_sync(0xffffffffu, x0, o);
@@ -769,15 +895,14 @@ __global__ void __launch_bounds__(kLT, 1) long_eval_kernel(LongArgs A) {
         // tokens are staged kLChunk at a time in a two-buffer cp.async ring:
         // their value rows and their probe weights (pass B) or key rows.
         auto scan = [&](bool suffix) {
-            const int nk = suffix ? nsuf : npre;
+            // the direction's rows; the scan ends at the last one needed
+            const int r0 = suffix ? kLNCD : 0;
+            int nk = suffix ? nsuf : npre;
+            while (nk > 0 && !sm.need[r0 + nk - 1]) nk--;
             if (nk == 0) return;
             // tokens of the scan: forward a, a + 1, ..; backward b - 1, b - 2, ..
-            int last = suffix ? b : a;     // the farthest candidate end
-            for (int k = 0; k < nk; k++) {
-                const int kr = suffix ? kLNCD + k : k;
-                last = suffix ? min(last, sm.ca[kr]) : max(last, sm.cb[kr]);
-            }
-            const int ntok = suffix ? b - last : last - a;
+            auto end_of = [&](int k) { return suffix ? b - sm.ca[r0 + k] : sm.cb[r0 + k] - a; };
+            const int ntok = end_of(nk - 1);
             float2 Mt0[CH / 2], Mt1[CH / 2], Mc0[CH / 2], Mc1[CH / 2];
             float Zt0 = 0.f, Zt1 = 0.f, Zc0 = 0.f, Zc1 = 0.f;
 #pragma unroll
@@ -801,11 +926,11 @@ __global__ void __launch_bounds__(kLT, 1) long_eval_kernel(LongArgs A) {
                     int tlo, m;
                     chunk_rows(c0, tlo, m);
                     unsigned char *dst = sm.ring[buf];
-                    constexpr int RB = DH * (int)sizeof(Tin);             // bytes of a K or V row
+                    constexpr int RB = S::RB;
                     const char *vsrc = reinterpret_cast<const char *>(Vl + (size_t)tlo * DH);
                     for (int q = tid; q < m * RB / 16; q += kLT) cp_async16(dst + 16 * q, vsrc + 16 * q, true);
                     unsigned char *dst2 = dst + kLChunk * RB;
-                    if (A.Eg) {
+                    if constexpr (EG) {
                         const char *esrc = reinterpret_cast<const char *>(A.Eg + ((size_t)lg * A.Nc + (tlo - A.cs)) * kLPP);
                         for (int q = tid; q < m * kLPP * 8 / 16; q += kLT) cp_async16(dst2 + 16 * q, esrc + 16 * q, true);
                     } else {
@@ -815,8 +940,11 @@ __global__ void __launch_bounds__(kLT, 1) long_eval_kernel(LongArgs A) {
                 }
                 cp_async_commit();
             };
-            int kk = 0, fold = 0;
-            bool badt = false;
+            // The sums are folded every kLFold tokens and at every row's end, also of
+            // rows not needed now, so that a row's bits do not depend on which
+            // others are evaluated.
+            int kk = 0, kend = end_of(0), next_fold = kLFold;
+            unsigned ebits = 0u;   // largest probe-weight bits: weights are >= 0, non-finite ones on top
             issue(0, 0);
             for (int c0 = 0, buf = 0; c0 < ntok; c0 += kLChunk, buf ^= 1) {
                 issue(c0 + kLChunk, buf ^ 1);
@@ -824,64 +952,66 @@ __global__ void __launch_bounds__(kLT, 1) long_eval_kernel(LongArgs A) {
                 __syncthreads();
                 int tlo, m;
                 chunk_rows(c0, tlo, m);
-                const Tin *vrow0 = reinterpret_cast<const Tin *>(sm.ring[buf]);
-                const unsigned char *aux = sm.ring[buf] + kLChunk * DH * (int)sizeof(Tin);
-                for (int i = 0; i < m; i++) {
-                    const int r = suffix ? m - 1 - i : i;   // row of the scan's token c0 + i
-                    float e0, e1;
-                    if (A.Eg) {
-                        const float2 e = reinterpret_cast<const float2 *>(aux)[r * kLPP + pp];
-                        e0 = has0 ? e.x : 0.f;
-                        e1 = has1 ? e.y : 0.f;
-                    } else {
-                        const Tin *krow = reinterpret_cast<const Tin *>(aux) + (size_t)r * DH;
-                        float2 ya = make_float2(0.f, 0.f), yb = ya;
+                const Tin *vrow0 = reinterpret_cast<const Tin *>(sm.ring[buf]) + 4 * c;
+                const unsigned char *aux = sm.ring[buf] + kLChunk * S::RB;
+                for (int i = 0; i < m;) {
+                    const int lim = max(i + 1, min(m, min(next_fold, kend) - c0));
+#pragma unroll 2
+                    for (; i < lim; i++) {
+                        const int r = suffix ? m - 1 - i : i;   // row of the scan's token c0 + i
+                        float e0, e1;
+                        if constexpr (EG) {   // zero for probes past W
+                            const float2 e = reinterpret_cast<const float2 *>(aux)[r * kLPP + pp];
+                            e0 = e.x;
+                            e1 = e.y;
+                        } else {
+                            const Tin *krow = reinterpret_cast<const Tin *>(aux) + (size_t)r * DH;
+                            float2 ya = make_float2(0.f, 0.f), yb = ya;
+#pragma unroll
+                            for (int gi = 0; gi < NG; gi++) {
+                                const float4 kv = lld4(krow + 4 * c + 32 * gi);
+                                const float2 ka = make_float2(kv.x, kv.y), kb = make_float2(kv.z, kv.w);
+                                ya = ffma2(qk0[2 * gi], ka, ya); ya = ffma2(qk0[2 * gi + 1], kb, ya);
+                                yb = ffma2(qk1[2 * gi], ka, yb); yb = ffma2(qk1[2 * gi + 1], kb, yb);
+                            }
+                            float y0 = ya.x + ya.y, y1 = yb.x + yb.y;
+#pragma unroll
+                            for (int o = kLPPW; o < 32; o <<= 1) {
+                                y0 += __shfl_xor_sync(0xffffffffu, y0, o);
+                                y1 += __shfl_xor_sync(0xffffffffu, y1, o);
+                            }
+                            e0 = has0 ? expf(y0 * inv_sqrt_d - mu0) : 0.f;
+                            e1 = has1 ? expf(y1 * inv_sqrt_d - mu1) : 0.f;
+                        }
+                        ebits = max(ebits, max(__float_as_uint(e0), __float_as_uint(e1)));
+                        const float2 ee0 = make_float2(e0, e0), ee1 = make_float2(e1, e1);
+                        Zc0 += e0;
+                        Zc1 += e1;
+                        const Tin *vrow = vrow0 + r * DH;
 #pragma unroll
                         for (int gi = 0; gi < NG; gi++) {
-                            const float4 kv = lld4(krow + 4 * c + 32 * gi);
-                            const float2 ka = make_float2(kv.x, kv.y), kb = make_float2(kv.z, kv.w);
-                            ya = ffma2(qa0[2 * gi], ka, ya); ya = ffma2(qa0[2 * gi + 1], kb, ya);
-                            yb = ffma2(qa1[2 * gi], ka, yb); yb = ffma2(qa1[2 * gi + 1], kb, yb);
+                            const float4 x = lld4(vrow + 32 * gi);
+                            const float2 va = make_float2(x.x, x.y), vb = make_float2(x.z, x.w);
+                            Mc0[2 * gi] = ffma2(ee0, va, Mc0[2 * gi]);
+                            Mc0[2 * gi + 1] = ffma2(ee0, vb, Mc0[2 * gi + 1]);
+                            Mc1[2 * gi] = ffma2(ee1, va, Mc1[2 * gi]);
+                            Mc1[2 * gi + 1] = ffma2(ee1, vb, Mc1[2 * gi + 1]);
                         }
-                        float y0 = ya.x + ya.y, y1 = yb.x + yb.y;
-#pragma unroll
-                        for (int o = kLPPW; o < 32; o <<= 1) {
-                            y0 += __shfl_xor_sync(0xffffffffu, y0, o);
-                            y1 += __shfl_xor_sync(0xffffffffu, y1, o);
-                        }
-                        e0 = has0 ? expf(y0 * inv_sqrt_d - mu0) : 0.f;
-                        e1 = has1 ? expf(y1 * inv_sqrt_d - mu1) : 0.f;
                     }
-                    badt |= !isfinite(e0) || !isfinite(e1);
-                    const float2 ee0 = make_float2(e0, e0), ee1 = make_float2(e1, e1);
-                    Zc0 += e0;
-                    Zc1 += e1;
-                    const Tin *vrow = vrow0 + (size_t)r * DH;
-#pragma unroll
-                    for (int gi = 0; gi < NG; gi++) {
-                        const float4 x = lld4(vrow + 4 * c + 32 * gi);
-                        const float2 va = make_float2(x.x, x.y), vb = make_float2(x.z, x.w);
-                        Mc0[2 * gi] = ffma2(ee0, va, Mc0[2 * gi]);
-                        Mc0[2 * gi + 1] = ffma2(ee0, vb, Mc0[2 * gi + 1]);
-                        Mc1[2 * gi] = ffma2(ee1, va, Mc1[2 * gi]);
-                        Mc1[2 * gi + 1] = ffma2(ee1, vb, Mc1[2 * gi + 1]);
-                    }
-                    if (++fold == kLFold) { fold_in(); fold = 0; }
-                    // candidates whose far end is this token
-                    const int t = suffix ? b - 1 - (c0 + i) : a + c0 + i;
-                    while (kk < nk) {
-                        const int kr = suffix ? kLNCD + kk : kk;
-                        if ((suffix ? sm.ca[kr] : sm.cb[kr] - 1) != t) break;
+                    const int done = c0 + i;
+                    if (done == next_fold || done == kend) {
                         fold_in();
-                        fold = 0;
-                        evaluate(kr, Zt0, Zt1, Mt0, Mt1);
-                        kk++;
+                        next_fold = done + kLFold;
+                    }
+                    while (done == kend) {
+                        if (sm.need[r0 + kk]) evaluate(r0 + kk, Zt0, Zt1, Mt0, Mt1);
+                        kend = ++kk < nk ? end_of(kk) : INT_MAX;
                     }
                 }
                 __syncthreads();   // the buffer is refilled by the next issue
             }
             cp_async_wait<0>();
-            if (badt) sm.bad = 1;
+            if (ebits >= 0x7f800000u) sm.bad = 1;
         };
         scan(false);
         scan(true);
@@ -890,6 +1020,7 @@ __global__ void __launch_bounds__(kLT, 1) long_eval_kernel(LongArgs A) {
         const float invW = 1.0f / (float)A.W;
         for (int q = tid; q < npre + nsuf; q += kLT) {
             const int k = q < npre ? q : kLNCD + (q - npre);
+            if (!sm.need[k]) continue;
             float d = 0.f, pw = 0.f;
 #pragma unroll
             for (int w = 0; w < kLNW; w++) { d += sm.redD[k][w]; pw += sm.redP[k][w]; }
@@ -897,6 +1028,55 @@ __global__ void __launch_bounds__(kLT, 1) long_eval_kernel(LongArgs A) {
             sm.candP[k] = pw * invW;
         }
         __syncthreads();
+        // G_bin of a cut is ((D - D_L) - D_R) + lambda_kappa kh with D_L, D_R >= 0,
+        // so D + lambda_kappa kh, and (D - D_L) + lambda_kappa kh once D_L is known,
+        // bound it, also as rounded (every operation is monotone).  A cut whose
+        // bound is below G_bin of stage 0's cut cannot be the best one; the
+        // extraction's sides cannot matter when that G_bin reaches D.
+        if (warp == 0) {
+            if (tid == 0) {
+                int pe = a, ssn = b;
+                for (int q = 0; q < npre; q++)
+                    if (sm.need[q]) { pe = max(pe, sm.cb[q]); w_len += sm.cb[q] - a; w_eval++; }
+                for (int q = kLNCD; q < kLNCD + nsuf; q++)
+                    if (sm.need[q]) { ssn = min(ssn, sm.ca[q]); w_len += b - sm.ca[q]; w_eval++; }
+                w_scan += (pe - a) + (b - ssn);
+            }
+            const int k1 = sm.k1, ncut = sm.ncut;
+            const bool decide = cands && !sm.forced && !sm.bad && stage < 2;
+            const float DI = root ? sm.candD[sm.whole] : A.nd_D[gv];
+            const int i = lane < ncut ? lane : 0;
+            unsigned rest = 0u;     // cuts whose sides are evaluated next
+            bool ext = false;
+            __syncwarp();
+            for (int q = lane; q < 2 * kLNCD; q += 32) sm.need[q] = 0;
+            __syncwarp();
+            if (decide) {
+                const float DL1 = sm.pidx[k1] >= 0 ? sm.candD[sm.pidx[k1]] : 0.f;
+                const float DR1 = sm.sidx[k1] >= 0 ? sm.candD[sm.sidx[k1]] : 0.f;
+                const float best1 = fmaf(A.lam_kappa, sm.kh[k1], (DI - DL1) - DR1);
+                bool need = stage == 0 ? lane < ncut && lane != k1 : ((sm.alive >> lane) & 1u) && lane != k1;
+                const float DL = stage == 1 && sm.pidx[i] >= 0 ? sm.candD[sm.pidx[i]] : 0.f;
+                if (need && A.prune) need = !(fmaf(A.lam_kappa, sm.kh[i], DI - DL) < best1);
+                rest = __ballot_sync(FULL, need);
+                ext = stage == 0 ? !(A.prune && best1 >= DI) : sm.extn != 0;
+                __syncwarp();
+                // stage 1's scan: the prefixes (rows already evaluated are evaluated
+                // again with the same bits); stage 2's: the suffixes
+                const int row = need ? (stage == 0 ? sm.pidx[i] : sm.sidx[i]) : -1;
+                const int erow = ext ? (stage == 0 ? sm.eL : sm.eR) : -1;
+                if (row >= 0) sm.need[row] = 1;
+                if (lane == 0 && erow >= 0) sm.need[erow] = 1;
+                if (lane == 0) {
+                    sm.alive = rest | 1u << k1;
+                    sm.extn = ext;
+                }
+            }
+            if (lane == 0) sm.more = rest != 0u || ext;
+        }
+        __syncthreads();
+        if (!sm.more) break;
+        }   // stages
         if (warp == 0) {
             LongRes rs;
             rs.nch = 0;
@@ -945,12 +1125,10 @@ __global__ void __launch_bounds__(kLT, 1) long_eval_kernel(LongArgs A) {
                     // binary cut: lane q evaluates cut q; max G_bin, ties -> smallest xi
                     float best = -INFINITY;
                     int bq = 0x7fffffff;
-                    if (lane < ncut) {
-                        const int xi = sm.cut[lane];
+                    if ((sm.alive >> lane) & 1u) {   // the cuts that no bound ruled out
                         const float DL = sm.pidx[lane] >= 0 ? sm.candD[sm.pidx[lane]] : 0.f;
                         const float DR = sm.sidx[lane] >= 0 ? sm.candD[sm.sidx[lane]] : 0.f;
-                        const float kh = (float)(A.kappa[xi - 1] - sm.kmin) * sm.krange;
-                        best = ((DI - DL) - DR) + A.lam_kappa * kh;
+                        best = fmaf(A.lam_kappa, sm.kh[lane], (DI - DL) - DR);
                         bq = lane;
                     }
 #pragma unroll
@@ -966,12 +1144,13 @@ __global__ void __launch_bounds__(kLT, 1) long_eval_kernel(LongArgs A) {
                         bL = sm.pidx[bq] >= 0 ? sm.candD[sm.pidx[bq]] : 0.f;
                         bR = sm.sidx[bq] >= 0 ? sm.candD[sm.sidx[bq]] : 0.f;
                     }
-                    // extraction at p*
+                    // extraction at p* (its D are read only where they were evaluated)
+                    const bool ext = sm.extn != 0;
                     int ea[3], eb[3], ne = 0;
                     float eD[3];
-                    if (ps > a) { ea[ne] = a; eb[ne] = ps; eD[ne] = ps - a >= 2 ? sm.candD[sm.eL] : 0.f; ne++; }
+                    if (ps > a) { ea[ne] = a; eb[ne] = ps; eD[ne] = ext && ps - a >= 2 ? sm.candD[sm.eL] : 0.f; ne++; }
                     ea[ne] = ps; eb[ne] = ps + 1; eD[ne] = 0.f; ne++;
-                    if (ps + 1 < b) { ea[ne] = ps + 1; eb[ne] = b; eD[ne] = b - ps - 1 >= 2 ? sm.candD[sm.eR] : 0.f; ne++; }
+                    if (ps + 1 < b) { ea[ne] = ps + 1; eb[ne] = b; eD[ne] = ext && b - ps - 1 >= 2 ? sm.candD[sm.eR] : 0.f; ne++; }
                     float gext = DI;
                     for (int q = 0; q < ne; q++) gext -= eD[q];
                     if (bxi < 0) {   // only reachable with non-finite gains
@@ -980,7 +1159,7 @@ __global__ void __launch_bounds__(kLT, 1) long_eval_kernel(LongArgs A) {
                         bR = sm.sidx[0] >= 0 ? sm.candD[sm.sidx[0]] : 0.f;
                     }
                     const float rho_ext = ne == 3 ? 0.5f * gext : gext;   // G_ext / (|children| - 1)
-                    if (forced || rho_ext > best) {
+                    if (forced || (ext && rho_ext > best)) {
                         nch = ne;
                         for (int q = 0; q < ne; q++) { rs.ca[q] = ea[q]; rs.cb[q] = eb[q]; rs.cD[q] = eD[q]; }
                     } else {
@@ -1006,12 +1185,9 @@ __global__ void __launch_bounds__(kLT, 1) long_eval_kernel(LongArgs A) {
             }
             if (lane == 0) {
                 A.res[it] = rs;
-                int pe = a, ssn = b, len = 0;
-                for (int q = 0; q < npre; q++) { pe = max(pe, sm.cb[q]); len += sm.cb[q] - sm.ca[q]; }
-                for (int q = 0; q < nsuf; q++) { ssn = min(ssn, sm.ca[kLNCD + q]); len += sm.cb[kLNCD + q] - sm.ca[kLNCD + q]; }
-                atomicAdd(&A.work[0], (unsigned long long)((pe - a) + (b - ssn)));
-                atomicAdd(&A.work[1], (unsigned long long)(npre + nsuf));
-                atomicAdd(&A.work[2], (unsigned long long)len);
+                atomicAdd(&A.work[0], w_scan);
+                atomicAdd(&A.work[1], w_eval);
+                atomicAdd(&A.work[2], w_len);
                 atomicAdd(&A.work[3], 1ull);
             }
         }
@@ -1106,30 +1282,29 @@ __global__ void long_commit_kernel(LongArgs A) {
     }
 }
 
-// CTAs of long_eval resident per SM (its shared memory set as at launch)
-template <int DH, typename Tin>
-int eval_occupancy() {
-    using S = LongSmem<DH>;
-    if (cudaFuncSetAttribute(long_eval_kernel<DH, Tin>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(S)) != cudaSuccess)
-        return 1;
-    int n = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, long_eval_kernel<DH, Tin>, kLT, sizeof(S)) != cudaSuccess)
-        return 1;
-    return n;
-}
-
-template <int DH, typename Tin>
-cudaError_t launch_eval(Ctx &c, const LongArgs &A, unsigned grid, cudaStream_t s) {
-    using S = LongSmem<DH>;
+// One resident wave: items are taken dynamically.
+template <int DH, typename Tin, bool EG>
+cudaError_t launch_eval(Ctx &c, const LongArgs &A, unsigned items, cudaStream_t s) {
+    using S = LongSmem<DH, Tin>;
     static_assert(sizeof(S) <= 227 * 1024, "long-unit kernel shared memory above the per-CTA limit");
+    static_assert(!EG || 2 * (sizeof(S) + 1024) <= 228 * 1024, "two CTAs per SM");
     const size_t sm = sizeof(S);
-    cudaError_t e = cudaFuncSetAttribute(long_eval_kernel<DH, Tin>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(long_eval_kernel<DH, Tin, EG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sm);
+    int occ = 1;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, long_eval_kernel<DH, Tin, EG>, kLT, sm);
     if (e != cudaSuccess) return e;
-    long_eval_kernel<DH, Tin><<<grid, kLT, sm, s>>>(A);
+    const unsigned grid = (unsigned)std::min<int64_t>((int64_t)c.num_sms * std::max(occ, 1), (int64_t)items);
+    long_eval_kernel<DH, Tin, EG><<<grid, kLT, sm, s>>>(A);
     c.launches += 1;
     return cudaGetLastError();
+}
+
+template <int DH>
+cudaError_t launch_eval_d(Ctx &c, const LongArgs &A, unsigned items, cudaStream_t s) {
+    if (c.p.dtype != GKV_BF16) return launch_eval<DH, float, false>(c, A, items, s);
+    return A.Eg ? launch_eval<DH, __nv_bfloat16, true>(c, A, items, s)
+                : launch_eval<DH, __nv_bfloat16, false>(c, A, items, s);
 }
 
 __global__ void long_units_kernel(const int32_t *long_slots, int n_long, int lg0, int nlg, int J, int32_t *out) {
@@ -1175,6 +1350,7 @@ cudaError_t launch_long_level(Ctx &c, const void *K, const void *V, const void *
     A.inv_sqrt_d = (float)(1.0 / sqrt((double)p.d));
     A.lamZ = (float)p.lambda_Z; A.lamM = (float)p.lambda_M; A.eps = (float)p.eps;
     A.lam_kappa = (float)p.lambda_kappa; A.base_frac = (float)p.base_frac;
+    A.prune = p.lambda_Z >= 0.0 && p.lambda_M >= 0.0;
     A.fresh = fresh; A.root_only = root_only; A.tau = tau;
     A.list = list; A.n_list = n_list; A.lg0 = lg0; A.nlg = nlg;
     A.it_gv = w.long_gv; A.it_uid = w.long_uid; A.it_kin = w.long_kin; A.it_ufl = w.long_ufl;
@@ -1204,14 +1380,7 @@ cudaError_t launch_long_level(Ctx &c, const void *K, const void *V, const void *
     for (int q = 0; q <= kUnitClasses; q++) cnt[q] = (unsigned)std::min<int64_t>((int64_t)cnt[q], w.long_cap);
     if (n_items_host) *n_items_host = cnt[0] + cnt[1] + cnt[2] + cnt[3];
     if (cnt[0] > 0) {
-        // one resident wave: items are taken dynamically
-        int occ = 1;
-        if (p.d == 128) occ = p.dtype == GKV_BF16 ? eval_occupancy<128, __nv_bfloat16>() : eval_occupancy<128, float>();
-        else occ = p.dtype == GKV_BF16 ? eval_occupancy<64, __nv_bfloat16>() : eval_occupancy<64, float>();
-        const unsigned grid = (unsigned)std::min<int64_t>((int64_t)c.num_sms * std::max(occ, 1), (int64_t)cnt[0]);
-        e = p.dtype == GKV_BF16
-                ? (p.d == 128 ? launch_eval<128, __nv_bfloat16>(c, A, grid, s) : launch_eval<64, __nv_bfloat16>(c, A, grid, s))
-                : (p.d == 128 ? launch_eval<128, float>(c, A, grid, s) : launch_eval<64, float>(c, A, grid, s));
+        e = p.d == 128 ? launch_eval_d<128>(c, A, cnt[0], s) : launch_eval_d<64>(c, A, cnt[0], s);
         if (e != cudaSuccess) return e;
         long_commit_kernel<<<(unsigned)n_units, 32, 0, s>>>(A);
         c.launches += 1;

@@ -20,6 +20,8 @@ bit-exact, prototypes within the dtype's tolerance, no near-tie exemption.
                512-token regions) at 16384 tokens with its drawn slots, at 4x,
                32x and 128x; the oracle's trees are built once, pooled
 """
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -94,3 +96,24 @@ def test_skew_slice_matches_the_oracle(skew_case, ratio):
     rep = P.compare(g, o, torch.bfloat16)
     assert g["E"] == len(o["cache"]["pos"])
     print("skew", ratio, rep)
+
+
+@pytest.mark.parametrize("lam,k_cand", [(0.0, 16), (0.002, 16), (1.0, 16), (0.002, 1), (0.05, 0)])
+@pytest.mark.parametrize("dtype,d,gq,W", [("bf16", 64, 4, 8), ("bf16", 128, 8, 40), ("fp32", 128, 2, 8)])
+def test_long_cut_bounds_match_the_oracle(dtype, d, gq, W, lam, k_cand):
+    # Which cuts of a long node are left out depends on lambda_kappa (none at 0, some at
+    # 0.002, nearly all at 1) and on the number of cuts; the lengths lie at the edges of the
+    # partial sums (32 tokens) and of the segment sums (8 warps x 4 tokens).  The inputs cover
+    # the three ways the probe weights are formed.
+    lens = [129, 3, 160, 161, 255, 40, 289, 513]
+    w = dataclasses.replace(synth.WORKLOADS["small"], L=1, G=1, Hq=gq, d=d)
+    x = synth.make_inputs(w, T=sum(lens) + 32, W=W)
+    K, V, Q = x.K, x.V, x.Q
+    if dtype == "fp32":
+        K, V, Q = K.float(), V.float(), Q.float()
+    slots = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    B = K.shape[2] // 4
+    kw = dict(slot_starts=slots, lambda_kappa=lam, k_cand=k_cand)
+    g = P.run_gpu(K, V, Q, B, w.rope_base, **kw)
+    o = P.run_oracle(K, V, Q, B, w.rope_base, **kw)
+    P.compare(g, o, torch.float32 if dtype == "fp32" else torch.bfloat16)
