@@ -347,8 +347,9 @@ struct LongSmem {
     unsigned rk[kLNW], fk[kLNW];     //           largest token value, floor score (keys)
     int rp[kLNW], fp[kLNW];          //           and their positions
     int bad;
-    unsigned alive;                  // cuts whose both sides are evaluated
-    int extn;                        // the extraction's sides are evaluated
+    unsigned pmask, alive;           // cuts whose prefix, whose both sides are evaluated
+    unsigned rest;                   // cuts under evaluation
+    int extP, extn, extr;            // the extraction's left side is evaluated; both are; under evaluation
     int more;                        // rows are left to evaluate
 };
 
@@ -361,7 +362,7 @@ __device__ __forceinline__ unsigned fokey(float x) {
 // Bound by the fp32 FMAs of the probe scan (2 W d per token) and by latency, so
 // two CTAs share an SM: the staging ring's bytes hold the segment partials and
 // the curvature candidates before the scans, and the queries are read back for
-// each evaluated row.  Skew 64K at 32x, all 16 launches: 161 -> 77 ms with the
+// each evaluated row.  Skew 64K at 32x, all 16 launches: 161 -> 60 ms with the
 // bound (half of the scanned tokens, 3 rows of about 36 for most nodes), the
 // second CTA, tokens loaded four at a time by the segment sums, scans in
 // stretches between fold points without a test per token, and the top-K drawn
@@ -555,16 +556,24 @@ __global__ void __launch_bounds__(kLT, EG ? 2 : 1) long_eval_kernel(LongArgs A) 
                 if (root) { sm.ca[npre0] = a; sm.cb[npre0] = b; sm.need[npre0] = 1; }
                 sm.npre = npre; sm.nsuf = nsuf; sm.eL = eL; sm.eR = eR; sm.whole = root ? npre0 : -1;
                 sm.ncut = ncut; sm.pstar = ps; sm.forced = forced; sm.k1 = k1;
-                // evaluated first: both sides of the cut of largest reward, or of a
-                // forced extraction; a fresh root's own
-                if (cands) {
-                    const int r0 = forced ? eL : sm.pidx[k1], r1 = forced ? eR : sm.sidx[k1];
-                    if (r0 >= 0) sm.need[r0] = 1;
-                    if (r1 >= 0) sm.need[r1] = 1;
-                }
-                sm.alive = cands && !forced ? 1u << k1 : 0u;
-                sm.extn = forced;
-                sm.more = 0;
+                sm.alive = 0u;
+                sm.extn = 0;
+            }
+            // Stage 0 evaluates prefixes: of the cut of largest reward, of the cuts
+            // that D alone would not rule out against that reward (all of a root's,
+            // whose D is not known yet: a row costs far less than a second scan),
+            // and the forced extraction's; a fresh root's own row comes with them.
+            const float DI0 = root || !A.prune ? INFINITY : A.nd_D[gv];
+            const float rew1 = __shfl_sync(FULL, A.lam_kappa * kh, k1);
+            const bool first = cands && !forced && lane < ncut &&
+                               (lane == k1 || !(fmaf(A.lam_kappa, kh, DI0) < rew1));
+            const unsigned fm = __ballot_sync(FULL, first);
+            const bool fext = cands && (forced || !(rew1 >= DI0));
+            if (first && pv) sm.need[prow] = 1;
+            if (lane == 0) {
+                if (fext && eL >= 0) sm.need[eL] = 1;
+                sm.rest = fm;
+                sm.extr = fext;
             }
             // segment boundaries: a, b, the cuts, p*, p* + 1
             const bool ps_in = ps > a && !__any_sync(FULL, xi == ps), er_in = er < b && !__any_sync(FULL, xi == er);
@@ -736,8 +745,9 @@ __global__ void __launch_bounds__(kLT, EG ? 2 : 1) long_eval_kernel(LongArgs A) 
         __syncthreads();
         const int npre = sm.npre, nsuf = sm.nsuf;
         unsigned long long w_scan = 0, w_eval = 0, w_len = 0;   // work counters (thread 0)
-        // Stages: 0 the rows chosen above; 1 the prefixes of the cuts that stage 0
-        // does not rule out, 2 their suffixes.
+        // Stages, one scan each: 0 the prefixes chosen above, 1 the suffixes of those
+        // that may still be the best cut; then, rarely, 2 the prefixes and 3 the
+        // suffixes of cuts that the best one found does not rule out.
         for (int stage = 0;; stage++) {
         // ---- phase C: candidate prototypes from their segments (warp per candidate)
         auto seg_of = [&](int pos) {   // index of the boundary at pos (every candidate end is one)
@@ -1031,7 +1041,7 @@ __global__ void __launch_bounds__(kLT, EG ? 2 : 1) long_eval_kernel(LongArgs A) 
         // G_bin of a cut is ((D - D_L) - D_R) + lambda_kappa kh with D_L, D_R >= 0,
         // so D + lambda_kappa kh, and (D - D_L) + lambda_kappa kh once D_L is known,
         // bound it, also as rounded (every operation is monotone).  A cut whose
-        // bound is below G_bin of stage 0's cut cannot be the best one; the
+        // bound is below the best G_bin evaluated cannot be the best one; the
         // extraction's sides cannot matter when that G_bin reaches D.
         if (warp == 0) {
             if (tid == 0) {
@@ -1043,36 +1053,70 @@ __global__ void __launch_bounds__(kLT, EG ? 2 : 1) long_eval_kernel(LongArgs A) 
                 w_scan += (pe - a) + (b - ssn);
             }
             const int k1 = sm.k1, ncut = sm.ncut;
-            const bool decide = cands && !sm.forced && !sm.bad && stage < 2;
+            const bool decide = cands && !sm.bad && stage < 3;
             const float DI = root ? sm.candD[sm.whole] : A.nd_D[gv];
             const int i = lane < ncut ? lane : 0;
-            unsigned rest = 0u;     // cuts whose sides are evaluated next
-            bool ext = false;
+            const unsigned rest = sm.rest;
+            const bool extr = sm.extr != 0, mine = (rest >> lane) & 1u;
+            unsigned pmask = stage == 0 ? rest : stage == 2 ? sm.pmask | rest : sm.pmask;
+            unsigned alive = sm.alive, next = 0u;
+            bool extP = stage == 0 ? extr : stage == 2 ? sm.extP || extr : sm.extP != 0;
+            bool extn = sm.extn != 0, next_ext = false;
             __syncwarp();
             for (int q = lane; q < 2 * kLNCD; q += 32) sm.need[q] = 0;
+            if (stage == 1 || stage == 3) {
+                alive |= rest;
+                extn |= extr;
+            }
+            const bool known = (pmask >> lane) & 1u;
+            const float DL = known && sm.pidx[i] >= 0 ? sm.candD[sm.pidx[i]] : 0.f;
+            const float ub = fmaf(A.lam_kappa, sm.kh[i], DI - DL);
+            // the best G_bin of the cuts evaluated
+            float lb = -INFINITY;
+            if ((alive >> lane) & 1u) {
+                const float DR = sm.sidx[i] >= 0 ? sm.candD[sm.sidx[i]] : 0.f;
+                lb = fmaf(A.lam_kappa, sm.kh[i], (DI - DL) - DR);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) lb = fmaxf(lb, __shfl_xor_sync(FULL, lb, o));
+            if (decide && sm.forced) {
+                next_ext = stage == 0;
+            } else if (decide) {
+                bool q;
+                if (stage == 0) {
+                    // the suffixes that are likely needed, in one scan: bounds within D of
+                    // the first cut's (what its own suffix may take off); the check
+                    // after stage 1 is the exact one
+                    const float ub1 = __shfl_sync(FULL, ub, k1);
+                    q = mine && (lane == k1 || !A.prune || !(ub < ub1 - DI));
+                    next_ext = extr && !(A.prune && A.lam_kappa * sm.kh[k1] >= DI);
+                } else if (stage == 2) {
+                    q = mine && (!A.prune || !(ub < lb));
+                    next_ext = extr;
+                } else {
+                    q = lane < ncut && !((alive >> lane) & 1u) && (!A.prune || !(ub < lb));
+                    next_ext = !extn && !(A.prune && lb >= DI);
+                }
+                next = __ballot_sync(FULL, q);
+            }
             __syncwarp();
-            if (decide) {
-                const float DL1 = sm.pidx[k1] >= 0 ? sm.candD[sm.pidx[k1]] : 0.f;
-                const float DR1 = sm.sidx[k1] >= 0 ? sm.candD[sm.sidx[k1]] : 0.f;
-                const float best1 = fmaf(A.lam_kappa, sm.kh[k1], (DI - DL1) - DR1);
-                bool need = stage == 0 ? lane < ncut && lane != k1 : ((sm.alive >> lane) & 1u) && lane != k1;
-                const float DL = stage == 1 && sm.pidx[i] >= 0 ? sm.candD[sm.pidx[i]] : 0.f;
-                if (need && A.prune) need = !(fmaf(A.lam_kappa, sm.kh[i], DI - DL) < best1);
-                rest = __ballot_sync(FULL, need);
-                ext = stage == 0 ? !(A.prune && best1 >= DI) : sm.extn != 0;
-                __syncwarp();
-                // stage 1's scan: the prefixes (rows already evaluated are evaluated
-                // again with the same bits); stage 2's: the suffixes
-                const int row = need ? (stage == 0 ? sm.pidx[i] : sm.sidx[i]) : -1;
-                const int erow = ext ? (stage == 0 ? sm.eL : sm.eR) : -1;
+            {
+                const bool pre = stage == 1;   // the next stage's scan
+                const bool todo = ((next >> lane) & 1u) && !(pre && known);
+                const int row = todo ? (pre ? sm.pidx[i] : sm.sidx[i]) : -1;
+                const int erow = next_ext && !(pre && extP) ? (pre ? sm.eL : sm.eR) : -1;
                 if (row >= 0) sm.need[row] = 1;
-                if (lane == 0 && erow >= 0) sm.need[erow] = 1;
                 if (lane == 0) {
-                    sm.alive = rest | 1u << k1;
-                    sm.extn = ext;
+                    if (erow >= 0) sm.need[erow] = 1;
+                    sm.pmask = pmask;
+                    sm.alive = alive;
+                    sm.rest = next;
+                    sm.extP = extP;
+                    sm.extn = extn;
+                    sm.extr = next_ext;
+                    sm.more = next != 0u || next_ext;
                 }
             }
-            if (lane == 0) sm.more = rest != 0u || ext;
         }
         __syncthreads();
         if (!sm.more) break;
