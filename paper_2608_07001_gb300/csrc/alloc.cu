@@ -580,6 +580,96 @@ __global__ void alloc_final_kernel(AllocArgs A) {
     }
 }
 
+// The whole selection of a small request in one block: the three digits'
+// histograms and picks in shared memory, in place of seven launches of a few
+// microseconds each (shared budget only).
+__global__ void __launch_bounds__(1024) alloc_select_kernel(AllocArgs A) {
+    __shared__ unsigned int sh[2048];
+    __shared__ unsigned int wsum[32];
+    __shared__ unsigned long long s_above;
+    __shared__ unsigned int s_prefix, s_total;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned long long B = (unsigned long long)A.B_free;
+    const int n_ops = (int)*A.n_ops, n_units = (int)A.n_units;
+    if (tid == 0) {
+        s_above = 0;
+        s_prefix = s_total = 0;
+    }
+    __syncthreads();
+    uint32_t mask = 0;
+    bool all = false;
+    for (int ps = 0; ps < 3 && !all; ps++) {
+        const int shift = ps == 0 ? 21 : ps == 1 ? 10 : 0, nbits = ps == 2 ? 10 : 11, nbin = 1 << nbits;
+        for (int b = tid; b < 2048; b += 1024) sh[b] = 0;
+        __syncthreads();
+        const uint32_t prefix = s_prefix;
+        unsigned int tot = 0;
+        for (int i0 = tid & ~31; i0 < n_units + n_ops; i0 += 1024) {
+            const int i = i0 + lane;
+            const bool in = i < n_units + n_ops;
+            uint32_t key = 0;
+            int cost = 0;
+            int64_t v;
+            if (in) op_key(A, i, key, cost, v);
+            tot += cost;
+            const int bin = in && (key & mask) == prefix ? (int)((key >> shift) & (nbin - 1)) : -1;
+            const unsigned grp = __match_any_sync(0xffffffffu, bin);
+            const unsigned sum = __reduce_add_sync(grp, (unsigned)cost);
+            if (bin >= 0 && lane == __ffs(grp) - 1) atomicAdd(&sh[bin], sum);
+        }
+        if (ps == 0) {   // total cost of all ops
+            tot = __reduce_add_sync(0xffffffffu, tot);
+            if (lane == 0 && tot) atomicAdd(&s_total, tot);
+        }
+        __syncthreads();
+        all = s_total <= B;
+        if (all) break;   // the same in every thread
+        // thread t owns bins nbin - 1 - 2 t and nbin - 2 - 2 t (as in alloc_scan)
+        const int b0 = nbin - 1 - 2 * tid, b1 = b0 - 1;
+        const unsigned h0 = b0 >= 0 ? sh[b0] : 0u, h1 = b1 >= 0 ? sh[b1] : 0u;
+        const unsigned x = h0 + h1;
+        unsigned incl = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        unsigned long long before = s_above + (incl - x);
+        for (int w = 0; w < warp; w++) before += wsum[w];
+        __syncthreads();
+        if (b0 >= 0 && before <= B && before + h0 > B) {
+            s_prefix |= (uint32_t)b0 << shift;
+            s_above = before;
+        } else if (b1 >= 0 && before + h0 <= B && before + h0 + h1 > B) {
+            s_prefix |= (uint32_t)b1 << shift;
+            s_above = before + h0;
+        }
+        mask |= (uint32_t)(nbin - 1) << shift;
+        __syncthreads();
+    }
+    if (tid < ST_N)
+        A.st[tid] = tid == ST_PREFIX ? s_prefix : tid == ST_ABOVE ? s_above : tid == ST_ALL ? (all ? 1ull : 0ull)
+                  : tid == ST_TOTAL ? s_total : tid == ST_ENDKEY || tid == ST_CROSS ? ~0ull : 0ull;
+}
+
+// What the host reads between tree passes, side by side behind the state words
+// (shared budget only), so that one copy fetches it: each copy to the host's
+// stack is a round trip of its own (options 16x, 15 passes: 7.15 -> 6.17 ms).
+__global__ void pass_report_kernel(unsigned long long *st, const int *count, const float *cut, const unsigned int *n_qual,
+                                   const unsigned long long *pot) {
+    PassReport r;
+    for (int q = 0; q < kUnitClasses + 1; q++) r.count[q] = count[q];
+    r.tau_bits = (uint32_t)st[ST_PREFIX];
+    r.all = st[ST_ALL] != 0;
+    r.cut = *cut;
+    r.n_qual = *n_qual;
+    r.total = st[ST_TOTAL];
+    r.pot = *pot;
+    *reinterpret_cast<PassReport *>(st + ST_N) = r;
+}
+
 __global__ void alloc_init_kernel(unsigned long long *st, unsigned long long *hist, int nseg) {
     const int nst = ST_N * (nseg > 1 ? nseg + 1 : 1);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nst; i += gridDim.x * blockDim.x)
@@ -705,6 +795,15 @@ __global__ void slot_classes_kernel(const int32_t *slots, int J, int32_t *list, 
 
 cudaError_t launch_threshold(Ctx &c, int J, cudaStream_t s) {
     AllocArgs A = make_args(c, J);
+    // One block up to 8192 ops (an Add per unit, at most a Split per two node
+    // slots), eight rounds of it: the seven launches cost 27 us there, a grid's
+    // worth of ops would keep one block longer than that.  pr1 (2000 ops, eight
+    // passes), with the report below in place of seven copies: 1.72 -> 1.31 ms.
+    if (A.nseg == 1 && A.n_units + c.node_cap / 2 <= 8192) {
+        alloc_select_kernel<<<1, 1024, 0, s>>>(A);
+        c.launches += 1;
+        return cudaGetLastError();
+    }
     alloc_init_kernel<<<A.nseg > 1 ? 256 : 1, 256, 0, s>>>(c.w.alloc_state, c.w.hist, A.nseg);
     const int blocks = grid_for(c, A.n_units + c.node_cap / 2);
     const int shifts[3] = {21, 10, 0};
@@ -733,6 +832,15 @@ cudaError_t launch_prune_list(Ctx &c, const int32_t *slots, int J, int32_t *list
                                                                     stride, count, long_list, c.w.pend_pot);
     c.launches += 1;
     return cudaGetLastError();
+}
+
+cudaError_t launch_pass_report(Ctx &c, const int *count, PassReport *host, cudaStream_t s) {
+    static_assert(ST_N * 8 + sizeof(PassReport) <= 16 * 8, "the report fits behind the state words");
+    pass_report_kernel<<<1, 1, 0, s>>>(c.w.alloc_state, count, c.w.pend_cut, c.w.pend_n, c.w.pend_pot);
+    c.launches += 1;
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return cudaMemcpyAsync(host, c.w.alloc_state + ST_N, sizeof(PassReport), cudaMemcpyDeviceToHost, s);
 }
 
 cudaError_t launch_pend_cut(Ctx &c, int J, int m, float *cut, unsigned int *n_qual, cudaStream_t s) {

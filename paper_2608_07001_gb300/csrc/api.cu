@@ -601,34 +601,18 @@ static cudaError_t build_passes(Ctx &c, const void *K, const void *V, const void
     float tau_prev = -INFINITY;   // tau of the previous pass
     cudaError_t e = cudaSuccess;
     for (int it = 0; e == cudaSuccess; it++) {
-        struct {
-            int count[kLongCnt + 1];
-            unsigned long long prefix, all, total, pot;
-            float cut;
-            unsigned int nqual;
-        } h = {{0, 0, 0, 0}, 0, 0, 0, 0, 0.f, 0};
+        gkv::PassReport h = {};
         {
             gkv::StageTimer tm(c, 3, s);
             e = gkv::launch_threshold(c, J, s);
             if (e == cudaSuccess && root_only) e = gkv::launch_pend_cut(c, J, pass_units, w.pend_cut, w.pend_n, s);
             if (e == cudaSuccess) e = gkv::launch_prune_list(c, w.slots, J, w.u_list, w.units_cap, w.dev_int + 2, w.long_list, s);
         }
-        if (e == cudaSuccess) e = cudaMemcpyAsync(h.count, w.dev_int + 2, sizeof h.count, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&h.prefix, w.alloc_state, 2 * sizeof(unsigned long long),
-                                                  cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&h.all, w.alloc_state + 2, sizeof(unsigned long long),
-                                                  cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&h.cut, w.pend_cut, sizeof(float), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&h.nqual, w.pend_n, sizeof(unsigned int), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&h.total, w.alloc_state + 6, sizeof(unsigned long long),
-                                                  cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&h.pot, w.pend_pot, sizeof(unsigned long long),
-                                                  cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = gkv::launch_pass_report(c, w.dev_int + 2, &h, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess || h.count[0] + h.count[1] + h.count[2] + h.count[kLongCnt] == 0) break;
-        uint32_t bits = (uint32_t)h.prefix;
         float tau;
-        memcpy(&tau, &bits, sizeof tau);
+        memcpy(&tau, &h.tau_bits, sizeof tau);
         if (h.all) tau = -INFINITY;
         const float tau_eff = fmaxf(tau, h.cut);
         // everything built so far fits and few units remain: expand them fully at once

@@ -371,6 +371,17 @@ size_t long_res_bytes();
 // out[q nlg + i] = the unit id of long slot long_slots[q] for (l, g) = lg0 + i.
 cudaError_t launch_long_units(Ctx &c, const int32_t *long_slots, int n_long, int lg0, int nlg, int J,
                               int32_t *out, cudaStream_t s);
+// Results of a pass's threshold and list launches.
+struct PassReport {
+    int count[kUnitClasses + 1];   // listed units of each class, long ones last
+    uint32_t tau_bits;
+    uint32_t all;                  // every op built so far fits the budget
+    float cut;                     // bound of the scheduling cut
+    unsigned int n_qual;
+    unsigned long long total, pot; // cost of the ops built, of completing the listed units
+};
+cudaError_t launch_pass_report(Ctx &c, const int *count, PassReport *host, cudaStream_t s);
+
 // Allocation threshold tau over the ops built so far (alloc_state prefix /
 // all-fit flag), and the units whose largest pending key bound reaches
 // max(tau, cut), split by slot length class: class q at list + q stride,

@@ -59,3 +59,16 @@ def test_cut_bounds_match_the_oracle(dtype, d, lam):
     g = P.run_gpu(K, V, Q, B, w.rope_base, lambda_kappa=lam)
     o = P.run_oracle(K, V, Q, B, w.rope_base, lambda_kappa=lam)
     P.compare(g, o, torch.float32 if dtype == "fp32" else torch.bfloat16)
+
+
+@pytest.mark.parametrize("last", [1, 2])   # 8192 ops at most (one block selects them), 8193
+@pytest.mark.parametrize("ratio", [0.5, 3, 60])   # everything fits; splits; not even every Add
+def test_small_selection_matches_the_oracle(last, ratio):
+    lens = [64] * 126 + [last]
+    w = dataclasses.replace(synth.WORKLOADS["small"], L=1, G=1, Hq=1, d=64)
+    x = synth.make_inputs(w, T=sum(lens) + 32, W=8)
+    slots = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    B = int(sum(lens) / ratio) + 32
+    g = P.run_gpu(x.K, x.V, x.Q, B, w.rope_base, slot_starts=slots)
+    o = P.run_oracle(x.K, x.V, x.Q, B, w.rope_base, slot_starts=slots)
+    P.compare(g, o, torch.bfloat16)
