@@ -164,12 +164,18 @@ __global__ void __launch_bounds__(kSeNT) sens_tile_kernel(const __nv_bfloat16 *_
 // One CTA: norms, means over the probes, raw values, their mean, omega.
 __global__ void __launch_bounds__(1024) sens_final_kernel(const float *sumsq, const float *fro, int LG, int U,
                                                           float eps, float *omega) {
-    __shared__ float wsum[32];
+    // the sum over the probes is compensated and the mean's is taken in double:
+    // their rounding would otherwise dominate omega's
+    __shared__ double wsum[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    float part = 0.f;
+    double part = 0.0;
     for (int k = tid; k < LG; k += 1024) {
-        float in = 0.f;
-        for (int u = 0; u < U; u++) in += sqrtf(sumsq[(size_t)k * kSeMaxU + u]);
+        float in = 0.f, comp = 0.f;
+        for (int u = 0; u < U; u++) {
+            const float y = sqrtf(sumsq[(size_t)k * kSeMaxU + u]) - comp, t = in + y;
+            comp = (t - in) - y;
+            in = t;
+        }
         in /= U;
         const float raw = sqrtf(sqrtf(fro[k]) * in);
         omega[k] = raw;
@@ -180,12 +186,12 @@ __global__ void __launch_bounds__(1024) sens_final_kernel(const float *sumsq, co
     if (lane == 0) wsum[warp] = part;
     __syncthreads();
     if (tid == 0) {
-        float s = 0.f;
+        double s = 0.0;
         for (int w = 0; w < 32; w++) s += wsum[w];
         wsum[0] = s / LG;
     }
     __syncthreads();
-    const float mean = wsum[0];
+    const float mean = (float)wsum[0];
     for (int k = tid; k < LG; k += 1024) omega[k] = omega[k] / (mean + eps);
 }
 
