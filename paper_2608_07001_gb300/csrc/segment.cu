@@ -101,8 +101,8 @@ __global__ void seg_norm_kernel(const Tin *V, const float *hidden, SegArgs a, fl
 }
 
 // ---------------------------------------------------------------------------
-// Curvature.  Block = 256 threads = 512 consecutive positions (two adjacent
-// ones per thread) of one segmentation layer.  The trajectory channels are
+// Curvature.  Block = 256 (or 64) threads = 512 (128) consecutive positions (two
+// adjacent ones per thread) of one segmentation layer.  The trajectory channels are
 // staged in chunks of kCurvCC channels, already normalised (hbar = h /
 // max(|h|, eps)), channel-major in shared memory so that the threads of a
 // warp read consecutive rows.  A thread loads the 34 rows around its two
@@ -113,11 +113,14 @@ __global__ void seg_norm_kernel(const Tin *V, const float *hidden, SegArgs a, fl
 // ---------------------------------------------------------------------------
 constexpr int kHalo = 16;                       // largest window
 constexpr int kCurvPP = 2;                      // positions per thread
-constexpr int kCurvPT = 256 * kCurvPP;          // positions per block
-constexpr int kCurvRows = kCurvPT + 2 * kHalo;  // staged rows
-constexpr int kCurvRS = kCurvRows + 2;          // row stride (even: 8-byte row loads)
 constexpr int kCurvCC = 32;                     // channels per stage
-constexpr size_t kCurvSmem = ((size_t)kCurvCC * kCurvRS + kCurvRows) * sizeof(float);
+template <int NT>                               // threads per block
+struct CurvCfg {
+    static constexpr int PT = NT * kCurvPP;         // positions per block
+    static constexpr int ROWS = PT + 2 * kHalo;     // staged rows
+    static constexpr int RS = ROWS + 2;             // row stride (even: 8-byte row loads)
+    static constexpr size_t SMEM = ((size_t)kCurvCC * RS + ROWS) * sizeof(float);
+};
 
 // 8 consecutive trajectory channels c .. c+7 (c % 8 == 0) of row t, or zeros
 // outside [0, T).
@@ -142,17 +145,18 @@ __device__ __forceinline__ void traj_load8(const Tin *V, const float *hidden, co
     for (int j = 0; j < 8; j++) v[j] = x.v[j];
 }
 
-template <typename Tin, bool kDefaultWindows>
-__global__ void __launch_bounds__(256) seg_curv_kernel(const Tin *V, const float *hidden,
+template <typename Tin, bool kDefaultWindows, int NT>
+__global__ void __launch_bounds__(NT) seg_curv_kernel(const Tin *V, const float *hidden,
                                                        SegArgs a, const float *inv_norm,
                                                        double *klw) {
+    constexpr int kCurvPT = CurvCfg<NT>::PT, kCurvRows = CurvCfg<NT>::ROWS, kCurvRS = CurvCfg<NT>::RS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *P = reinterpret_cast<float *>(smem_raw);   // [kCurvCC][kCurvRS] normalised values
     float *inv_s = P + (size_t)kCurvCC * kCurvRS;     // [kCurvRows]
     const int li = blockIdx.y, l = a.layers[li];
     const int i0 = blockIdx.x * kCurvPT, row0 = i0 - kHalo;
     const int tid = threadIdx.x;
-    for (int r = tid; r < kCurvRows; r += 256) {
+    for (int r = tid; r < kCurvRows; r += NT) {
         const int t = row0 + r;
         inv_s[r] = (t >= 0 && t < a.T) ? inv_norm[(size_t)li * a.T + t] : 0.f;
     }
@@ -176,11 +180,11 @@ __global__ void __launch_bounds__(256) seg_curv_kernel(const Tin *V, const float
         const int nq = min(kCurvCC, a.D - c0) >> 3;   // 8-channel chunks in this stage
         __syncthreads();
         // stage: the loads of 4 row chunks are issued before any is stored
-        for (int e0 = tid; e0 < kCurvRows * nq; e0 += 256 * 4) {
+        for (int e0 = tid; e0 < kCurvRows * nq; e0 += NT * 4) {
             float v[4][8];
 #pragma unroll
             for (int u = 0; u < 4; u++) {
-                const int e = e0 + 256 * u;
+                const int e = e0 + NT * u;
                 if (e < kCurvRows * nq) {
                     const int r = e / nq, q = e - r * nq;
                     traj_load8(V, hidden, a, l, li, row0 + r, c0 + 8 * q, v[u]);
@@ -188,7 +192,7 @@ __global__ void __launch_bounds__(256) seg_curv_kernel(const Tin *V, const float
             }
 #pragma unroll
             for (int u = 0; u < 4; u++) {
-                const int e = e0 + 256 * u;
+                const int e = e0 + NT * u;
                 if (e < kCurvRows * nq) {
                     const int r = e / nq, q = e - r * nq;
                     const float sc = inv_s[r];
@@ -404,6 +408,88 @@ __global__ void zsel_dev_kernel(const double *x, int n, const SelState *st, unsi
         dev[i] = dkey(fabs(x[i] - med));
 }
 
+// Both selects of a short input in one block: its keys stay in registers (8
+// per thread at most) and every digit is counted and picked in shared memory,
+// in place of 27 launches of 2 to 5 us.
+constexpr int kSelSmallT = 512, kSelSmallU = 8, kSelSmallB = kSelBins / kSelSmallT;
+__global__ void __launch_bounds__(kSelSmallT) zsel_small_kernel(const double *x, int n, long long rank, SelState *st) {
+    __shared__ unsigned int hist[kSelBins];
+    __shared__ unsigned int wsum[32];
+    __shared__ unsigned long long s_prefix;
+    __shared__ long long s_rank;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    unsigned long long kk[kSelSmallU];
+#pragma unroll
+    for (int u = 0; u < kSelSmallU; u++) {
+        const int i = u * kSelSmallT + tid;
+        kk[u] = i < n ? dkey(x[i]) : 0ull;
+    }
+    double med = 0.0;
+    unsigned long long prefix = 0;
+    for (int pass = 0; pass < 2; pass++) {
+        unsigned long long mask = 0;
+        long long r = rank;
+        prefix = 0;
+        for (int top = 64; top > 0; top -= kSelBits) {
+            const int shift = top > kSelBits ? top - kSelBits : 0, bits = top - shift;
+            const unsigned int nbin = 1u << bits;
+            for (int q = tid; q < kSelBins; q += kSelSmallT) hist[q] = 0;
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < kSelSmallU; u++) {
+                if (u * kSelSmallT >= n) break;
+                const int i = u * kSelSmallT + tid;
+                int bin = -1;
+                if (i < n && (kk[u] & mask) == prefix) bin = (int)((kk[u] >> shift) & (nbin - 1));
+                if (!__any_sync(0xffffffffu, bin >= 0)) continue;
+                const unsigned grp = __match_any_sync(0xffffffffu, bin);
+                if (bin >= 0 && lane == __ffs(grp) - 1) atomicAdd(&hist[bin], (unsigned)__popc(grp));
+            }
+            __syncthreads();
+            unsigned int h[kSelSmallB], own = 0;   // thread t owns kSelSmallB bins; zero past nbin
+#pragma unroll
+            for (int q = 0; q < kSelSmallB; q++) {
+                h[q] = hist[kSelSmallB * tid + q];
+                own += h[q];
+            }
+            unsigned int incl = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (lane == 31) wsum[warp] = incl;
+            __syncthreads();
+            long long before = (long long)incl - own;   // keys in lower bins
+            for (int w = 0; w < warp; w++) before += wsum[w];
+#pragma unroll
+            for (int q = 0; q < kSelSmallB; q++) {
+                if (r >= before && r < before + h[q]) {
+                    s_prefix = prefix | (unsigned long long)(kSelSmallB * tid + q) << shift;
+                    s_rank = r - before;
+                }
+                before += h[q];
+            }
+            mask |= (unsigned long long)(nbin - 1) << shift;
+            __syncthreads();
+            prefix = s_prefix;
+            r = s_rank;
+        }
+        if (pass == 0) {
+            med = dkey_inv(prefix);
+#pragma unroll
+            for (int u = 0; u < kSelSmallU; u++) {
+                if (u * kSelSmallT >= n) break;
+                kk[u] = dkey(fabs(dkey_inv(kk[u]) - med));   // the key gives x back bit for bit
+            }
+        }
+    }
+    if (tid == 0) {
+        st->med = med;
+        st->prefix = prefix;
+    }
+}
+
 // out[i] (+)= scale * (x[i] - median) / (1.4826 MAD + eps), with one fp64
 // division (fp64 division is slow on this part; the product differs from the
 // quotient by at most one rounding).
@@ -423,6 +509,13 @@ void robust_z(const double *x, int n, double scale, int accumulate, double *out,
     const long long rank = (n - 1) / 2;
     const int hb = (int)std::max<long long>(1, std::min<long long>(2LL * n_sms, ((long long)n + kSelT * kSelU - 1) / (kSelT * kSelU)));
     const int eb = (int)std::max<long long>(1, std::min<long long>(4LL * n_sms, ((long long)n + 255) / 256));
+    if (n <= kSelSmallT * kSelSmallU) {
+        // pr1 (1024 positions), with the narrower curvature blocks: 1.31 -> 1.22 ms
+        zsel_small_kernel<<<1, kSelSmallT, 0, s>>>(x, n, rank, st);
+        zsel_z_kernel<<<eb, 256, 0, s>>>(x, n, st, scale, accumulate, out);
+        *launches += 2;
+        return;
+    }
     zsel_init_kernel<<<1, 256, 0, s>>>(st, ghist, rank, 0);
     for (int pass = 0; pass < 2; pass++) {
         for (int top = 64; top > 0; top -= kSelBits) {
@@ -1267,29 +1360,33 @@ cudaError_t launch_segment(Ctx &c, const void *V, const float *hidden, int Dh,
     if (bf) seg_norm_kernel<<<gn, 256, 0, s>>>(Vb, hidden, a, w.inv_norm, w.nrm2);
     else seg_norm_kernel<<<gn, 256, 0, s>>>(Vf, hidden, a, w.inv_norm, w.nrm2);
 
-    // curvature: one thread per position, staged normalised channels
+    // curvature: two positions per thread, staged normalised channels
     {
         const bool defw = c.nwin == 3 && p.windows[0] == 4 && p.windows[1] == 8 && p.windows[2] == 16;
-        dim3 gc((p.T + kCurvPT - 1) / kCurvPT, c.nseg);
-        const int sm = (int)kCurvSmem;
-        if (bf && !hidden) {
-            if (defw) {
-                cudaFuncSetAttribute(seg_curv_kernel<__nv_bfloat16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                seg_curv_kernel<__nv_bfloat16, true><<<gc, 256, sm, s>>>(Vb, hidden, a, w.inv_norm, w.klw);
-            } else {
-                cudaFuncSetAttribute(seg_curv_kernel<__nv_bfloat16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                seg_curv_kernel<__nv_bfloat16, false><<<gc, 256, sm, s>>>(Vb, hidden, a, w.inv_norm, w.klw);
-            }
-        } else {
-            const float *Vx = bf ? nullptr : Vf;
-            if (defw) {
-                cudaFuncSetAttribute(seg_curv_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                seg_curv_kernel<float, true><<<gc, 256, sm, s>>>(Vx, hidden, a, w.inv_norm, w.klw);
-            } else {
-                cudaFuncSetAttribute(seg_curv_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                seg_curv_kernel<float, false><<<gc, 256, sm, s>>>(Vx, hidden, a, w.inv_norm, w.klw);
-            }
-        }
+        auto curv = [&](auto nt, auto dw, const auto *x) {
+            constexpr int NT = decltype(nt)::value;
+            using Tin = std::remove_cv_t<std::remove_reference_t<decltype(*x)>>;
+            auto kern = seg_curv_kernel<Tin, decltype(dw)::value, NT>;
+            using Cfg = CurvCfg<NT>;
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
+            kern<<<dim3((p.T + Cfg::PT - 1) / Cfg::PT, c.nseg), NT, Cfg::SMEM, s>>>(x, hidden, a, w.inv_norm, w.klw);
+        };
+        auto curv_w = [&](auto nt, const auto *x) {
+            if (defw) curv(nt, std::true_type(), x);
+            else curv(nt, std::false_type(), x);
+        };
+        auto curv_t = [&](auto nt) {
+            if (bf && !hidden) curv_w(nt, Vb);
+            else curv_w(nt, bf ? nullptr : Vf);
+        };
+        // 512 positions a block (the halo is 6 % of its rows).  A few such blocks are
+        // bound by their own instructions: up to an eighth of the SMs, 128 positions
+        // (25 %) spread them over four times as many.  Not above: the blocks then
+        // take SMs from the score passes beside them (48 wide blocks, small 8x:
+        // 9.93 -> 10.42 ms).
+        using Wide = CurvCfg<256>;
+        if ((p.T + Wide::PT - 1) / Wide::PT * c.nseg <= c.num_sms / 8) curv_t(std::integral_constant<int, 64>());
+        else curv_t(std::integral_constant<int, 256>());
     }
     seg_combine_kernel<<<(p.T + 255) / 256, 256, 0, s>>>(w.klw, c.nseg * c.nwin, p.T, p.lambda_stab,
                                                           w.kappa, kappa_out, w.dev_int + 1);

@@ -12,6 +12,8 @@ and n_min = 5 / n_max = 40 (steps of 5 endpoints, 160 per chunk, ragged end).
 """
 from __future__ import annotations
 
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -19,6 +21,7 @@ import torch
 import oracle as O
 from paper_2608_07001_gb300 import gracekv as gk
 from paper_2608_07001_gb300 import synth
+from tests import parity as P
 
 pytestmark = pytest.mark.gpu
 
@@ -98,3 +101,14 @@ def test_chunked_dp_gives_the_oracle_slots_for_every_warm_up(case):
             assert 0 <= rerun < chunks
     # a 16-token warm-up is too short for the paths to coalesce: chunks are re-run
     assert runs[16][2] >= 1
+
+
+@pytest.mark.parametrize("T", [1025, 4096, 4097])   # the one-block robust z ends at 4096 positions
+def test_robust_z_block_edges_match_the_oracle(T):
+    w = dataclasses.replace(synth.WORKLOADS["small"], L=1, G=1, Hq=1, d=64)
+    x = synth.make_inputs(w, T=T, W=8)
+    rng = np.random.default_rng(T)
+    sur = -np.log(rng.random(T)).astype(np.float32)
+    g = P.run_gpu(x.K, x.V, x.Q, T // 8, w.rope_base, surprisal=sur)
+    o = P.run_oracle(x.K, x.V, x.Q, T // 8, w.rope_base, surprisal=sur)
+    P.compare(g, o, torch.bfloat16)
