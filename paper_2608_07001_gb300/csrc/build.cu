@@ -232,6 +232,21 @@ __device__ __forceinline__ void ld8x2(const __nv_bfloat16 *p, float2 v[4]) {
     for (int i = 0; i < 4; i++) v[i] = __bfloat1622float2(h[i]);
 }
 
+// Row that a lane of an 8-row matrix tile reads in an instance of NMAX rows:
+// where they are no multiple of 8, the slot's last one in place of those past
+// it (the columns of rows past the slot are dropped).
+template <int NMAX>
+__host__ __device__ constexpr int tile_row(int row, int n) { return NMAX % 8 == 0 || row < n ? row : n - 1; }
+template <int NMAX>
+constexpr bool tile_rows_inside() {
+    for (int n = 1; n <= NMAX; n++)
+        for (int row = 0; row < (n + 7) / 8 * 8; row++)
+            if (tile_row<NMAX>(row, n) >= NMAX) return false;
+    return true;
+}
+static_assert(tile_rows_inside<kTinyUnit>() && tile_rows_inside<kShortUnit>() && tile_rows_inside<kMaxUnit>(),
+              "the probe weights' tiles stay inside the slot's array");
+
 // 8 floats to a 16-byte aligned shared-memory row.
 __device__ __forceinline__ void st8(float *p, const float v[8]) {
     reinterpret_cast<float4 *>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
@@ -647,7 +662,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
         const int ntn = (n + 7) / 8;
         for (int nt = warp / MT; nt < ntn; nt += WSTEP) {
             float acc[4] = {0.f, 0.f, 0.f, 0.f};
-            const float *kr = &sm.kc[nt * 8 + gr][c2];
+            const float *kr = &sm.kc[tile_row<NMAX>(nt * 8 + gr, n)][c2];
 #pragma unroll
             for (int ks = 0; ks < DH / 16; ks++) {
                 const float2 x0 = *reinterpret_cast<const float2 *>(kr + ks * 16);

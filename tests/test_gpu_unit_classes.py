@@ -72,3 +72,18 @@ def test_small_selection_matches_the_oracle(last, ratio):
     g = P.run_gpu(x.K, x.V, x.Q, B, w.rope_base, slot_starts=slots)
     o = P.run_oracle(x.K, x.V, x.Q, B, w.rope_base, slot_starts=slots)
     P.compare(g, o, torch.bfloat16)
+
+
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 33, 34, 35, 36])
+def test_probe_weight_tiles_end_at_the_slot(n):
+    # 320 probe rows per KV head: the unit kernel forms the probe weights itself, in tiles of
+    # 8 tokens; with 340 slots the 36-token class runs on its own instance, whose last tile
+    # has rows past the slot (and, above 32 tokens, past the instance's 36)
+    lens = [n] * 40 + [1 + i % 3 for i in range(300)]
+    w = dataclasses.replace(synth.WORKLOADS["small"], L=1, G=1, Hq=8, d=128)
+    x = synth.make_inputs(w, T=sum(lens) + 32, W=40)
+    slots = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    B = x.K.shape[2] // 3
+    g = P.run_gpu(x.K, x.V, x.Q, B, w.rope_base, slot_starts=slots)
+    o = P.run_oracle(x.K, x.V, x.Q, B, w.rope_base, slot_starts=slots)
+    P.compare(g, o, torch.bfloat16)
