@@ -73,7 +73,7 @@ struct BuildArgs {
     int L, G, Hq, T, d, W, gq, cs, Nc, J, k_cand;
     float inv_sqrt_d, lamZ, lamM, eps;
     float lam_kappa, base_frac;
-    int prune;                   // lambda_Z, lambda_M >= 0, so every D >= 0: cuts may be ruled out by bounds
+    int prune;                   // lambda_Z, lambda_M >= 0, so every D >= 0: cuts and nodes may be ruled out by bounds
     // work list: fresh launches index (slot list entry, lg), resume launches units
     int resume;                  // 0: build from the root, 1: resume pending nodes
     int root_only;               // fresh: evaluate only the root's own distortion (split stays pending)
@@ -141,8 +141,8 @@ __device__ __forceinline__ void rotate_to(float x, float y, float c, float s, fl
 }
 
 // Upper bound of a split's utility: U = omega R (D - sum D_children) / cost
-// <= omega R D, since every D >= 0 and cost >= 1 (Eqs. app_operation_gains,
-// app_unit_utility).  Rounded up by 1e-5 of its value: the R that the bound
+// <= omega R D where every D and omega are >= 0, since cost >= 1 (Eqs.
+// app_operation_gains, app_unit_utility).  Rounded up by 1e-5 of its value: the R that the bound
 // uses (one fp32 sum over the node's tokens) and the R of the later gain (the
 // sum of its children's sums) differ by at most ~1.3e-6 of R, and the products
 // add a few ulp, so rounding never makes a bound fall below the utility it bounds.
@@ -479,6 +479,10 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
     const Tin *Kp = static_cast<const Tin *>(A.K) + ((size_t)lg * A.T + sa) * DH;
     const Tin *Vp = static_cast<const Tin *>(A.V) + ((size_t)lg * A.T + sa) * DH;
     const float om = A.omega ? A.omega[lg] : 1.0f;
+    // key bound of a pending node of value R and distortion D, kin the key of its
+    // creator; with a negative weight or omega only the creator's key bounds it
+    const bool bounded = A.prune && om >= 0.f;
+    auto split_bound = [&](float kin, float R, float D) { return bounded ? fminf(kin, key_bound(om * R * D)) : kin; };
 
     // Probe weights E[t][u] (Eq. app_probe_distortion), stored at E[t][u % 32].x
     // (u < 32) or .y (u >= 32).  When the score pass wrote them for every token
@@ -1455,9 +1459,9 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
                 const int nch = B.nchild;
-                if (nch < 0) {   // pending root: its split key is at most min(U_add, omega R D)
+                if (nch < 0) {   // pending root
                     if (lane == 0) {
-                        const float bnd = B.forced ? FLT_MAX : fminf(nd.kin, key_bound(om * sm.rootR * nd.D));
+                        const float bnd = B.forced ? FLT_MAX : split_bound(nd.kin, sm.rootR, nd.D);
                         nd.nchild = -1;
                         A.nd_child0[gv] = -1; A.nd_nchild[gv] = -1; A.nd_cost[gv] = 0;
                         A.nd_U[gv] = bnd; A.nd_kappa[gv] = 0.f; A.nd_sel[gv] = 0;
@@ -1509,7 +1513,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                     bool chf = false;
                     if (ufl)
                         for (int t = B.ca[q]; t < B.cb[q] && !chf; t++) chf = sm.Ff[t] > -INFINITY;
-                    const float cbnd = B.cb[q] - B.ca[q] >= 2 ? (chf ? FLT_MAX : fminf(kap, key_bound(om * rq * B.cD[q]))) : 0.f;
+                    const float cbnd = B.cb[q] - B.ca[q] >= 2 ? (chf ? FLT_MAX : split_bound(kap, rq, B.cD[q])) : 0.f;
                     A.nd_U[gc] = cbnd;
                     A.nd_kappa[gc] = 0.f; A.nd_sel[gc] = 0;
                     if (B.cb[q] - B.ca[q] >= 2) {

@@ -83,7 +83,7 @@ struct LongArgs {
     float inv_sqrt_d, lamZ, lamM, eps, lam_kappa, base_frac;
     int fresh;                     // 1: the roots of the listed slots; 0: pending nodes of listed units
     int root_only;                 // fresh: only the root's own distortion (its split stays pending)
-    int prune;                     // lambda_Z, lambda_M >= 0, so every D >= 0: cuts may be ruled out by bounds
+    int prune;                     // lambda_Z, lambda_M >= 0, so every D >= 0: cuts and nodes may be ruled out by bounds
     float tau;                     // resume: evaluate pending nodes whose key bound >= tau
     const int32_t *list;           // fresh: slot indices; resume: unit ids
     int n_list, lg0, nlg;          // fresh units: slot list x (l, g) in [lg0, lg0 + nlg)
@@ -111,7 +111,7 @@ struct LongArgs {
     unsigned long long *work;
 };
 
-// Upper bound of a split's utility (see build.cu: U <= omega R D, rounded up).
+// Upper bound of a split's utility (see build.cu: U <= omega R D where both factors are >= 0, rounded up).
 __device__ __forceinline__ float lkey_bound(float x) { return x + fabsf(x) * 1e-5f; }
 
 __device__ __forceinline__ unsigned long long lokey(double x) {
@@ -1130,6 +1130,8 @@ __global__ void __launch_bounds__(kLT, EG ? 2 : 1) long_eval_kernel(LongArgs A) 
             const bool ufl = A.it_ufl[it] != 0;
             float kin = A.it_kin[it];
             float DI;
+            const bool bounded = A.prune && om >= 0.f;   // build.cu
+            auto split_bound = [&](float k, float R, float D) { return bounded ? fminf(k, lkey_bound(om * R * D)) : k; };
             const float nodeR = A.nd_R[gv];
             if (root) {   // D, D_drop and the Add gain of the slot (Eq. app_operation_gains)
                 const float Pd = sm.candP[sm.whole];
@@ -1158,7 +1160,7 @@ __global__ void __launch_bounds__(kLT, EG ? 2 : 1) long_eval_kernel(LongArgs A) 
                 rs.nch = 0;
             } else if (ronly) {   // the root's split is decided later: bound its key
                 rs.nch = -1;
-                rs.bound = forced ? FLT_MAX : fminf(kin, lkey_bound(om * nodeR * DI));
+                rs.bound = forced ? FLT_MAX : split_bound(kin, nodeR, DI);
             } else {
                 int nch;
                 if (n == 2) {
@@ -1223,7 +1225,7 @@ __global__ void __launch_bounds__(kLT, EG ? 2 : 1) long_eval_kernel(LongArgs A) 
                 rs.kap = forced ? FLT_MAX : fminf(rs.U, kin);
                 for (int q = 0; q < nch; q++)
                     rs.bnd[q] = rs.cb[q] - rs.ca[q] >= 2
-                                    ? (chf[q] ? FLT_MAX : fminf(rs.kap, lkey_bound(om * rs.rch[q] * rs.cD[q])))
+                                    ? (chf[q] ? FLT_MAX : split_bound(rs.kap, rs.rch[q], rs.cD[q]))
                                     : 0.f;
                 rs.nch = nch;
             }
