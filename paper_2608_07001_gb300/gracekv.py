@@ -221,10 +221,17 @@ def _addr(t: Optional[torch.Tensor]) -> int:
     return t.data_ptr()
 
 
+# The two calls under torch.cuda.current_stream(), where this PyTorch has them by these names.
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+_current_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _raw_stream(stream) -> int:
-    if stream is not None:
-        return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if stream is None:
+        if _current_device is not None and _current_raw_stream is not None:
+            return _current_raw_stream(_current_device())
+        stream = torch.cuda.current_stream()
+    return stream.cuda_stream
 
 
 def make_params(L, G, Hq, T, d, W, *, dtype, budget, rope_base, ctx_start=0, ctx_end=None,

@@ -70,3 +70,18 @@ def test_noalloc_refuses_mismatched_arguments_before_any_launch(gk):
         with pytest.raises(gk.GraceKVError, match=why) as e:
             gk.gracekv_row_stats_noalloc(k, q, 0, 64, out, ok, ok)
         assert e.value.status == gk.GKV_EINVAL
+
+
+@pytest.mark.parametrize("gone", ["_cuda_getDevice", "_cuda_getCurrentRawStream"])
+def test_raw_stream_without_the_private_names(gk, monkeypatch, gone):
+    # a PyTorch without one of the two private calls takes the public stream object
+    import importlib.util
+    import types
+    monkeypatch.delattr(torch._C, gone, raising=False)
+    spec = importlib.util.spec_from_file_location("gracekv_without", gk.__file__)
+    m = importlib.util.module_from_spec(spec)
+    monkeypatch.setitem(__import__("sys").modules, "gracekv_without", m)   # its dataclasses look their module up
+    spec.loader.exec_module(m)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=41))
+    assert m._raw_stream(None) == 41
+    assert m._raw_stream(types.SimpleNamespace(cuda_stream=7)) == 7
