@@ -1115,7 +1115,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
         const bool ext = B.ext;
         const bool el = ext && ps - a >= 2, er = ext && b - (ps + 1) >= 2;
         const int k1 = B.k1, ncut = B.ncut;
-        const float best1 = ((DI - B.cD[0]) - B.cD[1]) + A.lam_kappa * B.kh[k1];
+        const float best1 = fmaf(A.lam_kappa, B.kh[k1], (DI - B.cD[0]) - B.cD[1]);
         const float DL1 = B.cD[0], DR1 = B.cD[1];
         const int xi = lane < ncut ? B.cut[lane] : 0;
         const float rew = lane < ncut ? B.kh[lane] : 0.f;
@@ -1134,7 +1134,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
             const int np = both || pass == 0 ? npre : 0;
             int ns = 0, srow = 0, er_row = 0;
             if (pass == 1) {
-                if (!both && A.prune) need = need && !((DI - dl) + A.lam_kappa * rew < best1);
+                if (!both && A.prune) need = need && !(fmaf(A.lam_kappa, rew, DI - dl) < best1);
                 sv = need && b - xi >= 2;
                 const unsigned sm_ = __ballot_sync(FULL, sv);
                 ns = __popc(sm_) + (er ? 1 : 0);
@@ -1183,7 +1183,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
         // a cut ruled out by its D_L keeps G_bin's bound, which is below best1
         float val = -INFINITY;
         if (lane == k1) { dl = DL1; dr = DR1; val = best1; }
-        else if (need) val = ((DI - dl) - dr) + A.lam_kappa * rew;
+        else if (need) val = fmaf(A.lam_kappa, rew, (DI - dl) - dr);
         const unsigned key = lane < ncut ? fkey_ordered(val) : 0u;
         const unsigned kmx = __reduce_max_sync(FULL, key);   // every lane takes part
         const unsigned top = __ballot_sync(FULL, lane < ncut && key == kmx);
@@ -1385,7 +1385,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
             // ---- phase D1: decisions (warp per node) ---------------------------------
             // G_bin of a cut is ((D - D_L) - D_R) + lambda_kappa kh, and D_L, D_R >= 0:
             // D + lambda_kappa kh bounds it from above, in the rounded arithmetic too
-            // (every operation is monotone).  A cut whose bound is below G_bin of the
+            // (every operation is monotone; G_bin and its bounds all fuse the product).  A cut whose bound is below G_bin of the
             // cut already evaluated cannot be the best one, and its intervals are never
             // evaluated; neither are the extraction's sides when that G_bin reaches D,
             // which bounds rho_ext.  The other cuts are evaluated below, one node at a
@@ -1430,9 +1430,9 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                     continue;
                 }
                 const int k1 = B.k1;
-                const float best = ((DI - DL) - DR) + A.lam_kappa * B.kh[k1];
+                const float best = fmaf(A.lam_kappa, B.kh[k1], (DI - DL) - DR);
                 bool need = lane < B.ncut && lane != k1;
-                if (need && A.prune) need = !(DI + A.lam_kappa * B.kh[lane] < best);
+                if (need && A.prune) need = !(fmaf(A.lam_kappa, B.kh[lane], DI) < best);
                 const unsigned more = __ballot_sync(0xffffffffu, need);
                 const bool ext = !(A.prune && best >= DI);
                 if (lane == 0) {

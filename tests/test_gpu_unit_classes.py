@@ -87,3 +87,25 @@ def test_probe_weight_tiles_end_at_the_slot(n):
     g = P.run_gpu(x.K, x.V, x.Q, B, w.rope_base, slot_starts=slots)
     o = P.run_oracle(x.K, x.V, x.Q, B, w.rope_base, slot_starts=slots)
     P.compare(g, o, torch.bfloat16)
+
+
+@pytest.mark.parametrize("k_cand", [16, 3])
+@pytest.mark.parametrize("lam", [0.0, 0.05])
+@pytest.mark.parametrize("dtype,d", [("bf16", 64), ("fp32", 128)])
+def test_tied_cuts_take_the_smallest(dtype, d, lam, k_cand):
+    # V = 0 and lambda_Z = 0: every D is exactly 0 and the curvature of the zero trajectory
+    # takes few values, so the rewards, and with them the cuts, tie; neither the cut that is
+    # evaluated first nor a bound may move the choice from the smallest position
+    lens = [36, 2, 3, 5, 128, 37, 64, 65, 17, 129, 300]
+    w = dataclasses.replace(synth.WORKLOADS["small"], L=1, G=1, Hq=4, d=d)
+    x = synth.make_inputs(w, T=sum(lens) + 32, W=8)
+    K, V, Q = x.K, torch.zeros_like(x.V), x.Q
+    if dtype == "fp32":
+        K, V, Q = K.float(), V.float(), Q.float()
+    kw = dict(lambda_Z=0.0, lambda_kappa=lam, k_cand=k_cand,
+              slot_starts=np.concatenate([[0], np.cumsum(lens)]).astype(np.int32))
+    B = K.shape[2] // 2
+    g = P.run_gpu(K, V, Q, B, w.rope_base, **kw)
+    o = P.run_oracle(K, V, Q, B, w.rope_base, **kw)
+    assert not o["trees"].nodes["D"].any()
+    P.compare(g, o, torch.float32 if dtype == "fp32" else torch.bfloat16)
