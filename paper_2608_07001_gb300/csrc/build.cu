@@ -59,6 +59,15 @@ constexpr int kNCL = 8;          // threads per probe pair (4-element groups, in
 constexpr int kPPW = 32 / kNCL;  // probe pairs per warp: lane = 4 c + (pair % 4), so that the
                                  // 4 lanes reading one 16-byte chunk are adjacent (one shared-
                                  // memory wavefront serves them; lanes 8 apart would not merge)
+// A cut evaluated ahead of the others pays where its reward rules most of them
+// out, and costs a second sweep of the node where it does not: with
+// lambda_kappa at most kDirect of the node's D (of a fresh root's attention mass,
+// which weights its D, not known yet) all cuts are evaluated at once.  The mass
+// is formed below kDirectMax only: a slot of a long request holds far less.
+// 16 layers of llama32k, lambda_kappa 0 at 8x / 32x: 100.3 -> 82.4 / 35.0 ->
+// 29.2 ms, 2e-4: 95.4 -> 83.0 / 34.5 -> 29.7, 1e-3: 75.2 -> 67.9 / 29.6 -> 27.4;
+// shares of 0.1 to 0.5 were up to 5 % slower at 1e-4 to 1e-3, of 2 and 3 no faster.
+constexpr float kDirect = 1.0f, kDirectRoot = 1.0f, kDirectMax = 0.01f;
 constexpr int kNCR = 19;         // candidate rows held at a time: 17 cuts + p* side (+ 1)
 
 struct BuildArgs {
@@ -78,6 +87,7 @@ struct BuildArgs {
     int resume;                  // 0: build from the root, 1: resume pending nodes
     int root_only;               // fresh: evaluate only the root's own distortion (split stays pending)
     int max_levels;              // levels evaluated by this launch
+    int nrow;                    // candidate rows that the launch's shared memory holds (kNCR or Smem::NROW)
     float tau;                   // resume: evaluate pending nodes whose key bound >= tau
     const int32_t *list;         // fresh: slot indices; resume: unit ids; subtree: node indices
     int64_t stride;              // the launch's classes follow one another at this distance,
@@ -109,13 +119,15 @@ struct BatchNode {
     unsigned long long klo, khi;   // smallest and largest curvature key over the node's cut positions
     float kh[kMaxCuts];      // normalised curvature of the cuts
     float cD[3];
-    unsigned more;           // cuts that the first one evaluated does not rule out
+    unsigned more, keep;     // open node: cuts that the first one evaluated does not rule out; nor their D_L
     short node, pstar;
     short op;                // the node's place among the batch's Split ops (-1: none)
     short ca[3], cb[3];
     int8_t cut[kMaxCuts];    // local cut positions xi (ascending)
     int8_t ncut, k1;         // cuts; the one of largest curvature reward
     int8_t rl, rr, whole;    // rows of its sides (-1: single token) and of the node itself
+    int8_t direct;           // no cut is evaluated ahead of the others
+    int8_t np, ns;           // open node: prefixes and suffixes left to evaluate
     int8_t nchild;           // -1: pending root, -2: undecided
     int8_t forced;           // extraction at a singleton-floor position (a floor op)
     int8_t ext;              // the extraction's sides are needed
@@ -393,9 +405,9 @@ struct Smem {
     static constexpr int CTAS = NMAX <= kTinyUnit ? 3 : (NMAX <= kShortUnit ? 2 : 1);   // per SM
     static constexpr int NT = kNT * DIRS;
     static constexpr int NWARPS = NT / 32;
-    static constexpr int NB = 16;            // nodes per batch
+    static constexpr int NB = NWARPS;        // nodes per batch: one a warp
     static constexpr int MAXNODES = 2 * NMAX;
-    static constexpr int NROW = kNCR;        // candidate rows held at a time
+    static constexpr int NROW = kNCR * DIRS; // candidate rows held at a time: one side of a node, or both
     static constexpr int KTW = DH < 128 ? 128 : DH;        // a row also holds 32 float4 of sums
     static constexpr int MW = (MAXNODES + 31) / 32;
     static constexpr int KPAD = NMAX <= kShortUnit ? 8 : 0;
@@ -403,10 +415,6 @@ struct Smem {
                                              // MMA reads 8 rows at once, which then fall in distinct banks
     float vv[NMAX][DH];                      // values, converted once to fp32
     float2 E[NMAX][kNPP];                    // probe weights of probes (p, p + 32)
-    float ktil[NROW][KTW];                   // key prototypes; once the logits are taken, the row holds
-                                             // (residual / ||M||^2, Z) of the probes p and p + 32
-    float vtil[NROW][DH];
-    float2 zt[NROW][kNPP];                   // m_eff exp(logit) of the probes (p, p + 32)
     float2 RK[NMAX];                         // token value, ||k||
     unsigned long long kap[NMAX];            // order-preserving keys of the curvature
     uint8_t rk[NMAX];                        // the token's place among the slot's by curvature (0: largest)
@@ -414,12 +422,18 @@ struct Smem {
     Cand cand[NROW];
     NodeS nodes[MAXNODES];
     float Ff[NMAX];                          // floor score of an accepted floor position, -inf elsewhere
-    float candD[NROW], candP[NROW];          // per-row D and drop mass
+    float candD[NROW + kNCR], candP[NROW + kNCR];  // per-row D and drop mass (prefixes kept while the suffixes follow)
     unsigned lvl[2][MW];                     // nodes of the level (bit masks), of the next one
     unsigned op_base;                        // the batch's first Split op in the global list
     unsigned int wcnt[NWARPS][3];            // per-warp work counters
     float pend;
     float rootR;                             // R of a fresh root
+    struct Row {
+        alignas(16) float ktil[KTW];         // key prototype; once the logits are taken, the row holds
+                                             // (residual / ||M||^2, Z) of the probes p and p + 32
+        float vtil[DH];
+        float2 zt[kNPP];                     // m_eff exp(logit) of the probes (p, p + 32)
+    } rows[NROW];                            // the last ones only where A.nrow takes them in
 };
 
 // SUB: the subtree mode, a compile-time flag so that the other instances carry
@@ -849,7 +863,22 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
         const unsigned m = __ballot_sync(0xffffffffu, q);
         if (lane == 0 && warp < S::MW) sm.lvl[0][warp] = m;
     }
+    // a fresh root's attention mass, mean over the probes, where it decides how the
+    // root is evaluated (thread tid adds the tokens' weights of one probe)
+    const bool weigh = fresh && !A.root_only && A.prune && A.lam_kappa > 0.f && A.lam_kappa < kDirectMax;
+    if (weigh) {
+        const int e0 = tid & (2 * kNPP - 1), u = (e0 >> 1) + kNPP * (e0 & 1);
+        float p = 0.f;
+        for (int e = tid; e < n * 2 * kNPP; e += NT) p += Ef[e];
+        p = warp_sum(u < A.W ? p / A.row_Z[qrow(u)] : 0.f);
+        if (lane == 0) sm.candP[warp] = p;
+    }
     __syncthreads();
+    float mass = 0.f;
+    if (weigh) {
+        for (int w = 0; w < NWARPS; w++) mass += sm.candP[w];
+        mass /= A.W;
+    }
 
     unsigned int w_scan = 0, w_eval = 0, w_len = 0;   // work counters (lane 0 of each warp)
 
@@ -883,7 +912,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                 const float a0 = acc.lo(j) * ninv, a1 = acc.hi(j) * ninv;
                 mu2 = fmaf(a0, a0, fmaf(a1, a1, mu2));
                 const float2 cs = rot[j];
-                rotate_to<SF>(a0, a1, cs.x, cs.y, sm.ktil[row][pi0 + j], sm.ktil[row][pi0 + j + HALF]);
+                rotate_to<SF>(a0, a1, cs.x, cs.y, sm.rows[row].ktil[pi0 + j], sm.rows[row].ktil[pi0 + j + HALF]);
             }
             mu2 = warp_sum(mu2);
             if (lane == 0) {
@@ -932,8 +961,8 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
             const float winv = 1.0f / ((acc.rs + (float)nJ * beta) + A.eps);
 #pragma unroll
             for (int j = 0; j < PPL; j++) {
-                sm.vtil[row][pi0 + j] = fmaf(beta, acc.slo(j), acc.rlo(j)) * winv;
-                sm.vtil[row][pi0 + j + HALF] = fmaf(beta, acc.shi(j), acc.rhi(j)) * winv;
+                sm.rows[row].vtil[pi0 + j] = fmaf(beta, acc.slo(j), acc.rlo(j)) * winv;
+                sm.rows[row].vtil[pi0 + j + HALF] = fmaf(beta, acc.shi(j), acc.rhi(j)) * winv;
             }
         };
         PS s0;
@@ -992,7 +1021,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                 float2 xa = make_float2(0.f, 0.f), xb = make_float2(0.f, 0.f);
 #pragma unroll
                 for (int gi = 0; gi < NG; gi++) {
-                    const float4 x = *reinterpret_cast<const float4 *>(&sm.ktil[row][4 * c + 32 * gi]);
+                    const float4 x = *reinterpret_cast<const float4 *>(&sm.rows[row].ktil[4 * c + 32 * gi]);
                     const float2 ka = make_float2(x.x, x.y), kb = make_float2(x.z, x.w);
                     xa = ffma2(qa0[2 * gi], ka, xa);
                     xa = ffma2(qa0[2 * gi + 1], kb, xa);
@@ -1005,7 +1034,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
             const float x = reduce_scatter8(v, lane);
             const int row = i + (c & 3);
             if (row < nr)
-                reinterpret_cast<float *>(&sm.zt[row][pp])[c >> 2] =
+                reinterpret_cast<float *>(&sm.rows[row].zt[pp])[c >> 2] =
                     sm.cand[row].meff * expf(x * inv_sqrt_d - mu_log);
         }
     };
@@ -1046,12 +1075,12 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
 #pragma unroll 2
                 for (; t < stop; t++) add(t);
             }
-            const float2 z = sm.zt[k][pp];
+            const float2 z = sm.rows[k].zt[pp];
             const float2 nz0 = make_float2(-z.x, -z.x), nz1 = make_float2(-z.y, -z.y);
             float2 r0 = make_float2(0.f, 0.f), r1 = r0, m0 = r0, m1 = r0;
 #pragma unroll
             for (int gi = 0; gi < NG; gi++) {
-                const float4 x = *reinterpret_cast<const float4 *>(&sm.vtil[k][4 * c + 32 * gi]);
+                const float4 x = *reinterpret_cast<const float4 *>(&sm.rows[k].vtil[4 * c + 32 * gi]);
                 const float2 va = make_float2(x.x, x.y), vb = make_float2(x.z, x.w);
 #pragma unroll
                 for (int h = 0; h < 2; h++) {
@@ -1069,7 +1098,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
             // at most 2 ulp, far below the distortion tolerance.
             const float x = reduce_scatter4(r0.x + r0.y, r1.x + r1.y, m0.x + m0.y, m1.x + m1.y, lane);
             const float y = __shfl_xor_sync(0xffffffffu, x, 2 * kPPW);
-            if (c < 4) sm.ktil[k][4 * pp + c] = (c & 2) ? ((c & 1) ? Z.y : Z.x) : __fdividef(x, y + epsf);
+            if (c < 4) sm.rows[k].ktil[4 * pp + c] = (c & 2) ? ((c & 1) ? Z.y : Z.x) : __fdividef(x, y + epsf);
         }
     };
     // D_u (Eq. app_probe_distortion) of the rows [0, nr), weighted by the
@@ -1077,12 +1106,12 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
     // row, lane p the probes p and p + 32.  The sums run over groups of four
     // lanes, then over the groups in order.  Probes past W have E = 0 and
     // invZ = 0, so they add nothing.
-    auto finish = [&](int nr) {
+    auto finish = [&](int nr, int out) {
         const float invW = 1.0f / A.W;
         for (int k = warp; k < nr; k += NWARPS) {
             if (sm.cand[k].b <= sm.cand[k].a) continue;
-            const float4 q = *reinterpret_cast<const float4 *>(&sm.ktil[k][4 * lane]);   // ratios, Z
-            const float2 z = sm.zt[k][lane];
+            const float4 q = *reinterpret_cast<const float4 *>(&sm.rows[k].ktil[4 * lane]);   // ratios, Z
+            const float2 z = sm.rows[k].zt[lane];
             const float Z0 = q.z, Z1 = q.w;
             const float dz0 = Z0 - z.x, dz1 = Z1 - z.y;
             const float D0 = fmaf(lamZ, __fdividef(dz0 * dz0, fmaf(Z0, Z0, epsf)), lamM * q.x);
@@ -1098,92 +1127,66 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
             float d = 0.f;
 #pragma unroll
             for (int w = 0; w < 32 / kPPW; w++) d += __shfl_sync(0xffffffffu, x, kPPW * w + (lane & 1));
-            if (lane < 2) (lane ? sm.candP : sm.candD)[k] = d * invW;
+            if (lane < 2) (lane ? sm.candP : sm.candD)[out + k] = d * invW;
         }
     };
 
-    // The candidates of a node that the first ones could not rule out: both
-    // sides of the cuts in B.more and of the extraction (B.ext).  The prefixes
-    // first; their D tightens the cuts' bounds before the suffixes (together
-    // when all of them fit the rows).  Warp 0 lays the rows out and decides;
-    // the same decision as over all cuts, ties to the smallest xi.
-    auto evaluate_rest = [&](BatchNode &B) {
-        NodeS &nd = sm.nodes[B.node];
+    // A fresh root's D, Ddrop and Add gain (Eq. app_operation_gains), from its own row.
+    auto root_done = [&](NodeS &nd, int row) {
+        const float Pd = sm.candP[row];
+        const float D = nd.b - nd.a >= 2 ? sm.candD[row] : 0.f;
+        nd.D = D;
+        float gain = om * sm.rootR * (Pd - D);
+        if (gain < 0.f) gain = 0.f;
+        nd.kin = ufl ? FLT_MAX : gain;   // a floor slot's Add is a floor op
+        A.u_Uadd[uid] = gain;
+        A.u_Ddrop[uid] = Pd;
+        A.nd_D[gidx(0)] = D;
+    };
+    // The cuts of an open node, one per lane, and its rows: prefixes of the cuts
+    // in B.more and of the extraction by ascending end (then a direct root
+    // itself), suffixes of the cuts in B.keep by descending start.
+    struct Open {
+        int a, b, ps, xi, prow, srow, el_row, er_row;   // rows relative to the node's first of a direction
+        float rew;
+        bool pv, sv, el, er, elr, err;   // el, er: the extraction's sides; elr, err: in rows of their own
+    };
+    auto open_rows = [&](const BatchNode &B) {
+        const unsigned FULL = 0xffffffffu, lt = (1u << lane) - 1u, gt = ~((2u << lane) - 1u);
+        const NodeS &nd = sm.nodes[B.node];
+        Open o;
+        o.a = nd.a;
+        o.b = nd.b;
+        o.ps = B.pstar;
+        o.xi = lane < B.ncut ? B.cut[lane] : 0;
+        o.rew = lane < B.ncut ? B.kh[lane] : 0.f;
+        o.pv = ((B.more >> lane) & 1u) && o.xi - o.a >= 2;
+        o.sv = ((B.keep >> lane) & 1u) && o.b - o.xi >= 2;
+        o.el = B.ext && o.ps - o.a >= 2;
+        o.er = B.ext && o.b - (o.ps + 1) >= 2;
+        // a side equal to a cut's shares its row
+        o.elr = o.el && !__any_sync(FULL, o.pv && o.xi == o.ps);
+        o.err = o.er && !__any_sync(FULL, o.sv && o.xi == o.ps + 1);
+        o.prow = __popc(__ballot_sync(FULL, o.pv) & lt) + (o.elr && o.ps < o.xi ? 1 : 0);
+        o.srow = __popc(__ballot_sync(FULL, o.sv) & gt) + (o.err && o.ps + 1 > o.xi ? 1 : 0);
+        o.el_row = __popc(__ballot_sync(FULL, o.pv && o.xi < o.ps));
+        o.er_row = __popc(__ballot_sync(FULL, o.sv && o.xi > o.ps + 1));
+        return o;
+    };
+    auto best_first = [&](const BatchNode &B) {   // G_bin of the cut evaluated ahead
+        return B.direct ? -INFINITY : fmaf(A.lam_kappa, B.kh[B.k1], (sm.nodes[B.node].D - B.cD[0]) - B.cD[1]);
+    };
+    // The decision over all cuts that no bound ruled out, ties to the smallest xi.
+    auto decide_open = [&](BatchNode &B, int sufD) {
         const unsigned FULL = 0xffffffffu;
-        const int a = nd.a, b = nd.b, ps = B.pstar;
-        const float DI = nd.D;
-        const bool ext = B.ext;
-        const bool el = ext && ps - a >= 2, er = ext && b - (ps + 1) >= 2;
-        const int k1 = B.k1, ncut = B.ncut;
-        const float best1 = fmaf(A.lam_kappa, B.kh[k1], (DI - B.cD[0]) - B.cD[1]);
-        const float DL1 = B.cD[0], DR1 = B.cD[1];
-        const int xi = lane < ncut ? B.cut[lane] : 0;
-        const float rew = lane < ncut ? B.kh[lane] : 0.f;
-        bool need = (B.more >> lane) & 1u;
-        // every warp forms the same lists; the rows are written by warp 0
-        const bool pv = need && xi - a >= 2;
-        const unsigned lt = (1u << lane) - 1u, gt = ~((2u << lane) - 1u);
-        const unsigned pm = __ballot_sync(FULL, pv);
-        const int npre = __popc(pm) + (el ? 1 : 0);
-        const int prow = __popc(pm & lt) + (el && ps < xi ? 1 : 0);
-        const int el_row = __popc(__ballot_sync(FULL, pv && xi <= ps));
-        bool sv = need && b - xi >= 2;
-        const bool both = npre + __popc(__ballot_sync(FULL, sv)) + (er ? 1 : 0) <= S::NROW;
-        float dl = 0.f, dr = 0.f, eDL = 0.f, eDR = 0.f;
-        for (int pass = both ? 1 : 0; pass < 2; pass++) {
-            const int np = both || pass == 0 ? npre : 0;
-            int ns = 0, srow = 0, er_row = 0;
-            if (pass == 1) {
-                if (!both && A.prune) need = need && !(fmaf(A.lam_kappa, rew, DI - dl) < best1);
-                sv = need && b - xi >= 2;
-                const unsigned sm_ = __ballot_sync(FULL, sv);
-                ns = __popc(sm_) + (er ? 1 : 0);
-                srow = np + __popc(sm_ & gt) + (er && ps + 1 > xi ? 1 : 0);
-                er_row = np + __popc(__ballot_sync(FULL, sv && xi >= ps + 1));
-            }
-            if (warp == 0) {
-                if (np && pv) sm.cand[prow] = {(short)a, (short)xi, 0.f};
-                if (ns && sv) sm.cand[srow] = {(short)xi, (short)b, 0.f};
-                if (lane == 0) {
-                    if (np && el) sm.cand[el_row] = {(short)a, (short)ps, 0.f};
-                    if (ns && er) sm.cand[er_row] = {(short)(ps + 1), (short)b, 0.f};
-                }
-                int len = (np && pv ? xi - a : 0) + (ns && sv ? b - xi : 0);
-                int pe = np && pv ? xi : a, ss = ns && sv ? xi : b;
-                len = __reduce_add_sync(FULL, len);
-                pe = __reduce_max_sync(FULL, pe);
-                ss = __reduce_min_sync(FULL, ss);
-                if (np && el) { pe = max(pe, ps); len += ps - a; }
-                if (ns && er) { ss = min(ss, ps + 1); len += b - ps - 1; }
-                w_scan += (pe - a) + (b - ss);
-                w_eval += np + ns;
-                w_len += len;
-            }
-            if (np + ns == 0) continue;   // the same in every warp
-            __syncthreads();
-            int task = 0;
-            prototypes(0, np, std::false_type(), task);
-            prototypes(np, np + ns, std::true_type(), task);
-            logits(np + ns);
-            __syncthreads();
-            if (DIRS == 1 || warp < kNT / 32) scan(a, 0, np, std::false_type());
-            if (DIRS == 1 || warp >= kNT / 32) scan(b - 1, np, np + ns, std::true_type());
-            __syncthreads();
-            finish(np + ns);
-            __syncthreads();
-            if (np) {
-                if (pv) dl = sm.candD[prow];
-                if (el) eDL = sm.candD[el_row];
-            }
-            if (ns) {
-                if (sv) dr = sm.candD[srow];
-                if (er) eDR = sm.candD[er_row];
-            }
-        }
-        // a cut ruled out by its D_L keeps G_bin's bound, which is below best1
+        const Open o = open_rows(B);
+        const float DI = sm.nodes[B.node].D, best1 = best_first(B);
+        const int ncut = B.ncut;
+        float dl = o.pv ? sm.candD[B.pre_b + o.prow] : 0.f, dr = o.sv ? sm.candD[sufD + B.suf_b + o.srow] : 0.f;
+        // a cut ruled out keeps a bound below best1
         float val = -INFINITY;
-        if (lane == k1) { dl = DL1; dr = DR1; val = best1; }
-        else if (need) val = fmaf(A.lam_kappa, rew, (DI - dl) - dr);
+        if (!B.direct && lane == B.k1) { dl = B.cD[0]; dr = B.cD[1]; val = best1; }
+        else if ((B.keep >> lane) & 1u) val = fmaf(A.lam_kappa, o.rew, (DI - dl) - dr);
         const unsigned key = lane < ncut ? fkey_ordered(val) : 0u;
         const unsigned kmx = __reduce_max_sync(FULL, key);   // every lane takes part
         const unsigned top = __ballot_sync(FULL, lane < ncut && key == kmx);
@@ -1191,25 +1194,71 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
         const float best = __shfl_sync(FULL, val, bq);
         if (!(best > -INFINITY)) bq = 0;   // only reachable with non-finite gains
         const float bL = __shfl_sync(FULL, dl, bq), bR = __shfl_sync(FULL, dr, bq);
-        __syncthreads();   // every warp has read the node's entry
-        if (warp == 0 && lane == 0) {
-            bool take = false;
-            if (ext) {   // rho_ext = G_ext / (|children| - 1)
-                const int ne = 1 + (ps > a) + (ps + 1 < b);
-                float gext = DI;
-                if (ps > a) gext -= eDL;
-                if (ps + 1 < b) gext -= eDR;
-                take = (ne == 3 ? 0.5f * gext : gext) > best;
-            }
-            if (take) {
-                set_extraction(B, a, b, eDL, eDR);
-            } else {
-                B.nchild = 2;
-                B.ca[0] = (short)a; B.cb[0] = B.cut[bq]; B.cD[0] = bL;
-                B.ca[1] = B.cut[bq]; B.cb[1] = (short)b; B.cD[1] = bR;
-            }
+        if (lane) return;
+        const float eDL = o.el ? sm.candD[B.pre_b + o.el_row] : 0.f, eDR = o.er ? sm.candD[sufD + B.suf_b + o.er_row] : 0.f;
+        bool take = false;
+        if (B.ext) {   // rho_ext = G_ext / (|children| - 1)
+            const int ne = 1 + (o.ps > o.a) + (o.ps + 1 < o.b);
+            float gext = DI;
+            if (o.ps > o.a) gext -= eDL;
+            if (o.ps + 1 < o.b) gext -= eDR;
+            take = (ne == 3 ? 0.5f * gext : gext) > best;
         }
-        __syncthreads();
+        if (take) {
+            set_extraction(B, o.a, o.b, eDL, eDR);
+        } else {
+            B.nchild = 2;
+            B.ca[0] = (short)o.a; B.cb[0] = B.cut[bq]; B.cD[0] = bL;
+            B.ca[1] = B.cut[bq]; B.cb[1] = (short)o.b; B.cD[1] = bR;
+        }
+    };
+    // D_L of a node's prefixes known: the cuts that need no suffix drop out.
+    auto narrow_open = [&](BatchNode &B) {
+        const Open o = open_rows(B);
+        const float dl = o.pv ? sm.candD[B.pre_b + o.prow] : 0.f;
+        bool need = (B.more >> lane) & 1u;
+        if (need && A.prune) need = !(fmaf(A.lam_kappa, o.rew, sm.nodes[B.node].D - dl) < best_first(B));
+        const unsigned keep = __ballot_sync(0xffffffffu, need);
+        const bool err = o.er && !__any_sync(0xffffffffu, need && o.xi == o.ps + 1);
+        const int ns = __popc(__ballot_sync(0xffffffffu, need && o.b - o.xi >= 2)) + err;
+        if (lane == 0) {
+            B.keep = keep;
+            B.ns = (int8_t)ns;
+        }
+    };
+    // The rows of an open node from row r on: np prefixes, then ns suffixes (0: none now).
+    auto lay_out = [&](BatchNode &B, int r, int np, int ns, bool pre) {
+        const Open o = open_rows(B);
+        if (np && o.pv) sm.cand[r + o.prow] = {(short)o.a, (short)o.xi, 0.f};
+        if (ns && o.sv) sm.cand[r + np + o.srow] = {(short)o.xi, (short)o.b, 0.f};
+        int len = (np && o.pv ? o.xi - o.a : 0) + (ns && o.sv ? o.b - o.xi : 0);
+        int pe = np && o.pv ? o.xi : o.a, ss = ns && o.sv ? o.xi : o.b;
+        len = __reduce_add_sync(0xffffffffu, len);
+        pe = __reduce_max_sync(0xffffffffu, pe);
+        ss = __reduce_min_sync(0xffffffffu, ss);
+        if (lane == 0) {
+            if (np && o.elr) {
+                sm.cand[r + o.el_row] = {(short)o.a, (short)o.ps, 0.f};
+                pe = max(pe, o.ps);
+                len += o.ps - o.a;
+            }
+            if (ns && o.err) {
+                sm.cand[r + np + o.er_row] = {(short)(o.ps + 1), (short)o.b, 0.f};
+                ss = min(ss, o.ps + 1);
+                len += o.b - o.ps - 1;
+            }
+            if (np && B.direct && B.node == 0 && fresh) {
+                sm.cand[r + np - 1] = {(short)o.a, (short)o.b, 0.f};
+                pe = o.b;
+                len += o.b - o.a;
+            }
+            if (pre) { B.pre_b = (int8_t)r; B.pre_e = (int8_t)(r + np); }   // kept while the suffixes follow
+            B.suf_b = (int8_t)(r + np);
+            B.suf_e = (int8_t)(r + np + ns);
+            w_scan += (pe - o.a) + (o.b - ss);
+            w_eval += np + ns;
+            w_len += len;
+        }
     };
 
     int cur = 0;
@@ -1232,8 +1281,12 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                 const int a = sm.nodes[v].a, b = sm.nodes[v].b, nv = b - a;
                 const bool root = v == 0 && fresh;
                 const bool ronly = root && A.root_only;   // only the node's own distortion
-                const int rows = (nv >= 3 && !ronly ? 2 : 0) + (root ? 1 : 0);
-                if (nrow + rows > S::NROW) break;
+                // no cut is evaluated ahead where the bound could hardly rule another out
+                // (floor slots: an extraction may be forced)
+                const bool direct = nv >= 3 && !ronly && !ufl &&
+                                    !(A.prune && A.lam_kappa > (root ? kDirectRoot * mass : kDirect * sm.nodes[v].D));
+                const int rows = direct ? 0 : (nv >= 3 && !ronly ? 2 : 0) + (root ? 1 : 0);
+                if (nrow + rows > kNCR) break;
                 lbits &= lbits - 1;
                 const int row0 = nrow;
                 nrow += rows;
@@ -1336,14 +1389,16 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                 if (lane == 0) {
                     // the intervals evaluated first: both sides of the cut of largest
                     // reward, or of a forced extraction; a fresh root's own
-                    const int lo = !cands ? a : (forced ? pb : B.cut[k1]), hi = !cands ? b : (forced ? pb + 1 : B.cut[k1]);
+                    const bool ahead = cands && !direct;
+                    const int lo = !ahead ? a : (forced ? pb : B.cut[k1]), hi = !ahead ? b : (forced ? pb + 1 : B.cut[k1]);
                     const bool pv = lo - a >= 2, sv = b - hi >= 2;
                     int k = row0;
                     B.pre_b = (int8_t)k;
                     B.rl = pv ? (int8_t)k : (int8_t)-1;
                     if (pv) sm.cand[k++] = {(short)a, (short)lo, 0.f};
-                    B.whole = root ? (int8_t)k : (int8_t)-1;
-                    if (root) sm.cand[k++] = {(short)a, (short)b, 0.f};
+                    const bool own = root && !direct;
+                    B.whole = own ? (int8_t)k : (int8_t)-1;
+                    if (own) sm.cand[k++] = {(short)a, (short)b, 0.f};
                     B.pre_e = B.suf_b = (int8_t)k;
                     B.rr = sv ? (int8_t)k : (int8_t)-1;
                     if (sv) sm.cand[k++] = {(short)hi, (short)b, 0.f};
@@ -1353,100 +1408,180 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                     B.op = (short)op;
                     B.pstar = (short)pb;
                     B.forced = (int8_t)forced;
+                    B.direct = (int8_t)direct;
                     B.ncut = (int8_t)ncut;
                     B.k1 = (int8_t)k1;
                     // work counters: tokens swept, candidates evaluated, their lengths
-                    w_scan += (root ? nv : (pv ? lo - a : 0)) + (sv ? b - hi : 0);
+                    w_scan += (own ? nv : (pv ? lo - a : 0)) + (sv ? b - hi : 0);
                     w_eval += B.suf_e - B.pre_b;
-                    w_len += (pv ? lo - a : 0) + (sv ? b - hi : 0) + (root ? nv : 0);
+                    w_len += (pv ? lo - a : 0) + (sv ? b - hi : 0) + (own ? nv : 0);
                 }
             }
             // the ops' places in the global list, fetched while the batch is evaluated
             if (nops > 0 && tid == NT - 1) sm.op_base = atomicAdd(A.n_ops, (unsigned)nops);
             if (nb == 0) break;
-            __syncthreads();
-            // ---- phases B/C: prototypes, logits, scans in both directions, sums --
-            int task = 0;
-            for (int bi = 0; bi < nb; bi++) {
-                prototypes(sm.bn[bi].pre_b, sm.bn[bi].pre_e, std::false_type(), task);
-                prototypes(sm.bn[bi].suf_b, sm.bn[bi].suf_e, std::true_type(), task);
-            }
-            logits(nrow);   // after a barrier
-            __syncthreads();
-            for (int bi = 0; bi < nb; bi++) {
-                const BatchNode &B = sm.bn[bi];
-                const NodeS &nd = sm.nodes[B.node];
-                if (DIRS == 1 || warp < kNT / 32) scan(nd.a, B.pre_b, B.pre_e, std::false_type());
-                if (DIRS == 1 || warp >= kNT / 32) scan(nd.b - 1, B.suf_b, B.suf_e, std::true_type());
-            }
-            __syncthreads();
-            finish(nrow);
-            __syncthreads();
-            // ---- phase D1: decisions (warp per node) ---------------------------------
-            // G_bin of a cut is ((D - D_L) - D_R) + lambda_kappa kh, and D_L, D_R >= 0:
-            // D + lambda_kappa kh bounds it from above, in the rounded arithmetic too
-            // (every operation is monotone; G_bin and its bounds all fuse the product).  A cut whose bound is below G_bin of the
-            // cut already evaluated cannot be the best one, and its intervals are never
-            // evaluated; neither are the extraction's sides when that G_bin reaches D,
-            // which bounds rho_ext.  The other cuts are evaluated below, one node at a
-            // time.  D of a node is at most its attention mass, so on long contexts the
-            // curvature's reward decides nearly every cut.
-            bool open = false;   // the warp's nodes need more candidates
-            for (int bi = warp; bi < nb; bi += NWARPS) {
-                BatchNode &B = sm.bn[bi];
-                NodeS &nd = sm.nodes[B.node];
-                const int a = nd.a, b = nd.b, nv = b - a;
-                if (B.whole >= 0 && lane == 0) {   // root: D, Ddrop, Add gain (Eq. app_operation_gains)
-                    const float Pd = sm.candP[B.whole];
-                    const float D = nv >= 2 ? sm.candD[B.whole] : 0.f;
-                    nd.D = D;
-                    float gain = om * sm.rootR * (Pd - D);
-                    if (gain < 0.f) gain = 0.f;
-                    nd.kin = ufl ? FLT_MAX : gain;   // a floor slot's Add is a floor op
-                    A.u_Uadd[uid] = gain;
-                    A.u_Ddrop[uid] = Pd;
-                    A.nd_D[gidx(0)] = D;
-                }
-                __syncwarp();
-                if (A.root_only && B.whole >= 0 && nv >= 2) {   // its split is decided later
-                    if (lane == 0) B.nchild = -1;
-                    continue;
-                }
-                if (nv < 3) {
-                    if (lane == 0) {
-                        B.nchild = 0;
-                        if (nv == 2) {
-                            B.nchild = 2;
-                            B.ca[0] = (short)a; B.cb[0] = (short)(a + 1); B.cD[0] = 0.f;
-                            B.ca[1] = (short)(a + 1); B.cb[1] = (short)b; B.cD[1] = 0.f;
-                        }
+            // Rounds: first the rows laid out above, then those of the batch's open
+            // nodes (the candidates that the first ones could not rule out), as many
+            // nodes [b0, b1) at a time as fit the rows: both sides of the cuts in
+            // B.more and of the extraction (B.ext).  Their prefixes go first, and the
+            // D of those tighten the cuts' bounds before the suffixes follow; both
+            // go together when all of them fit.  A node's own warp lays its rows out
+            // and decides.  (One open node at a time, with the barriers of a round
+            // each, was slower than evaluating every candidate at once where few
+            // cuts are ruled out.)  One loop for all rounds keeps one copy of their code.
+            int b0 = 0, b1 = nb, nr = nrow, dout = 0;
+            bool first = true, pre = true, suf = true, dir = false;
+            for (;;) {
+                __syncthreads();
+                // ---- phases B/C: prototypes, logits, scans in both directions, sums --
+                if (nr > 0) {
+                    int task = 0;
+                    for (int bi = b0; bi < b1; bi++) {
+                        const BatchNode &B = sm.bn[bi];
+                        if (!first && B.nchild != -2) continue;
+                        if (pre) prototypes(B.pre_b, B.pre_e, std::false_type(), task);
+                        if (suf) prototypes(B.suf_b, B.suf_e, std::true_type(), task);
                     }
-                    continue;
+                    logits(nr);   // after a barrier
+                    __syncthreads();
+                    for (int bi = b0; bi < b1; bi++) {
+                        const BatchNode &B = sm.bn[bi];
+                        if (!first && B.nchild != -2) continue;
+                        const NodeS &nd = sm.nodes[B.node];
+                        if (pre && (DIRS == 1 || warp < kNT / 32)) scan(nd.a, B.pre_b, B.pre_e, std::false_type());
+                        if (suf && (DIRS == 1 || warp >= kNT / 32)) scan(nd.b - 1, B.suf_b, B.suf_e, std::true_type());
+                    }
+                    __syncthreads();
+                    finish(nr, pre ? 0 : dout);
+                    __syncthreads();
                 }
-                const float DI = nd.D;
-                const float DL = B.rl >= 0 ? sm.candD[B.rl] : 0.f, DR = B.rr >= 0 ? sm.candD[B.rr] : 0.f;
-                if (B.forced) {
-                    if (lane == 0) set_extraction(B, a, b, DL, DR);
-                    continue;
+                if (first) {
+                    // ---- phase D1: decisions (warp per node) ---------------------------------
+                    // G_bin of a cut is ((D - D_L) - D_R) + lambda_kappa kh, and D_L, D_R >= 0:
+                    // D + lambda_kappa kh bounds it from above, in the rounded arithmetic too
+                    // (every operation is monotone; G_bin and its bounds all fuse the
+                    // product).  A cut whose bound is below G_bin of the cut already evaluated
+                    // cannot be the best one, and its intervals are never evaluated; neither are
+                    // the extraction's sides when that G_bin reaches D, which bounds rho_ext.
+                    // D of a node is at most its attention mass, so on long contexts the
+                    // curvature's reward decides nearly every cut.
+                    bool open = false;   // the warp's nodes need more candidates
+                    for (int bi = warp; bi < nb; bi += NWARPS) {
+                        BatchNode &B = sm.bn[bi];
+                        NodeS &nd = sm.nodes[B.node];
+                        const int a = nd.a, b = nd.b, nv = b - a;
+                        if (B.whole >= 0 && lane == 0) root_done(nd, B.whole);
+                        __syncwarp();
+                        if (A.root_only && B.whole >= 0 && nv >= 2) {   // its split is decided later
+                            if (lane == 0) B.nchild = -1;
+                            continue;
+                        }
+                        if (nv < 3) {
+                            if (lane == 0) {
+                                B.nchild = 0;
+                                if (nv == 2) {
+                                    B.nchild = 2;
+                                    B.ca[0] = (short)a; B.cb[0] = (short)(a + 1); B.cD[0] = 0.f;
+                                    B.ca[1] = (short)(a + 1); B.cb[1] = (short)b; B.cD[1] = 0.f;
+                                }
+                            }
+                            continue;
+                        }
+                        const float DI = nd.D;
+                        const float DL = B.rl >= 0 ? sm.candD[B.rl] : 0.f, DR = B.rr >= 0 ? sm.candD[B.rr] : 0.f;
+                        if (B.forced) {
+                            if (lane == 0) set_extraction(B, a, b, DL, DR);
+                            continue;
+                        }
+                        bool need = lane < B.ncut, ext = true;
+                        if (!B.direct) {
+                            const int k1 = B.k1;
+                            const float best = fmaf(A.lam_kappa, B.kh[k1], (DI - DL) - DR);
+                            need = need && lane != k1;
+                            if (need && A.prune) need = !(fmaf(A.lam_kappa, B.kh[lane], DI) < best);
+                            ext = !(A.prune && best >= DI);
+                            if (lane == 0) {
+                                B.ca[0] = (short)a; B.cb[0] = B.cut[k1]; B.cD[0] = DL;
+                                B.ca[1] = B.cut[k1]; B.cb[1] = (short)b; B.cD[1] = DR;
+                            }
+                        }
+                        const unsigned more = __ballot_sync(0xffffffffu, need);
+                        const bool undecided = more || ext;
+                        if (lane == 0) B.nchild = undecided ? -2 : 2;
+                        if (!undecided) continue;
+                        const int xi = need ? B.cut[lane] : 0;
+                        const int ps = B.pstar;
+                        const bool elr = ext && ps - a >= 2 && !__any_sync(0xffffffffu, need && xi == ps);
+                        const bool err = ext && b - ps - 1 >= 2 && !__any_sync(0xffffffffu, need && xi == ps + 1);
+                        const int np = __popc(__ballot_sync(0xffffffffu, need && xi - a >= 2)) + elr +
+                                       (B.direct && B.node == 0 && fresh);
+                        const int ns = __popc(__ballot_sync(0xffffffffu, need && b - xi >= 2)) + err;
+                        if (lane == 0) {
+                            B.more = B.keep = more;
+                            B.ext = ext;
+                            B.np = (int8_t)np;
+                            B.ns = (int8_t)ns;
+                        }
+                        open = true;
+                    }
+                    if (!__syncthreads_or(open)) break;
+                    first = false;
+                    b1 = 0;
+                } else {
+                    if (pre && fresh && b0 == 0 && warp == 0 && sm.bn[0].direct && sm.bn[0].node == 0) {
+                        if (lane == 0) root_done(sm.nodes[0], sm.bn[0].pre_e - 1);
+                        __syncwarp();
+                    }
+                    if (!suf) {   // the suffixes of the same nodes
+                        if (!dir) {   // (direct nodes have no cut yet that could rule one out)
+                            for (int bi = b0; bi < b1; bi++)
+                                if (sm.bn[bi].nchild == -2 && bi % NWARPS == warp) narrow_open(sm.bn[bi]);
+                            __syncthreads();
+                        }
+                        nr = 0;
+                        for (int bi = b0; bi < b1; bi++) {
+                            BatchNode &B = sm.bn[bi];
+                            if (B.nchild != -2) continue;
+                            const int ns = B.ns;
+                            if (bi % NWARPS == warp) lay_out(B, nr, 0, ns, false);
+                            nr += ns;
+                        }
+                        pre = false;
+                        suf = true;
+                        continue;
+                    }
+                    for (int bi = b0; bi < b1; bi++)
+                        if (sm.bn[bi].nchild == -2 && bi % NWARPS == warp) decide_open(sm.bn[bi], dout);
                 }
-                const int k1 = B.k1;
-                const float best = fmaf(A.lam_kappa, B.kh[k1], (DI - DL) - DR);
-                bool need = lane < B.ncut && lane != k1;
-                if (need && A.prune) need = !(fmaf(A.lam_kappa, B.kh[lane], DI) < best);
-                const unsigned more = __ballot_sync(0xffffffffu, need);
-                const bool ext = !(A.prune && best >= DI);
-                if (lane == 0) {
-                    B.ca[0] = (short)a; B.cb[0] = B.cut[k1]; B.cD[0] = DL;
-                    B.ca[1] = B.cut[k1]; B.cb[1] = (short)b; B.cD[1] = DR;
-                    B.nchild = more || ext ? -2 : 2;
-                    B.more = more;
-                    B.ext = ext;
+                // the next open nodes
+                b0 = b1;
+                int np = 0, ns = 0;
+                bool some = false;
+                dir = true;
+                for (; b1 < nb; b1++) {
+                    const BatchNode &B = sm.bn[b1];
+                    if (B.nchild != -2) continue;
+                    if (np + B.np > kNCR || ns + B.ns > kNCR) break;   // never a group's first node
+                    np += B.np;
+                    ns += B.ns;
+                    some = true;
+                    dir = dir && B.direct;
                 }
-                open |= more || ext;
-            }
-            if (__syncthreads_or(open)) {
-                for (int bi = 0; bi < nb; bi++)
-                    if (sm.bn[bi].nchild == -2) evaluate_rest(sm.bn[bi]);   // ends with a barrier
+                if (!some) {
+                    __syncthreads();
+                    break;
+                }
+                suf = np + ns <= kNCR || (DIRS == 2 && dir && np + ns <= A.nrow);
+                pre = true;
+                dout = suf ? 0 : S::NROW;
+                nr = 0;
+                for (int bi = b0; bi < b1; bi++) {
+                    BatchNode &B = sm.bn[bi];
+                    if (B.nchild != -2) continue;
+                    const int p = B.np, q = suf ? B.ns : 0;
+                    if (bi % NWARPS == warp) lay_out(B, nr, p, q, true);
+                    nr += p + q;
+                }
             }
             // ---- phase D2: numbering, children, gains, keys (warp per node) --------
             // Child indices are deterministic: the batch's nodes in order, after the
@@ -1559,9 +1694,12 @@ cudaError_t launch_t(Ctx &c, BuildArgs &A, unsigned grid, cudaStream_t s) {
     static_assert(sizeof(S) <= 227 * 1024, "unit kernel shared memory above the per-CTA limit");
     static_assert((sizeof(S) + 1024) * S::CTAS <= 228 * 1024, "unit kernel shared memory above the SM's");
     if (grid == 0) return cudaSuccess;
-    size_t sm = sizeof(S);
+    // rows for both sides of a node only where nodes evaluate all cuts at once:
+    // the L1 cache keeps the rest
+    A.nrow = A.prune && A.lam_kappa >= kDirectMax ? kNCR : S::NROW;
+    const size_t sm = sizeof(S) - (S::NROW - A.nrow) * sizeof(typename S::Row);
     cudaError_t e = cudaFuncSetAttribute(unit_build_kernel<DH, Tin, NMAX, SUB>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(S));
     if (e != cudaSuccess) return e;
     unit_build_kernel<DH, Tin, NMAX, SUB><<<grid, S::NT, sm, s>>>(A);
     c.launches += 1;

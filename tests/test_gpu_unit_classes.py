@@ -109,3 +109,43 @@ def test_tied_cuts_take_the_smallest(dtype, d, lam, k_cand):
     o = P.run_oracle(K, V, Q, B, w.rope_base, **kw)
     assert not o["trees"].nodes["D"].any()
     P.compare(g, o, torch.float32 if dtype == "fp32" else torch.bfloat16)
+
+
+@pytest.mark.parametrize("lam", [0.0, 1e-4, 1e-3])
+@pytest.mark.parametrize("k_cand", [16, 5, 0])
+@pytest.mark.parametrize("dtype,d,gq,W", [("bf16", 64, 4, 8), ("bf16", 128, 8, 40), ("fp32", 128, 2, 8)])
+def test_open_cuts_match_the_oracle(dtype, d, gq, W, k_cand, lam):
+    # Little or no curvature reward leaves every cut open: nodes evaluate all of them at once,
+    # as many nodes at a time as fit the 19 rows (16 candidates, the midpoint, the extraction
+    # and a root itself fill them), in every slot class
+    lens = EDGES + [4, 5, 19, 20, 21, 40, 100] + [1 + i % 5 for i in range(40)]
+    w = dataclasses.replace(synth.WORKLOADS["small"], L=1, G=1, Hq=gq, d=d)
+    x = synth.make_inputs(w, T=sum(lens) + 32, W=W)
+    K, V, Q = x.K, x.V, x.Q
+    if dtype == "fp32":
+        K, V, Q = K.float(), V.float(), Q.float()
+    kw = dict(lambda_kappa=lam, k_cand=k_cand, slot_starts=np.concatenate([[0], np.cumsum(lens)]).astype(np.int32))
+    B = K.shape[2] // 3
+    g = P.run_gpu(K, V, Q, B, w.rope_base, **kw)
+    o = P.run_oracle(K, V, Q, B, w.rope_base, **kw)
+    P.compare(g, o, torch.float32 if dtype == "fp32" else torch.bfloat16)
+
+
+@pytest.mark.parametrize("dtype,d", [("bf16", 64), ("fp32", 128)])
+@pytest.mark.parametrize("max_len", [36, 64, 128])
+def test_no_reward_scans_a_node_once_per_direction(dtype, d, max_len):
+    # without a curvature reward no cut can rule another out: none is evaluated ahead of the
+    # others, which would sweep the node's tokens a second time
+    lens = [1 + (7 * i) % max_len for i in range(120)]
+    w = dataclasses.replace(synth.WORKLOADS["small"], L=1, G=1, Hq=4, d=d)
+    x = synth.make_inputs(w, T=sum(lens) + 32, W=8)
+    K, V, Q = x.K, x.V, x.Q
+    if dtype == "fp32":
+        K, V, Q = K.float(), V.float(), Q.float()
+    slots = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    g = P.run_gpu(K, V, Q, K.shape[2] // 4, w.rope_base, lambda_kappa=0.0, slot_starts=slots)
+    ex = g["export"]
+    n = ex["b"] - ex["a"]
+    _, _, work = g["comp"].ctx.gracekv_stats()
+    evaluated = (ex["nchild"] > 0) | (n == 1)   # single tokens: a root's own row
+    assert work["scan_steps"] <= 2 * int(n[evaluated].sum()), work
