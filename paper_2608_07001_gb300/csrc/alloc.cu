@@ -657,14 +657,13 @@ __global__ void __launch_bounds__(1024) alloc_select_kernel(AllocArgs A) {
 // What the host reads between tree passes, side by side behind the state words
 // (shared budget only), so that one copy fetches it: each copy to the host's
 // stack is a round trip of its own (options 16x, 15 passes: 7.15 -> 6.17 ms).
-__global__ void pass_report_kernel(unsigned long long *st, const int *count, const float *cut, const unsigned int *n_qual,
+__global__ void pass_report_kernel(unsigned long long *st, const int *count, const float *cut,
                                    const unsigned long long *pot) {
     PassReport r;
     for (int q = 0; q < kUnitClasses + 1; q++) r.count[q] = count[q];
     r.tau_bits = (uint32_t)st[ST_PREFIX];
     r.all = st[ST_ALL] != 0;
     r.cut = *cut;
-    r.n_qual = *n_qual;
     r.total = st[ST_TOTAL];
     r.pot = *pot;
     *reinterpret_cast<PassReport *>(st + ST_N) = r;
@@ -741,8 +740,7 @@ __global__ void pend_hist_kernel(const float *u_pend, int64_t n_units, const uns
 
 // One block of 1024 threads: thread t owns the 64 bins below kPendBins - 64 t;
 // the bin where the count of larger-or-equal bounds first reaches m gives the cut.
-__global__ void __launch_bounds__(1024) pend_cut_kernel(const unsigned int *hist, int m, float *cut,
-                                                        unsigned int *n_qual) {
+__global__ void __launch_bounds__(1024) pend_cut_kernel(const unsigned int *hist, int m, float *cut) {
     __shared__ unsigned int wsum[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int hi = kPendBins - 64 * tid;   // bins [hi - 64, hi), descending
@@ -767,7 +765,6 @@ __global__ void __launch_bounds__(1024) pend_cut_kernel(const unsigned int *hist
     }
     __syncthreads();
     const unsigned int before = wsum[warp] + incl - own;   // bounds in bins >= hi
-    if (tid == 1023) *n_qual = before + own;
     if (before < (unsigned)m && before + own >= (unsigned)m) {
         unsigned int acc = before;
         for (int b = hi - 1; b >= hi - 64; b--) {
@@ -836,20 +833,20 @@ cudaError_t launch_prune_list(Ctx &c, const int32_t *slots, int J, int32_t *list
 
 cudaError_t launch_pass_report(Ctx &c, const int *count, PassReport *host, cudaStream_t s) {
     static_assert(ST_N * 8 + sizeof(PassReport) <= 16 * 8, "the report fits behind the state words");
-    pass_report_kernel<<<1, 1, 0, s>>>(c.w.alloc_state, count, c.w.pend_cut, c.w.pend_n, c.w.pend_pot);
+    pass_report_kernel<<<1, 1, 0, s>>>(c.w.alloc_state, count, c.w.pend_cut, c.w.pend_pot);
     c.launches += 1;
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return cudaMemcpyAsync(host, c.w.alloc_state + ST_N, sizeof(PassReport), cudaMemcpyDeviceToHost, s);
 }
 
-cudaError_t launch_pend_cut(Ctx &c, int J, int m, float *cut, unsigned int *n_qual, cudaStream_t s) {
+cudaError_t launch_pend_cut(Ctx &c, int J, int m, float *cut, cudaStream_t s) {
     const int64_t nu = (int64_t)c.p.L * c.p.G * J;
     cudaError_t e = cudaMemsetAsync(c.w.pend_hist, 0, sizeof(unsigned int) * kPendBins, s);
     if (e != cudaSuccess) return e;
     pend_hist_kernel<<<(unsigned)((nu + 255) / 256), 256, 0, s>>>(c.w.u_pend, nu, c.w.alloc_state,
                                                                    c.w.pend_hist);
-    pend_cut_kernel<<<1, 1024, 0, s>>>(c.w.pend_hist, m, cut, n_qual);
+    pend_cut_kernel<<<1, 1024, 0, s>>>(c.w.pend_hist, m, cut);
     c.launches += 2;
     return cudaGetLastError();
 }

@@ -291,7 +291,7 @@ gkv_status gracekv_create(const gkv_params *pin, gracekv_ctx **out) {
                 dalloc(x, &w.mh_psum, (size_t)64))) &&
               dalloc(x, &w.hist, (size_t)2048 * (p.quota_alloc ? LG : 1)) &&
               dalloc(x, &w.alloc_state, (size_t)16 * (p.quota_alloc ? (size_t)LG + 1 : 1)) && dalloc(x, &w.work, 4) &&
-              dalloc(x, &w.pend_hist, 1 << 16) && dalloc(x, &w.pend_cut, 1) && dalloc(x, &w.pend_n, 1) &&
+              dalloc(x, &w.pend_hist, 1 << 16) && dalloc(x, &w.pend_cut, 1) &&
               dalloc(x, &w.pend_pot, 1);
     if (!ok) {
         gracekv_destroy(x);
@@ -559,10 +559,15 @@ static cudaError_t build_fresh(Ctx &c, const void *K, const void *V, const void 
     const bool full = c.p.quota_alloc != 0;
     const bool root_only = !full && c.B_free < nu;
     // While everything built so far fits the budget the next pass expands every
-    // pending node; levels that are sure to be reached are built at once: each
-    // about doubles the ops (the Adds are nu of them, the root splits as many).
-    // Not with long units, whose levels set the number of passes anyway (skew 64K
-    // at 32x: 153 -> 169 ms).  small 8x 11.74 -> 10.77 ms, pr1 1.85 -> 1.72 ms.
+    // pending node, so levels that the budget will probably reach are built at
+    // once: a level of cuts doubles the ops (the Adds are nu of them), one of
+    // extractions costs up to twice that, and then nodes are built that the
+    // next pass would have ruled out (the selection is the same).  Levels certain
+    // to be reached (3 nu for two, 7 nu for three) were slower or as fast in
+    // every measured shape, lambda_kappa 0 to 0.05: 16 layers of llama32k at 8x
+    // (4.2 nu) 37.4 -> 40.6 ms.  Not with long units, whose levels set the number
+    // of passes anyway (skew 64K at 32x: 153 -> 169 ms).  small 8x 11.74 ->
+    // 10.77 ms, pr1 1.85 -> 1.72 ms against one level.
     const int levels = c.n_long > 0 ? 1 : c.B_free >= 4 * nu ? 3 : c.B_free >= 2 * nu ? 2 : 1;
     gkv::StageTimer tm(c, 3, s);
     cudaError_t e = gkv::launch_unit_build(c, K, V, Q, omega, w.slots, c.J, 0, root_only ? 1 : 0,
@@ -605,7 +610,7 @@ static cudaError_t build_passes(Ctx &c, const void *K, const void *V, const void
         {
             gkv::StageTimer tm(c, 3, s);
             e = gkv::launch_threshold(c, J, s);
-            if (e == cudaSuccess && root_only) e = gkv::launch_pend_cut(c, J, pass_units, w.pend_cut, w.pend_n, s);
+            if (e == cudaSuccess && root_only) e = gkv::launch_pend_cut(c, J, pass_units, w.pend_cut, s);
             if (e == cudaSuccess) e = gkv::launch_prune_list(c, w.slots, J, w.u_list, w.units_cap, w.dev_int + 2, w.long_list, s);
         }
         if (e == cudaSuccess) e = gkv::launch_pass_report(c, w.dev_int + 2, &h, s);

@@ -11,8 +11,10 @@
 // [a, xi) and suffixes [xi, b) of I for the binary cuts X_v (top-16 positions
 // by curvature in [a, b-2], cut xi = t + 1, plus the midpoint; App. B.4
 // Eq. app_tree_split_candidates) and the two sides of the salient-token
-// extraction at p* = argmax R_tok (Eq. app_extract_split).  For each
-// candidate J the prototype (ktil, vtil, m_eff; Eqs. app_rope_prototype,
+// extraction at p* = argmax R_tok (Eq. app_extract_split).  The sides of the
+// cut of largest curvature reward are evaluated first; cuts and extractions
+// that an exact bound then rules out are never evaluated (phase D1).  For each
+// evaluated candidate J the prototype (ktil, vtil, m_eff; Eqs. app_rope_prototype,
 // app_value_prototype, app_effective_multiplicity) is formed by direct sums
 // over J; then a forward scan (prefixes) and a backward scan (suffixes) over
 // the node's tokens accumulate Z_u(J) and M_u(J) (Eq.
@@ -37,12 +39,12 @@
 // resume launch may build several levels without expanding what its tau
 // already rules out.
 //
-// Layout.  256 threads; thread (p, c) owns the probes p and p + 32 and the
+// Layout.  256 threads per scan direction; thread (p, c) owns the probes p and p + 32 and the
 // elements 4 c + 32 g + j (j < 4) of every d-vector: each value, prototype or
 // key chunk it reads from shared memory serves two probes, and 8 consecutive
 // threads read 128 contiguous bytes (one wavefront, no bank conflicts).
-// Slots of up to 64 tokens use a 64-token instance whose footprint allows two
-// CTAs per SM; longer slots use the 128-token instance.
+// Three instances by slot length: up to 36 tokens three CTAs fit on an SM, up to
+// 64 two; up to 128 tokens one CTA of 512 threads scans both directions at once.
 #include "gkv_internal.cuh"
 
 #include <cfloat>
@@ -206,22 +208,6 @@ __device__ __forceinline__ int round_half_even_mid(int a, int b) {
     return (lo & 1) == 0 ? lo : lo + 1;
 }
 
-// 8 consecutive elements of a shared-memory row as floats (one or two 16-byte loads).
-__device__ __forceinline__ void ld8(const float *p, float v[8]) {
-    float4 a = reinterpret_cast<const float4 *>(p)[0], b = reinterpret_cast<const float4 *>(p)[1];
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-}
-__device__ __forceinline__ void ld8(const __nv_bfloat16 *p, float v[8]) {
-    uint4 u = reinterpret_cast<const uint4 *>(p)[0];
-    const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&u);
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-        float2 f = __bfloat1622float2(h[i]);
-        v[2 * i] = f.x;
-        v[2 * i + 1] = f.y;
-    }
-}
-
 // 4 consecutive elements (8- or 16-byte aligned) as floats.
 __device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 __device__ __forceinline__ float4 ld4(const __nv_bfloat16 *p) {
@@ -229,19 +215,6 @@ __device__ __forceinline__ float4 ld4(const __nv_bfloat16 *p) {
     const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.x));
     const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.y));
     return make_float4(a.x, a.y, b.x, b.y);
-}
-
-// 8 consecutive elements of a shared-memory row as 4 float pairs.
-__device__ __forceinline__ void ld8x2(const float *p, float2 v[4]) {
-    const float4 a = reinterpret_cast<const float4 *>(p)[0], b = reinterpret_cast<const float4 *>(p)[1];
-    v[0] = make_float2(a.x, a.y); v[1] = make_float2(a.z, a.w);
-    v[2] = make_float2(b.x, b.y); v[3] = make_float2(b.z, b.w);
-}
-__device__ __forceinline__ void ld8x2(const __nv_bfloat16 *p, float2 v[4]) {
-    const uint4 u = reinterpret_cast<const uint4 *>(p)[0];
-    const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&u);
-#pragma unroll
-    for (int i = 0; i < 4; i++) v[i] = __bfloat1622float2(h[i]);
 }
 
 // Row that a lane of an 8-row matrix tile reads in an instance of NMAX rows:
@@ -269,28 +242,6 @@ __device__ __forceinline__ void st8(float *p, const float v[8]) {
 __device__ __forceinline__ unsigned fkey_ordered(float x) {
     const unsigned u = __float_as_uint(x + 0.f);
     return u >> 31 ? ~u : u | 0x80000000u;
-}
-
-// N consecutive elements of a shared-memory row as floats (N = 1 or 2).
-template <int N>
-__device__ __forceinline__ void ld_pairs(const float *p, float v[N]) {
-    if constexpr (N == 2) {
-        const float2 x = *reinterpret_cast<const float2 *>(p);
-        v[0] = x.x; v[1] = x.y;
-    } else {
-#pragma unroll
-        for (int j = 0; j < N; j++) v[j] = p[j];
-    }
-}
-template <int N>
-__device__ __forceinline__ void ld_pairs(const __nv_bfloat16 *p, float v[N]) {
-    if constexpr (N == 2) {
-        const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p));
-        v[0] = x.x; v[1] = x.y;
-    } else {
-#pragma unroll
-        for (int j = 0; j < N; j++) v[j] = __bfloat162float(p[j]);
-    }
 }
 
 // Sum over a probe pair's 8 chunk lanes (lane bits 2..4) of each of 8 values,
@@ -500,7 +451,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
 
     // Probe weights E[t][u] (Eq. app_probe_distortion), stored at E[t][u % 32].x
     // (u < 32) or .y (u >= 32).  When the score pass wrote them for every token
-    // they are copied in with the slot (cp.async, 4 bytes each); otherwise
+    // they are copied in with the slot (cp.async, 16 bytes each); otherwise
     // they are formed below from the raw keys.
     float *Ef = reinterpret_cast<float *>(&sm.E[0][0]);
     auto eidx = [](int t, int u) { return t * 2 * kNPP + 2 * (u & (kNPP - 1)) + (u >> 5); };
@@ -1420,15 +1371,15 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
             // the ops' places in the global list, fetched while the batch is evaluated
             if (nops > 0 && tid == NT - 1) sm.op_base = atomicAdd(A.n_ops, (unsigned)nops);
             if (nb == 0) break;
-            // Rounds: first the rows laid out above, then those of the batch's open
+            // Turns: first the rows laid out above, then those of the batch's open
             // nodes (the candidates that the first ones could not rule out), as many
             // nodes [b0, b1) at a time as fit the rows: both sides of the cuts in
             // B.more and of the extraction (B.ext).  Their prefixes go first, and the
             // D of those tighten the cuts' bounds before the suffixes follow; both
             // go together when all of them fit.  A node's own warp lays its rows out
-            // and decides.  (One open node at a time, with the barriers of a round
+            // and decides.  (One open node at a time, with the barriers of a turn
             // each, was slower than evaluating every candidate at once where few
-            // cuts are ruled out.)  One loop for all rounds keeps one copy of their code.
+            // cuts are ruled out.)  One loop for all turns keeps one copy of their code.
             int b0 = 0, b1 = nb, nr = nrow, dout = 0;
             bool first = true, pre = true, suf = true, dir = false;
             for (;;) {

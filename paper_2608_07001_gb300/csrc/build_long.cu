@@ -95,7 +95,7 @@ struct LongArgs {
     int32_t *u_start, *u_cnt;      // per listed unit: its block of work items
     unsigned int *n_items;         // [4]: work items, small subtrees of each class
     unsigned int *it_next;         // the next work item to take (zero at the level's start)
-    int32_t *sub;                  // [2][cap_items] small subtrees' roots (global node indices)
+    int32_t *sub;                  // [kUnitClasses][cap_items] small subtrees' roots (global node indices)
     int64_t cap_items;
     // node records and unit arrays (build.cu's layout)
     int32_t *nd_a, *nd_b, *nd_child0, *nd_parent, *nd_unit;

@@ -104,7 +104,6 @@ struct Workspace {
     // bound-ordered expansion of pending nodes
     unsigned int *pend_hist = nullptr;         // [65536] units per bound bin
     float *pend_cut = nullptr;                 // [1] lower bound of the next pass
-    unsigned int *pend_n = nullptr;            // [1] units that reach the threshold
     unsigned long long *pend_pot = nullptr;    // [1] entries a full expansion of those units could take
     // trees of long units (slots above kMaxUnit tokens, build_long.cu): one
     // level's work items, per listed unit its block of them, the unit lists
@@ -377,7 +376,6 @@ struct PassReport {
     uint32_t tau_bits;
     uint32_t all;                  // every op built so far fits the budget
     float cut;                     // bound of the scheduling cut
-    unsigned int n_qual;
     unsigned long long total, pot; // cost of the ops built, of completing the listed units
 };
 cudaError_t launch_pass_report(Ctx &c, const int *count, PassReport *host, cudaStream_t s);
@@ -393,9 +391,8 @@ cudaError_t launch_prune_list(Ctx &c, const int32_t *slots, int J, int32_t *list
 // Bound-ordered expansion: among the units whose largest pending key bound
 // reaches the threshold, the cut that keeps about `m` of them (the lower edge
 // of the bin of the m-th largest bound; -inf when fewer qualify), written to
-// *cut, with the number that qualify at the threshold in *n_qual.  The prune
-// list then uses max(threshold, *cut).
-cudaError_t launch_pend_cut(Ctx &c, int J, int m, float *cut, unsigned int *n_qual, cudaStream_t s);
+// *cut.  The prune list then uses max(threshold, *cut).
+cudaError_t launch_pend_cut(Ctx &c, int J, int m, float *cut, cudaStream_t s);
 
 cudaError_t launch_allocate(Ctx &c, int J, cudaStream_t s);
 // singleton floor (floor.cu): candidates, cap and accepted positions of every (l, g)
