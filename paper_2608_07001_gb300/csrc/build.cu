@@ -379,12 +379,18 @@ struct Smem {
     unsigned int wcnt[NWARPS][3];            // per-warp work counters
     float pend;
     float rootR;                             // R of a fresh root
-    struct Row {
-        alignas(16) float ktil[KTW];         // key prototype; once the logits are taken, the row holds
-                                             // (residual / ||M||^2, Z) of the probes p and p + 32
-        float vtil[DH];
-        float2 zt[kNPP];                     // m_eff exp(logit) of the probes (p, p + 32)
-    } rows[NROW];                            // the last ones only where A.nrow takes them in
+    // Candidate rows, each: the key prototype (KTW; once the logits are taken,
+    // (residual / ||M||^2, Z) of the probes p and p + 32), the value prototype (DH)
+    // and m_eff exp(logit) of the probes (p, p + 32).  The 128-token instance keeps
+    // a row together, so that its last rows may lie past the launch's shared memory
+    // (A.nrow); the others keep the parts apart (1 % faster).
+    static constexpr int ROWF = KTW + DH + 2 * kNPP;
+    alignas(16) float rows[NROW * ROWF];
+    __device__ __forceinline__ float *ktil(int r) { return rows + r * (DIRS == 2 ? ROWF : KTW); }
+    __device__ __forceinline__ float *vtil(int r) { return rows + (DIRS == 2 ? r * ROWF + KTW : NROW * KTW + r * DH); }
+    __device__ __forceinline__ float2 *zt(int r) {
+        return reinterpret_cast<float2 *>(rows + (DIRS == 2 ? r * ROWF + KTW + DH : NROW * (KTW + DH) + r * 2 * kNPP));
+    }
 };
 
 // SUB: the subtree mode, a compile-time flag so that the other instances carry
@@ -863,7 +869,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                 const float a0 = acc.lo(j) * ninv, a1 = acc.hi(j) * ninv;
                 mu2 = fmaf(a0, a0, fmaf(a1, a1, mu2));
                 const float2 cs = rot[j];
-                rotate_to<SF>(a0, a1, cs.x, cs.y, sm.rows[row].ktil[pi0 + j], sm.rows[row].ktil[pi0 + j + HALF]);
+                rotate_to<SF>(a0, a1, cs.x, cs.y, sm.ktil(row)[pi0 + j], sm.ktil(row)[pi0 + j + HALF]);
             }
             mu2 = warp_sum(mu2);
             if (lane == 0) {
@@ -912,8 +918,8 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
             const float winv = 1.0f / ((acc.rs + (float)nJ * beta) + A.eps);
 #pragma unroll
             for (int j = 0; j < PPL; j++) {
-                sm.rows[row].vtil[pi0 + j] = fmaf(beta, acc.slo(j), acc.rlo(j)) * winv;
-                sm.rows[row].vtil[pi0 + j + HALF] = fmaf(beta, acc.shi(j), acc.rhi(j)) * winv;
+                sm.vtil(row)[pi0 + j] = fmaf(beta, acc.slo(j), acc.rlo(j)) * winv;
+                sm.vtil(row)[pi0 + j + HALF] = fmaf(beta, acc.shi(j), acc.rhi(j)) * winv;
             }
         };
         PS s0;
@@ -972,7 +978,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                 float2 xa = make_float2(0.f, 0.f), xb = make_float2(0.f, 0.f);
 #pragma unroll
                 for (int gi = 0; gi < NG; gi++) {
-                    const float4 x = *reinterpret_cast<const float4 *>(&sm.rows[row].ktil[4 * c + 32 * gi]);
+                    const float4 x = *reinterpret_cast<const float4 *>(&sm.ktil(row)[4 * c + 32 * gi]);
                     const float2 ka = make_float2(x.x, x.y), kb = make_float2(x.z, x.w);
                     xa = ffma2(qa0[2 * gi], ka, xa);
                     xa = ffma2(qa0[2 * gi + 1], kb, xa);
@@ -985,7 +991,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
             const float x = reduce_scatter8(v, lane);
             const int row = i + (c & 3);
             if (row < nr)
-                reinterpret_cast<float *>(&sm.rows[row].zt[pp])[c >> 2] =
+                reinterpret_cast<float *>(&sm.zt(row)[pp])[c >> 2] =
                     sm.cand[row].meff * expf(x * inv_sqrt_d - mu_log);
         }
     };
@@ -1026,12 +1032,12 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
 #pragma unroll 2
                 for (; t < stop; t++) add(t);
             }
-            const float2 z = sm.rows[k].zt[pp];
+            const float2 z = sm.zt(k)[pp];
             const float2 nz0 = make_float2(-z.x, -z.x), nz1 = make_float2(-z.y, -z.y);
             float2 r0 = make_float2(0.f, 0.f), r1 = r0, m0 = r0, m1 = r0;
 #pragma unroll
             for (int gi = 0; gi < NG; gi++) {
-                const float4 x = *reinterpret_cast<const float4 *>(&sm.rows[k].vtil[4 * c + 32 * gi]);
+                const float4 x = *reinterpret_cast<const float4 *>(&sm.vtil(k)[4 * c + 32 * gi]);
                 const float2 va = make_float2(x.x, x.y), vb = make_float2(x.z, x.w);
 #pragma unroll
                 for (int h = 0; h < 2; h++) {
@@ -1049,7 +1055,7 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
             // at most 2 ulp, far below the distortion tolerance.
             const float x = reduce_scatter4(r0.x + r0.y, r1.x + r1.y, m0.x + m0.y, m1.x + m1.y, lane);
             const float y = __shfl_xor_sync(0xffffffffu, x, 2 * kPPW);
-            if (c < 4) sm.rows[k].ktil[4 * pp + c] = (c & 2) ? ((c & 1) ? Z.y : Z.x) : __fdividef(x, y + epsf);
+            if (c < 4) sm.ktil(k)[4 * pp + c] = (c & 2) ? ((c & 1) ? Z.y : Z.x) : __fdividef(x, y + epsf);
         }
     };
     // D_u (Eq. app_probe_distortion) of the rows [0, nr), weighted by the
@@ -1061,8 +1067,8 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
         const float invW = 1.0f / A.W;
         for (int k = warp; k < nr; k += NWARPS) {
             if (sm.cand[k].b <= sm.cand[k].a) continue;
-            const float4 q = *reinterpret_cast<const float4 *>(&sm.rows[k].ktil[4 * lane]);   // ratios, Z
-            const float2 z = sm.rows[k].zt[lane];
+            const float4 q = *reinterpret_cast<const float4 *>(&sm.ktil(k)[4 * lane]);   // ratios, Z
+            const float2 z = sm.zt(k)[lane];
             const float Z0 = q.z, Z1 = q.w;
             const float dz0 = Z0 - z.x, dz1 = Z1 - z.y;
             const float D0 = fmaf(lamZ, __fdividef(dz0 * dz0, fmaf(Z0, Z0, epsf)), lamM * q.x);
@@ -1513,6 +1519,8 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                     const BatchNode &B = sm.bn[b1];
                     if (B.nchild != -2) continue;
                     if (np + B.np > kNCR || ns + B.ns > kNCR) break;   // never a group's first node
+                    // with a direction on each half of the warps, both at once while they fit
+                    if (DIRS == 2 && some && np + ns + B.np + B.ns > (dir && B.direct ? A.nrow : kNCR)) break;
                     np += B.np;
                     ns += B.ns;
                     some = true;
@@ -1648,7 +1656,7 @@ cudaError_t launch_t(Ctx &c, BuildArgs &A, unsigned grid, cudaStream_t s) {
     // rows for both sides of a node only where nodes evaluate all cuts at once:
     // the L1 cache keeps the rest
     A.nrow = A.prune && A.lam_kappa >= kDirectMax ? kNCR : S::NROW;
-    const size_t sm = sizeof(S) - (S::NROW - A.nrow) * sizeof(typename S::Row);
+    const size_t sm = sizeof(S) - (S::NROW - A.nrow) * S::ROWF * sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(unit_build_kernel<DH, Tin, NMAX, SUB>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(S));
     if (e != cudaSuccess) return e;
