@@ -1379,31 +1379,30 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
             if (nb == 0) break;
             // Turns: first the rows laid out above, then those of the batch's open
             // nodes (the candidates that the first ones could not rule out), as many
-            // nodes [b0, b1) at a time as fit the rows: both sides of the cuts in
+            // nodes at a time as fit the rows: both sides of the cuts in
             // B.more and of the extraction (B.ext).  Their prefixes go first, and the
             // D of those tighten the cuts' bounds before the suffixes follow; both
             // go together when all of them fit.  A node's own warp lays its rows out
             // and decides.  (One open node at a time, with the barriers of a turn
             // each, was slower than evaluating every candidate at once where few
             // cuts are ruled out.)  One loop for all turns keeps one copy of their code.
-            int b0 = 0, b1 = nb, nr = nrow, dout = 0;
+            unsigned grp = (1u << nb) - 1u, left = 0u;   // the turn's nodes; open ones still to come
+            int nr = nrow, dout = 0, lnp = 0, lns = 0;   // lane i: the open node i's candidates
             bool first = true, pre = true, suf = true, dir = false;
             for (;;) {
                 __syncthreads();
                 // ---- phases B/C: prototypes, logits, scans in both directions, sums --
                 if (nr > 0) {
                     int task = 0;
-                    for (int bi = b0; bi < b1; bi++) {
-                        const BatchNode &B = sm.bn[bi];
-                        if (!first && B.nchild != -2) continue;
+                    for (unsigned m = grp; m; m &= m - 1) {
+                        const BatchNode &B = sm.bn[__ffs(m) - 1];
                         if (pre) prototypes(B.pre_b, B.pre_e, std::false_type(), task);
                         if (suf) prototypes(B.suf_b, B.suf_e, std::true_type(), task);
                     }
                     logits(nr);   // after a barrier
                     __syncthreads();
-                    for (int bi = b0; bi < b1; bi++) {
-                        const BatchNode &B = sm.bn[bi];
-                        if (!first && B.nchild != -2) continue;
+                    for (unsigned m = grp; m; m &= m - 1) {
+                        const BatchNode &B = sm.bn[__ffs(m) - 1];
                         const NodeS &nd = sm.nodes[B.node];
                         if (pre && (DIRS == 1 || warp < kNT / 32)) scan(nd.a, B.pre_b, B.pre_e, std::false_type());
                         if (suf && (DIRS == 1 || warp >= kNT / 32)) scan(nd.b - 1, B.suf_b, B.suf_e, std::true_type());
@@ -1483,62 +1482,68 @@ __global__ void __launch_bounds__(Smem<DH, NMAX>::NT, Smem<DH, NMAX>::CTAS) unit
                     }
                     if (!__syncthreads_or(open)) break;
                     first = false;
-                    b1 = 0;
+                    const bool op = lane < nb && sm.bn[lane].nchild == -2;
+                    left = __ballot_sync(0xffffffffu, op);
+                    if (op) { lnp = sm.bn[lane].np; lns = sm.bn[lane].ns; }
                 } else {
-                    if (pre && fresh && b0 == 0 && warp == 0 && sm.bn[0].direct && sm.bn[0].node == 0) {
+                    if (pre && fresh && (grp & 1u) && warp == 0 && sm.bn[0].direct && sm.bn[0].node == 0) {
                         if (lane == 0) root_done(sm.nodes[0], sm.bn[0].pre_e - 1);
                         __syncwarp();
                     }
                     if (!suf) {   // the suffixes of the same nodes
                         if (!dir) {   // (direct nodes have no cut yet that could rule one out)
-                            for (int bi = b0; bi < b1; bi++)
-                                if (sm.bn[bi].nchild == -2 && bi % NWARPS == warp) narrow_open(sm.bn[bi]);
+                            for (unsigned m = grp; m; m &= m - 1) {
+                                const int bi = __ffs(m) - 1;
+                                if (bi % NWARPS == warp) narrow_open(sm.bn[bi]);
+                            }
                             __syncthreads();
+                            if ((grp >> lane) & 1u) lns = sm.bn[lane].ns;
                         }
                         nr = 0;
-                        for (int bi = b0; bi < b1; bi++) {
-                            BatchNode &B = sm.bn[bi];
-                            if (B.nchild != -2) continue;
-                            const int ns = B.ns;
-                            if (bi % NWARPS == warp) lay_out(B, nr, 0, ns, false);
+                        for (unsigned m = grp; m; m &= m - 1) {
+                            const int bi = __ffs(m) - 1, ns = __shfl_sync(0xffffffffu, lns, bi);
+                            if (bi % NWARPS == warp) lay_out(sm.bn[bi], nr, 0, ns, false);
                             nr += ns;
                         }
                         pre = false;
                         suf = true;
                         continue;
                     }
-                    for (int bi = b0; bi < b1; bi++)
-                        if (sm.bn[bi].nchild == -2 && bi % NWARPS == warp) decide_open(sm.bn[bi], dout);
+                    for (unsigned m = grp; m; m &= m - 1) {
+                        const int bi = __ffs(m) - 1;
+                        if (bi % NWARPS == warp) decide_open(sm.bn[bi], dout);
+                    }
                 }
-                // the next open nodes
-                b0 = b1;
-                int np = 0, ns = 0;
-                bool some = false;
-                dir = true;
-                for (; b1 < nb; b1++) {
-                    const BatchNode &B = sm.bn[b1];
-                    if (B.nchild != -2) continue;
-                    if (np + B.np > kNCR || ns + B.ns > kNCR) break;   // never a group's first node
-                    // with a direction on each half of the warps, both at once while they fit
-                    if (DIRS == 2 && some && np + ns + B.np + B.ns > (dir && B.direct ? A.nrow : kNCR)) break;
-                    np += B.np;
-                    ns += B.ns;
-                    some = true;
-                    dir = dir && B.direct;
-                }
-                if (!some) {
+                if (!left) {
                     __syncthreads();
                     break;
                 }
-                suf = np + ns <= kNCR || (DIRS == 2 && dir && np + ns <= A.nrow);
+                // the next open nodes
+                const unsigned dm = __ballot_sync(0xffffffffu, ((left >> lane) & 1u) && sm.bn[lane].direct);
+                int np = 0, ns = 0;
+                grp = 0u;
+                dir = true;
+                while (left) {
+                    const int bi = __ffs(left) - 1;
+                    const int p = __shfl_sync(0xffffffffu, lnp, bi), q = __shfl_sync(0xffffffffu, lns, bi);
+                    const bool d = dir && ((dm >> bi) & 1u);
+                    if (grp && (np + p > kNCR || ns + q > kNCR)) break;   // (a node's own always fit)
+                    // with a direction on each half of the warps, both at once while they fit
+                    if (DIRS == 2 && grp && np + ns + p + q > (d ? A.nrow : kNCR)) break;
+                    np += p;
+                    ns += q;
+                    dir = d;
+                    grp |= 1u << bi;
+                    left &= left - 1;
+                }
+                suf = np + ns <= kNCR || (dir && np + ns <= A.nrow);
                 pre = true;
                 dout = suf ? 0 : S::NROW;
                 nr = 0;
-                for (int bi = b0; bi < b1; bi++) {
-                    BatchNode &B = sm.bn[bi];
-                    if (B.nchild != -2) continue;
-                    const int p = B.np, q = suf ? B.ns : 0;
-                    if (bi % NWARPS == warp) lay_out(B, nr, p, q, true);
+                for (unsigned m = grp; m; m &= m - 1) {
+                    const int bi = __ffs(m) - 1;
+                    const int p = __shfl_sync(0xffffffffu, lnp, bi), q = suf ? __shfl_sync(0xffffffffu, lns, bi) : 0;
+                    if (bi % NWARPS == warp) lay_out(sm.bn[bi], nr, p, q, true);
                     nr += p + q;
                 }
             }
