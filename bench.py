@@ -38,9 +38,9 @@ PEAK_FALLBACK = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustaine
                  "sm_max_mhz": 2070.0}
 FP32_LANES = 128
 # DRAM bytes of one compression in the dominant stage, from an ncu capture
-# (profiles/unit_build_llama128k_2layers_32x.md: the 2-layer slice's 2.29 GB
+# (profiles/unit_build_llama128k_2layers_32x.md: the 2-layer slice's 2.27 GB
 # scaled by 16 to 32 layers); reported only for the workload it was taken on
-STAGE_TRAFFIC = {("unit_trees", "llama128k@32x"): (36.62e9, "ncu dram bytes of every unit_build launch "
+STAGE_TRAFFIC = {("unit_trees", "llama128k@32x"): (36.38e9, "ncu dram bytes of every unit_build launch "
                                                            "of one compression on the 2-layer slice x 16")}
 
 
@@ -466,10 +466,11 @@ def main():
     Wp = Q.shape[2]
     if dom == "unit_trees":
         # probe scans (W*d FMA per token step), candidate evaluation (logit,
-        # residual and ||M||^2: 4 W d FMA), prototype sums (3 d per token),
-        # probe weights of every token (W d FMA)
+        # residual and ||M||^2: 4 W d FMA), prototype sums (3 d per token); the probe
+        # weights of every token (W d FMA) only where the score pass does not form them
+        score_weights = K.dtype == torch.bfloat16 and Q.shape[1] // G * Wp <= 256
         flops = (2 * Wp * d * work["scan_steps"] + 8 * Wp * d * work["cand_evals"]
-                 + 6 * d * work["cand_len_sum"] + 2 * Wp * d * L * G * comp.ctx.n_c)
+                 + 6 * d * work["cand_len_sum"] + (0 if score_weights else 2 * Wp * d * L * G * comp.ctx.n_c))
         peak = n_sms * FP32_LANES * 2 * pk.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
         ach = flops / (per_step[dom] / 1e3) / 1e12
         tr = STAGE_TRAFFIC.get((dom, workload_config(w, args.ratio, L)["workload"]))
