@@ -66,7 +66,7 @@ constexpr int kPPW = 32 / kNCL;  // probe pairs per warp: lane = 4 c + (pair % 4
 // lambda_kappa at most kDirect of the node's D (of a fresh root's attention mass,
 // which weights its D, not known yet) all cuts are evaluated at once.  The mass
 // is formed below kDirectMax only: a slot of a long request holds far less.
-// 16 layers of llama32k, lambda_kappa 0 at 8x / 32x: 100.3 -> 82.4 / 35.0 ->
+// 16 layers of llama32k, lambda_kappa 0 at 8x / 32x: 100.2 -> 81.9 / 35.0 ->
 // 29.2 ms, 2e-4: 95.4 -> 83.0 / 34.5 -> 29.7, 1e-3: 75.2 -> 67.9 / 29.6 -> 27.4;
 // shares of 0.1 to 0.5 were up to 5 % slower at 1e-4 to 1e-3, of 2 and 3 no faster.
 constexpr float kDirect = 1.0f, kDirectRoot = 1.0f, kDirectMax = 0.01f;
